@@ -162,11 +162,6 @@ cudaError_t launch_fp64_bench(int32_t iters, int32_t grid, double *sink, cudaStr
 cudaError_t launch_smem_atomic_bench(int32_t variant, int32_t iters, int32_t grid,
                                      unsigned long long *sink, cudaStream_t s);
 
-// Exclusive scan of n int32 counts into int64 (one block): pref[0 .. n] (may be
-// null) and strided[r] = pref[r * stride] for r = 0 .. n / stride (may be null).
-cudaError_t launch_exclusive_scan(const int32_t *cnt, int64_t n, int64_t *pref, int32_t stride,
-                                  int64_t *strided, cudaStream_t s);
-
 // Device buffers of one call, taken stream-ordered (cudaMallocAsync) and
 // returned stream-ordered when the object goes out of scope.
 struct Scratch {
@@ -189,6 +184,10 @@ struct Scratch {
         for (void *b : bufs) cudaFreeAsync(b, s);
     }
 };
+
+// Exclusive scan of n int32 counts into pref[0 .. n] (fh_peakmap.cu).
+template <typename T>
+cudaError_t scan_exclusive(const int32_t *cnt, int64_t n, T *pref, Scratch &sc, cudaStream_t s);
 
 // ---- host helpers (fh_api.cu) ----
 int set_error(int code, const char *fmt, ...);

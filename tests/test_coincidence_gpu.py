@@ -163,3 +163,47 @@ def test_cluster_coincidences_match_oracle(fh, co):
     with pytest.raises(fh.FHError) as ei:
         fh.fh_cluster_coincidences(da, db, 1.0e6, 2.0e6, 1.5e6, la, lb, out)
     assert ei.value.code == fh.FH_ERR_INVALID_ARG
+
+
+def _cells_case(name):
+    """Sets at the edges of the (frequency, spin-down) cells."""
+    if name == "capped":      # far more cells wanted than candidates
+        a = synth.candidates_on_grid(48, 1, 150, (5, 3, 100000, 90000))
+        b = a + np.array([0, 0, 1.0, -1.0, 0, 0, 0, 0])
+        return np.concatenate([a, b]), np.concatenate([b[::-1], a])
+    if name == "outside":     # set 1 partly far outside set 2, partly one cell away
+        b = synth.candidates_on_grid(49, 1, 400, (6, 4, 40, 12))
+        a = np.concatenate([b + np.array([0, 0, x, y, 0, 0, 0, 0])
+                            for x, y in ((1e7, 0), (-41.0, 0), (39.0, 1.0), (0, 13.0), (0, -1e9))])
+        return a, b
+    if name == "crowded":     # more partners per candidate than the count keeps
+        return (synth.candidates_on_grid(50, 1, 700, (3, 2, 9, 5)),
+                synth.candidates_on_grid(50, 2, 500, (3, 2, 9, 5)))
+    if name == "one_cell":    # no range at all in frequency and spin-down
+        a = synth.candidates_on_grid(51, 1, 300, (300, 40, 1, 1))
+        return a, a[::-1]
+    # beyond binary32: values and widths of 1e36 to 1e40, and subnormal widths
+    a = synth.candidates_on_grid(52, 1, 300, (7, 5, 30, 10))
+    a[:, 2] *= 1e39
+    a[:, 6] = 1e39
+    a[:, 3] *= 1e-39
+    a[:, 7] = 1e-39
+    return a, a[::-1]
+
+
+@pytest.mark.parametrize("name", ["capped", "outside", "crowded", "one_cell", "beyond"])
+def test_cells_of_frequency_and_spin_down(fh, co, name):
+    a, b = _cells_case(name)
+    for d_max in (0.0, 1.0, 1.5):
+        check_cluster(fh, co, a, d_max)
+    for win in ((0, 0, 0, 0), (1, 1, 1, 1), (0, 1, 1, 2)):
+        check_coinc(fh, co, a, b, 0.0, 0.0, 0.0, win)
+
+
+@pytest.mark.parametrize("n", [4096, 4097, 8192, 8193])
+def test_scan_tiles(fh, co, n):
+    """Set sizes whose cell counts end at, and one past, the scan's tiles."""
+    a = synth.candidate_set(53, 1, n, clusters=20, cluster_size=5)
+    check_cluster(fh, co, a, 2.0)
+    check_coinc(fh, co, a[:500], a, 0.0, 0.0, 0.0, (2, 2, 2, 2))
+    check_coinc(fh, co, a, a[:300], 0.0, 0.0, 0.0, (2, 2, 2, 2))
