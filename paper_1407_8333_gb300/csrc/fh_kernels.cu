@@ -1636,11 +1636,15 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
 }
 
 // ---------------------------------------------------------------- a6
-// grid (n_sb, n_dir), 1024 threads: greedy picks of one sub-band of one direction.
+// grid (n_sb, n_dir): greedy picks of one sub-band of one direction.
 // Order of the picks: profile key descending (count, then smaller row), then
-// smaller cell.  A sub-band of up to kSelPer x 1024 cells is held in registers
-// (kSelPer cells per thread); each pick zeroes the keys within `excl` cells of
-// it, so later picks skip them.  Wider sub-bands rescan the profile per pick.
+// smaller cell.  A sub-band of up to kSelPer cells per thread is held in
+// registers; each pick zeroes the keys within `excl` cells of it, so later picks
+// skip them.  Wider sub-bands rescan the profile per pick.
+// Latency-bound: a pick is a chain of loads, warp reductions and two barriers,
+// so a block has only the threads that kSelPer cells each leave it (the
+// launch's choice), and more sub-bands run side by side: 2560 sub-bands of 1024
+// cells take 17 us with 128 threads, 123 us with 1024.
 constexpr int kSelThreads = 1024;
 constexpr int kSelPer = 8;
 
@@ -1670,11 +1674,11 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectArgs a)
     const unsigned long long *prof =
         reinterpret_cast<const unsigned long long *>(a.profile) + (int64_t)d_abs * a.n_f0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const bool in_regs = hi - lo <= kSelPer * kSelThreads;
+    const bool in_regs = hi - lo <= kSelPer * (int)blockDim.x;
     unsigned long long key[kSelPer];
 #pragma unroll
     for (int j = 0; j < kSelPer; ++j) {
-        const int b = lo + threadIdx.x + j * kSelThreads;
+        const int b = lo + threadIdx.x + j * (int)blockDim.x;
         key[j] = (in_regs && b < hi) ? prof[b] : 0ull;
     }
     if (threadIdx.x == 0) { npick = 0; stop = 0; }
@@ -1687,7 +1691,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectArgs a)
             // a thread's cells ascend with j: a strict > keeps the smaller cell on ties
 #pragma unroll
             for (int j = 0; j < kSelPer; ++j)
-                if (key[j] > bk) { bk = key[j]; bc = lo + threadIdx.x + j * kSelThreads; }
+                if (key[j] > bk) { bk = key[j]; bc = lo + threadIdx.x + j * (int)blockDim.x; }
         } else {
             for (int b = lo + threadIdx.x; b < hi; b += blockDim.x) {
                 bool ex = false;
@@ -1733,7 +1737,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectArgs a)
             const int pc = picks[np];
 #pragma unroll
             for (int j = 0; j < kSelPer; ++j) {
-                const int b = lo + threadIdx.x + j * kSelThreads;
+                const int b = lo + threadIdx.x + j * (int)blockDim.x;
                 const int dd = b > pc ? b - pc : pc - b;
                 if (dd <= a.excl) key[j] = 0ull;
             }
@@ -2079,7 +2083,11 @@ cudaError_t launch_select(const SelectArgs &a, cudaStream_t s)
 {
     if (a.n_dir <= 0 || a.n_sb <= 0) return cudaSuccess;
     dim3 grid(a.n_sb, a.n_dir);
-    select_kernel<<<grid, kSelThreads, 0, s>>>(a);
+    // whole warps that hold the sub-band at kSelPer cells per thread
+    const int cells = std::min(a.subband_cells, a.n_f0);
+    const int threads = (int)std::min<int64_t>(kSelThreads, ((int64_t)cells + 32 * kSelPer - 1) /
+                                                                (32 * kSelPer) * 32);
+    select_kernel<<<grid, threads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
