@@ -742,6 +742,30 @@ __device__ __forceinline__ void diff_step(int32_t *H0, int lane, int64_t &X, con
     }
 }
 
+// x += y and x -= y on 64-bit positions as an explicit 32-bit carry chain
+// (low words with carry out, high words with carry in).  The result is the
+// same two's-complement sum; the walks run faster with this form than with the
+// compiler's own 64-bit add (the paired one by 1.8 % on the 900 Hz workload and
+// 0.9 % on the 50 Hz one, the unpaired one by 2 % on the 50 Hz adaptive map).
+__device__ __forceinline__ void add_carry(int64_t &x, int64_t y)
+{
+    asm("{\n\t.reg .u32 xl, xh, yl, yh;\n\t"
+        "mov.b64 {xl, xh}, %0;\n\tmov.b64 {yl, yh}, %1;\n\t"
+        "add.cc.u32 xl, xl, yl;\n\taddc.u32 xh, xh, yh;\n\t"
+        "mov.b64 %0, {xl, xh};\n\t}"
+        : "+l"(x)
+        : "l"(y));
+}
+__device__ __forceinline__ void sub_carry(int64_t &x, int64_t y)
+{
+    asm("{\n\t.reg .u32 xl, xh, yl, yh;\n\t"
+        "mov.b64 {xl, xh}, %0;\n\tmov.b64 {yl, yh}, %1;\n\t"
+        "sub.cc.u32 xl, xl, yl;\n\tsubc.u32 xh, xh, yh;\n\t"
+        "mov.b64 %0, {xl, xh};\n\t}"
+        : "+l"(x)
+        : "l"(y));
+}
+
 // Step T of a peak's 32 row updates.  The lane visits row lane ^ g(T),
 // g(T) = T ^ (T >> 1) (a Gray code; T, g(T), the bit b that flips next and its
 // sign are compile-time constants): for every step the 32 lanes of a warp
@@ -784,11 +808,11 @@ __device__ __forceinline__ void pair_step(uint32_t rbase, int64_t &X1, int64_t &
     if constexpr (T < 31) {
         constexpr int b = ctz5(T + 1);
         if constexpr ((gt >> b) & 1) {
-            X1 -= e[b];
-            X2 -= e[b];
+            sub_carry(X1, e[b]);
+            sub_carry(X2, e[b]);
         } else {
-            X1 += e[b];
-            X2 += e[b];
+            add_carry(X1, e[b]);
+            add_carry(X2, e[b]);
         }
     }
 }
@@ -799,30 +823,6 @@ __device__ __forceinline__ void pair_steps(std::integer_sequence<int, Ts...>, ui
                                            uint32_t stride, uint32_t E, uint32_t w)
 {
     (pair_step<CLAMP, WEIGHTED, Ts>(rbase, X1, X2, e, stride, E, w), ...);
-}
-
-// x += y and x -= y on 64-bit positions as an explicit 32-bit carry chain
-// (low words with carry out, high words with carry in).  The result is the
-// same two's-complement sum; the paired walk ran faster with this form than
-// with the compiler's own 64-bit add (by 1.8 % on the 900 Hz workload, 0.9 %
-// on the 50 Hz one).
-__device__ __forceinline__ void add_carry(int64_t &x, int64_t y)
-{
-    asm("{\n\t.reg .u32 xl, xh, yl, yh;\n\t"
-        "mov.b64 {xl, xh}, %0;\n\tmov.b64 {yl, yh}, %1;\n\t"
-        "add.cc.u32 xl, xl, yl;\n\taddc.u32 xh, xh, yh;\n\t"
-        "mov.b64 %0, {xl, xh};\n\t}"
-        : "+l"(x)
-        : "l"(y));
-}
-__device__ __forceinline__ void sub_carry(int64_t &x, int64_t y)
-{
-    asm("{\n\t.reg .u32 xl, xh, yl, yh;\n\t"
-        "mov.b64 {xl, xh}, %0;\n\tmov.b64 {yl, yh}, %1;\n\t"
-        "sub.cc.u32 xl, xl, yl;\n\tsubc.u32 xh, xh, yh;\n\t"
-        "mov.b64 %0, {xl, xh};\n\t}"
-        : "+l"(x)
-        : "l"(y));
 }
 
 // Step T of the paired walk (two directions of one pair, two 16-bit counters
@@ -866,31 +866,31 @@ __device__ __forceinline__ void quad_step(uint32_t rbase, int64_t &X1, int64_t &
     }
 }
 
-template <bool CLAMP, int... Ts>
-__device__ __forceinline__ void quad_steps(std::integer_sequence<int, Ts...>, uint32_t rbase,
-                                           int64_t X1, int64_t X2, int64_t Y1, int64_t Y2,
-                                           const int64_t (&e)[5], uint32_t stride, uint32_t E)
+// The first S steps of the paired walk (unclamped; S = 4, 8, 16 or 32): a
+// compacted last round and a short pass leave the unrolled walk early.  (A loop
+// of S steps of its own, with each row's drift multiplied out, took 28
+// instructions per step against 17: 2.9 % of the kernel on the 900 Hz workload,
+// 4.18 -> 4.06 ms per direction pair.)
+template <int T0, int... Ts>
+__device__ __forceinline__ void quad_range(std::integer_sequence<int, Ts...>, uint32_t rbase,
+                                           int64_t &X1, int64_t &X2, int64_t &Y1, int64_t &Y2,
+                                           const int64_t (&e)[5], uint32_t stride)
 {
-    (quad_step<CLAMP, Ts>(rbase, X1, X2, Y1, Y2, e, stride, E), ...);
+    (quad_step<false, T0 + Ts>(rbase, X1, X2, Y1, Y2, e, stride, 0u), ...);
 }
-
-// The first S Gray-code steps of the paired walk (unclamped), for a compacted
-// last round (S < 32): a loop rather than unrolled steps, so that the paired
-// kernel's registers stay within a 24-warp block.  Row lane ^ g(t) is reached
-// from the start row lane by adding (lane - row) D.
-__device__ __forceinline__ void quad_steps_short(int S, uint32_t rbase, uint32_t lane, int64_t X1,
-                                                 int64_t X2, int64_t Y1, int64_t Y2, int64_t dv,
-                                                 uint32_t stride)
+__device__ __forceinline__ void quad_steps(int S, uint32_t rbase, int64_t X1, int64_t X2,
+                                           int64_t Y1, int64_t Y2, const int64_t (&e)[5],
+                                           uint32_t stride)
 {
-#pragma unroll 1
-    for (int t = 0; t < S; ++t) {
-        const uint32_t gt = (uint32_t)(t ^ (t >> 1));
-        const int64_t dl = (int64_t)((int)lane - (int)(lane ^ gt)) * dv;
-        const uint32_t rb = rbase ^ (gt << 2);
-        asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(cell_of(X1 + dl) * stride + rb) : "memory");
-        asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(cell_of(X2 + dl) * stride + rb) : "memory");
-        asm volatile("red.shared.add.u32 [%0], 65536;" ::"r"(cell_of(Y1 + dl) * stride + rb) : "memory");
-        asm volatile("red.shared.add.u32 [%0], 65536;" ::"r"(cell_of(Y2 + dl) * stride + rb) : "memory");
+    using std::make_integer_sequence;
+    quad_range<0>(make_integer_sequence<int, 4>{}, rbase, X1, X2, Y1, Y2, e, stride);
+    if (S > 4) {
+        quad_range<4>(make_integer_sequence<int, 4>{}, rbase, X1, X2, Y1, Y2, e, stride);
+        if (S > 8) {
+            quad_range<8>(make_integer_sequence<int, 8>{}, rbase, X1, X2, Y1, Y2, e, stride);
+            if (S > 16)
+                quad_range<16>(make_integer_sequence<int, 16>{}, rbase, X1, X2, Y1, Y2, e, stride);
+        }
     }
 }
 
@@ -911,7 +911,7 @@ __device__ __forceinline__ void diff_steps(std::integer_sequence<int, Ts...>, in
 // a stripe starting at cell s (so L in [0, W + K - 1) covers every stripe that
 // touches the tile), row stride 32 words: row r lives in bank r.
 //
-// Accumulate: each warp takes 32 FFTs at a time (lane <-> FFT) and reads, per
+// Accumulate: each warp takes runs of FFTs, 32 at a time (lane <-> FFT), and reads, per
 // FFT, the window of peaks that can reach the tile on some row of the slab
 // (precomputed by windows_kernel, else a binary search).  The windowed peaks
 // of the 32 FFTs are dealt out to the lanes in rounds of 32 slots (a warp scan
@@ -955,7 +955,8 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
     static_assert(!PACK || (MODE == FH_MODE_START && !WEIGHTED), "packed counters: plain START");
     extern __shared__ __align__(16) int32_t smem_raw[];
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
+    // (out of a shuffle: known to be uniform in the warp)
+    const int warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
     const int nwarps = blockDim.x >> 5;
     // counters: `guard` cells below the tile, the tile's W + K - 1 cells (plus
     // the dump cell), `guard` cells above; cell 0 sits at a 128-byte aligned
@@ -1068,7 +1069,11 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
             // 2^ceil(log2 R) rows of its aligned block of Srows lanes, counting
             // virtual row lane mod Srows in the lane's own bank (row lane ^ g(t));
             // the 32 / Srows copies of a row are summed before the emit.
-            const int Srows = SHORT ? (R <= 1 ? 1 : R <= 2 ? 2 : R <= 4 ? 4 : R <= 8 ? 8 : 16) : 32;
+            // (The paired walk's shortest is 4 steps.)
+            const int Srows = !SHORT ? 32
+                              : R <= 1 && !QUAD ? 1
+                              : R <= 2 && !QUAD ? 2
+                              : R <= 4 ? 4 : R <= 8 ? 8 : 16;
 
             // zero the counters (with the guard cells in the fast path); reset the chunk counter
             {
@@ -1080,16 +1085,28 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
             __syncthreads();
 
             // accumulate
-            // chunks of 32 FFTs (lane <-> FFT): the first round one per warp, then
-            // whoever is free
-            for (int c = warp; c < nchunks;) {
+            // Runs of FFTs, dealt 32 FFTs at a time (lane <-> FFT): every warp's first run
+            // is three quarters of its share, then whoever is free takes a short one.
+            // Inside a run only whole rounds of 32 slots are walked: the next 32 FFTs start
+            // at the first FFT with slots left, `skip` of which are already done.  So
+            // a warp has a partial round per run instead of one per 32 FFTs (3 % fewer
+            // atomics on the 900 Hz workload).  T, and with it the rounds' control flow,
+            // comes out of a shuffle so that the compiler knows it to be the same in all
+            // lanes (else it guards every round's shuffles against divergence: 33
+            // million more branch instructions per launch and 2 % of the time).
+            const int run0 = (3 * nchunks) / (4 * nwarps), run1 = max(1, run0 >> 4);
+            int run = warp;  // runs below nwarps are first runs
+            int i0 = run0 > 0 ? run0 * warp * 32 : warp * 32;
+            int i_end = run0 > 0 ? run0 * (warp + 1) * 32 : i0 + 32;
+            int skip = 0;
+            while (i0 < n_fft) {
                 int64_t cb, dv, q0;
                 int n;
                 // the FFT's weight on this direction (adaptive map), 1 for the plain map
                 int32_t wt = 1;
                 if constexpr (WEIGHTED)
-                    if (wts != nullptr && (c << 5) + lane < n_fft) wt = __ldg(wts + (c << 5) + lane);
-                const int i_l = (c << 5) + lane;
+                    if (wts != nullptr && i0 + lane < n_fft) wt = __ldg(wts + i0 + lane);
+                const int i_l = i0 + lane < i_end ? i0 + lane : n_fft;
                 const uint32_t wv = (wrow != nullptr && i_l < n_fft) ? wrow[i_l] : kWinLookup;
                 if (wrow != nullptr && wv != kWinLookup) {
                     // precomputed window: one coalesced load (start relative to the FFT's
@@ -1116,14 +1133,14 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                     n = 0;
                 } else {
                     int64_t cbs;
-                    lookup_window(Ap, offs, S0, Dt, n_fft, (c << 5) + lane, js, R_slab, base_shift,
+                    lookup_window(Ap, offs, S0, Dt, n_fft, i_l, js, R_slab, base_shift,
                                   e_fixed, cbs, dv, q0, n);
                     if (QUAD && !ROWQ) {
                         // the union (as one index range) with the other direction's window
                         int64_t cb2, dv2, q0b;
                         int nb;
-                        lookup_window(Ad_b, offs, S0, Dt, n_fft, (c << 5) + lane, js, R_slab,
-                                      base_shift, e_fixed, cb2, dv2, q0b, nb);
+                        lookup_window(Ad_b, offs, S0, Dt, n_fft, i_l, js, R_slab, base_shift,
+                                      e_fixed, cb2, dv2, q0b, nb);
                         if (nb > 0) {
                             const int64_t hi = n > 0 ? max(q0 + n, q0b + nb) : q0b + nb;
                             q0 = n > 0 ? min(q0, q0b) : q0b;
@@ -1136,6 +1153,10 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                 // consecutive peaks of the window; an odd count leaves the last slot's
                 // second peak empty), DIFF mode one peak per slot
                 constexpr bool kPairs = MODE == FH_MODE_START;
+                if (lane == 0) {
+                    q0 += kPairs ? 2 * skip : skip;
+                    n -= kPairs ? 2 * skip : skip;
+                }
                 const int m = kPairs ? (n + 1) >> 1 : n;
                 // exclusive scan of the per-FFT slot counts, owner table of non-empty FFTs
                 int P = m;
@@ -1144,9 +1165,12 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                     const int y = __shfl_up_sync(kFull, P, o);
                     if (lane >= o) P += y;
                 }
-                const int T = __shfl_sync(kFull, P, 31);
+                const int T_all = __shfl_sync(kFull, P, 31);
                 P -= m;
                 const bool has = m > 0;
+                // whole rounds, unless the run ends here or there is not even one
+                const bool part = i0 + 32 >= i_end || T_all < 32;
+                const int T = __shfl_sync(kFull, part ? T_all : T_all & ~31, 0);
                 // the slot's first peak is kq + (pairs ? 2 : 1) g; the window ends at qe
                 const int kq = (int)q0 - (kPairs ? 2 * P : P);
                 const int qe = (int)q0 + n;
@@ -1162,8 +1186,10 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                 // publishes kq = q0 - 2 P (q0 - P) and its window end qe.
                 int before = 0;
                 // QUAD: b1, b2 are the same peaks' positions in direction d_b
-                auto fetch = [&](int base, int64_t &a1, int64_t &a2, int64_t &b1, int64_t &b2,
-                                 bool &two, int &owner) {
+                // full_tag: a whole round, every slot below T (`live` folds to true: 15 of the
+                // about 200 instructions around a round's walk)
+                auto fetch = [&](auto full_tag, int base, int64_t &a1, int64_t &a2, int64_t &b1,
+                                 int64_t &b2, bool &two, int &owner) {
                     const unsigned rel = (unsigned)(P - base);
                     const unsigned bits =
                         __reduce_or_sync(kFull, (has && rel < 32u) ? (1u << rel) : 0u);
@@ -1172,7 +1198,7 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                     owner = tab[oc < 0 ? 0 : oc];
                     const int okq = __shfl_sync(kFull, kq, owner);
                     const int g = base + lane;
-                    const bool live = g < T;
+                    const bool live = decltype(full_tag)::value || g < T;
                     if (kPairs) {
                         const int oqe = __shfl_sync(kFull, qe, owner);
                         const int k = okq + 2 * g;
@@ -1203,16 +1229,17 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                 // peaks whose position in the other direction is that close, so each
                 // position lies within the pair's distance of it, which the guard also
                 // holds.  QUAD: Y1, Y2 are the same peaks in direction d_b.
-                auto setup = [&](int g, int vlane, int64_t a1, int64_t a2, int64_t b1, int64_t b2,
-                                 bool two, int owner, int64_t &X1, int64_t &X2, int64_t &Y1,
-                                 int64_t &Y2, int64_t (&e)[5], int32_t &ow) {
+                auto setup = [&](auto full_tag, int g, int vlane, int64_t a1, int64_t a2,
+                                 int64_t b1, int64_t b2, bool two, int owner, int64_t &X1,
+                                 int64_t &X2, int64_t &Y1, int64_t &Y2, int64_t (&e)[5],
+                                 int32_t &ow) {
                     if constexpr (WEIGHTED)
                         ow = __shfl_sync(kFull, wt, owner);
                     else
                         ow = 1;
                     const int64_t ocb = __shfl_sync(kFull, cb, owner);
                     const int64_t odv0 = __shfl_sync(kFull, dv, owner);
-                    const bool live = g < T;
+                    const bool live = decltype(full_tag)::value || g < T;
                     const int64_t odv = live ? odv0 : 0;
                     // e[b] = +-(D << b), + when bit b of the lane is set
                     const int64_t ndv = -odv;
@@ -1242,40 +1269,51 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                 int64_t a1_nx = 0, a2_nx = 0, b1_nx = 0, b2_nx = 0;
                 bool two_nx = false;
                 int own_nx = 0;
-                if (kAhead && T > 0) fetch(0, a1_nx, a2_nx, b1_nx, b2_nx, two_nx, own_nx);
+                if (kAhead && T > 0) fetch(std::false_type{}, 0, a1_nx, a2_nx, b1_nx, b2_nx, two_nx, own_nx);
                 for (int base = 0; base < T; base += 32) {
                     int64_t a1 = a1_nx, a2 = a2_nx, b1 = b1_nx, b2 = b2_nx;
                     bool two = two_nx;
                     int owner = own_nx;
-                    if (!kAhead) fetch(base, a1, a2, b1, b2, two, owner);
-                    else if (base + 32 < T)
-                        fetch(base + 32, a1_nx, a2_nx, b1_nx, b2_nx, two_nx, own_nx);
-                    // A last round of L <= 16 slots (unclamped START walk): S = the
-                    // power of two >= L; slot q = lane mod S is walked by the 32 / S
-                    // lanes lane = q + S p, lane p taking rows S p .. S p + S - 1 in
-                    // S Gray-code steps (row = lane ^ g(t), t < S).  Every (slot, row)
-                    // is added once, the 32 lanes stay on 32 banks, and the start
-                    // X = A - cb - lane D and the step table are those of a full round.
-                    // (A short pass walks Srows steps with one slot per lane instead.)
-                    int S = Srows;
-                    if (!SHORT && MODE == FH_MODE_START && fast && T - base <= 16) {
-                        const int L = T - base;
-                        S = L <= 1 ? 1 : (L <= 2 ? 2 : (L <= 4 ? 4 : (L <= 8 ? 8 : 16)));
-                        const int src = lane & (S - 1);
-                        a1 = __shfl_sync(kFull, a1, src);
-                        a2 = __shfl_sync(kFull, a2, src);
-                        if constexpr (QUAD) {
-                            b1 = __shfl_sync(kFull, b1, src);
-                            b2 = __shfl_sync(kFull, b2, src);
-                        }
-                        two = __shfl_sync(kFull, (int)two, src) != 0;
-                        owner = __shfl_sync(kFull, owner, src);
-                    }
                     int64_t X1, X2 = 0, Y1 = 0, Y2 = 0, e[5];
                     int32_t ow;
-                    setup(SHORT ? base + lane : base + (lane & (S - 1)),
-                          SHORT ? (lane & (Srows - 1)) : lane, a1, a2, b1, b2, two, owner, X1, X2,
-                          Y1, Y2, e, ow);
+                    int S = Srows;
+                    const int vlane = SHORT ? (lane & (Srows - 1)) : lane;
+                    if (QUAD && base + 32 <= T) {
+                        // a whole round: every slot is live
+                        fetch(std::true_type{}, base, a1, a2, b1, b2, two, owner);
+                        setup(std::true_type{}, base + lane, vlane, a1, a2, b1, b2, two, owner, X1,
+                              X2, Y1, Y2, e, ow);
+                    } else {
+                        if (!kAhead)
+                            fetch(std::false_type{}, base, a1, a2, b1, b2, two, owner);
+                        else if (base + 32 < T)
+                            fetch(std::false_type{}, base + 32, a1_nx, a2_nx, b1_nx, b2_nx, two_nx,
+                                  own_nx);
+                        // A last round of L <= 16 slots (unclamped START walk): S = the
+                        // power of two >= L (at least 4 on the paired walk); slot q = lane mod S is walked by the 32 / S
+                        // lanes lane = q + S p, lane p taking rows S p .. S p + S - 1 in
+                        // S Gray-code steps (row = lane ^ g(t), t < S).  Every (slot, row)
+                        // is added once, the 32 lanes stay on 32 banks, and the start
+                        // X = A - cb - lane D and the step table are those of a full round.
+                        // (A short pass walks Srows steps with one slot per lane instead.)
+                        if (!SHORT && MODE == FH_MODE_START && fast && T - base <= 16) {
+                            const int L = T - base;
+                            S = L <= 1 && !QUAD ? 1
+                                : L <= 2 && !QUAD ? 2
+                                : L <= 4 ? 4 : L <= 8 ? 8 : 16;
+                            const int src = lane & (S - 1);
+                            a1 = __shfl_sync(kFull, a1, src);
+                            a2 = __shfl_sync(kFull, a2, src);
+                            if constexpr (QUAD) {
+                                b1 = __shfl_sync(kFull, b1, src);
+                                b2 = __shfl_sync(kFull, b2, src);
+                            }
+                            two = __shfl_sync(kFull, (int)two, src) != 0;
+                            owner = __shfl_sync(kFull, owner, src);
+                        }
+                        setup(std::false_type{}, SHORT ? base + lane : base + (lane & (S - 1)),
+                              vlane, a1, a2, b1, b2, two, owner, X1, X2, Y1, Y2, e, ow);
+                    }
                     if (MODE == FH_MODE_START) {
                         using std::make_integer_sequence;
                         // the cell stride as a compile-time constant in the
@@ -1286,12 +1324,7 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                         if constexpr (QUAD) {
                             // the same peaks in direction d_b, in the high halves
                             // (the paired walk runs unclamped only)
-                            if (S == 32)
-                                quad_steps<false>(make_integer_sequence<int, 32>{}, rbase, X1, X2,
-                                                  Y1, Y2, e, st, ee);
-                            else  // e[0] = +-D, + on odd lanes
-                                quad_steps_short(S, rbase, (uint32_t)lane, X1, X2, Y1, Y2,
-                                                 (lane & 1) ? e[0] : -e[0], st);
+                            quad_steps(S, rbase, X1, X2, Y1, Y2, e, st);
                         } else if (fast) {
                             switch (S) {
                             case 1:
@@ -1321,9 +1354,23 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                     }
                 }
                 __syncwarp();
-                int nc = 0;
-                if (lane == 0) nc = atomicAdd(next_chunk, 1);
-                c = __shfl_sync(kFull, nc, 0);
+                if (T < T_all) {
+                    // on to the FFT that slot T belongs to
+                    const unsigned at = __ballot_sync(kFull, has && P <= T && T < P + m);
+                    const int j = __ffs(at) - 1;
+                    skip = T - __shfl_sync(kFull, P, j);
+                    i0 += j;
+                } else {
+                    skip = 0;
+                    i0 += 32;
+                    if (i0 >= i_end) {
+                        if (lane == 0) run = atomicAdd(next_chunk, 1);
+                        run = __shfl_sync(kFull, run, 0);
+                        const int r = run - nwarps;
+                        i0 = (run0 > 0 ? run0 * nwarps + r * run1 : run) * 32;
+                        i_end = i0 + run1 * 32;
+                    }
+                }
             }
             if (sched != nullptr && dsel == 0 && threadIdx.x == 0)
                 *next_item = (int32_t)atomicAdd(sched, 1u);

@@ -1,0 +1,87 @@
+"""Edges of the transform's accumulation (runs of FFTs, whole and short rounds,
+narrowed tiles) and of the selection's block sizes, against the oracle: maps,
+profile picks and counts bit for bit."""
+import numpy as np
+import pytest
+
+from paper_1407_8333_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fh():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1407_8333_gb300 import build, fh as fhmod
+    build.build()
+    fhmod.load()
+    return fhmod
+
+
+def search(fh, inp, pp, weights=None, **shape):
+    import torch
+    n_dir = inp.sky.shape[0]
+    dev = [torch.from_numpy(np.ascontiguousarray(x)).cuda()
+           for x in (inp.t, inp.offsets, inp.freq, inp.v, inp.sky)]
+    plan = fh.fh_create_plan(fh.make_desc(pp, inp.t.shape[0], n_dir, inp.n_peaks, **shape))
+    try:
+        fh.fh_correct_doppler(plan, *dev)
+        if weights is not None:
+            fh.fh_set_weights(plan, weights, 4)
+        maps = torch.empty((n_dir, pp["n_fdot"], pp["n_f0"]), dtype=torch.int32, device="cuda")
+        fh.fh_transform(plan, 0, n_dir, maps)
+        cand = fh.fh_select_candidates(plan, 0, n_dir)
+        return maps.cpu().numpy(), cand.reshape(n_dir, -1, pp["top_k"])
+    finally:
+        fh.fh_destroy_plan(plan)
+
+
+def check(fh, inp, pp, weights=None, **shape):
+    import oracle
+    kw = {} if weights is None else dict(weights=weights, frac_bits=4)
+    want = oracle.search(inp, pp, want_maps=True, **kw)
+    maps, cand = search(fh, inp, pp, weights, **shape)
+    assert np.array_equal(maps, want["maps"])
+    for k in ("cell", "row", "count"):
+        assert np.array_equal(cand[k], want[k])
+
+
+# with 4 warps a run is 3/16 of the FFTs' chunks: 5 chunks of 32 (none), 6 (one each),
+# 11 and 43 (runs of 2 and 8, the last with a remainder)
+@pytest.mark.parametrize("n_fft", [160, 191, 192, 193, 351, 1376])
+@pytest.mark.parametrize("n_dir, n_fdot", [(1, 33), (1, 70), (2, 36), (3, 4), (2, 17)])
+def test_runs_of_ffts(fh, n_fft, n_dir, n_fdot):
+    for p in (0.02, 0.3):   # fewer than a round of slots per 32 FFTs, and many
+        inp, pp = synth.random_case(900 + n_fft + n_fdot, n_fft=n_fft, n_bins=30, n_fdot=n_fdot,
+                                    n_dir=n_dir, p=p, vmax=2e-6)
+        check(fh, inp, pp, block_warps=4, tile_cells=128)
+
+
+@pytest.mark.parametrize("n_fft", [193, 351])
+def test_runs_of_ffts_weighted(fh, n_fft):
+    inp, pp = synth.random_case(77 + n_fft, n_fft=n_fft, n_bins=30, n_fdot=20, n_dir=2, p=0.2)
+    w = 0.25 * (1 + np.arange(2 * n_fft).reshape(2, n_fft) % 7)
+    check(fh, inp, pp, weights=w, block_warps=4, tile_cells=128)
+
+
+@pytest.mark.parametrize("n_bins", [13, 200, 1000, 1531])
+def test_default_tile_of_few_items(fh, n_bins):
+    """The library's own tile where one direction has few items: bands at and
+    around the width it is narrowed to."""
+    for n_dir in (1, 2):
+        inp, pp = synth.random_case(31 + n_bins, n_fft=40, n_bins=n_bins, n_fdot=9, n_dir=n_dir,
+                                    p=0.05, vmax=2e-6)
+        check(fh, inp, pp)
+
+
+# 8 cells per thread in whole warps: one warp up to 256 cells, 1024 threads from 7937,
+# the profile read again per pick beyond 8192
+@pytest.mark.parametrize("subband_bins, k_over", [(1, 1), (85, 3), (256, 1), (257, 1), (1023, 8),
+                                                  (1024, 8), (1171, 7)])
+def test_selection_block_sizes(fh, subband_bins, k_over):
+    inp, pp = synth.random_case(61 + subband_bins, n_fft=12, n_bins=1200, k_over=k_over, n_fdot=3,
+                                n_dir=2, p=0.1, subband_bins=subband_bins, top_k=4,
+                                excl_cells=2 * k_over, sep_cells=3 * k_over)
+    check(fh, inp, pp)
