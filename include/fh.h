@@ -250,14 +250,15 @@ int fh_select_candidates(fh_plan plan, int32_t dir_begin, int32_t n_dir, fh_cand
  * FH_ERR_UNSORTED, FH_ERR_INVALID_ARG) since the last fh_correct_doppler. */
 int fh_sync(fh_plan plan, void *stream);
 
-/* Time fh_transform over its launch shapes on the current directions (at most
- * 8 of them: the per-item work does not depend on the count) and keep the
- * fastest in the plan; returns its tile width and block warps.  The shapes
- * are: pairs on or off (where the plain START map allows them: two
- * directions with one 16-bit count each per shared word, or for a single
- * direction the two 32-row halves of 64-row slabs), block warps (16, 20, 24,
- * 32) and tile widths up to the widest that fits shared memory with the
- * guard cells of that choice; then, for the fastest of them, the item
+/* Time fh_transform over its launch shapes on the current directions (8 of
+ * them, more where their items are few: the per-item work does not depend on the
+ * count) and keep the fastest in the plan; returns its tile width and block
+ * warps.  The shapes are: pairs on or off (where the plain START map allows
+ * them: two directions with one 16-bit count each per shared word, or for a
+ * single direction the two 32-row halves of 64-row slabs), block warps (16, 20,
+ * 24, 32) and tile widths up to the widest that fits shared memory with the
+ * guard cells of that choice (few items: also widths that make whole waves of
+ * them); then, for the fastest of them, the item
  * schedule (blocks taking their next item from a device counter, or every
  * grid-th item).  The shape is chosen for the plan as it stands, weights
  * included: after fh_set_weights, tune again for the weighted map (which

@@ -230,6 +230,7 @@ struct fh_plan_s {
     int32_t n_sb = 0;
     int32_t mode = FH_MODE_START;
     int32_t tile_cells = 0;
+    bool tile_auto = false;  // the library's own tile: narrowed where items are few
     int32_t block_warps = 32;
     double *t = nullptr, *freq = nullptr, *v = nullptr, *sky = nullptr;
     int64_t *offsets = nullptr, *S0 = nullptr, *D = nullptr, *A = nullptr;
@@ -470,6 +471,7 @@ int fh_create_plan(const fh_plan_desc *desc, fh_plan *out)
         delete p;
         return set_error(FH_ERR_INVALID_ARG, "tile_cells too wide for shared memory");
     }
+    p->tile_auto = desc->tile_cells == 0;
     const Sizes s = plan_sizes(*desc);
     struct {
         void **ptr;
@@ -850,9 +852,23 @@ static int32_t plan_guard(fh_plan p, int32_t kind)
                                : p->guard;
 }
 
+// The library's default tile for a call of `stacks` (unit, slab) stacks of tiles:
+// the widest, unless its items fill less than half of the SMs; then as narrow
+// as gives half of them an item (not below 128 cells: every tile repeats the
+// guard cells' work and its windows).  One direction of 21 rows x 10240 cells
+// (8 items at the widest tile): transform 16.6 us, 10.7 us at 128 cells, with the
+// window pre-pass 24.2 and 20.7 us (256 cells: 20.0, 96 cells: 23.5).
+static int32_t filling_tile(int32_t widest, int32_t n_f0, int64_t stacks, int32_t n_sm)
+{
+    const int64_t half = std::max(1, n_sm / 2);
+    if (stacks * ((n_f0 + widest - 1) / widest) >= half) return widest;
+    const int64_t w = ((int64_t)n_f0 * stacks + half - 1) / half;
+    return std::min<int32_t>(widest, (int32_t)std::max<int64_t>(128, (w + 15) / 16 * 16));
+}
+
 static int run_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *out_maps,
                          int32_t tile, int32_t nwarps, int32_t schedule, cudaStream_t s,
-                         int32_t pair_pref, int32_t item_counter)
+                         int32_t pair_pref, int32_t item_counter, bool tile_auto = false)
 {
     const fh_plan_desc &d = p->d;
     // keep the tile's counters within shared memory with this plan's guard cells
@@ -861,6 +877,13 @@ static int run_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *o
     const int32_t guard = plan_guard(p, kind);
     const int32_t wmax = default_tile(d, p->device, p->mode, nwarps, guard);
     if (tile > wmax) tile = wmax;
+    if (tile_auto) {
+        const int32_t rows = kind == kPairRows ? 2 * kRows : kRows;
+        tile = filling_tile(tile, d.n_f0,
+                            (int64_t)(pairs ? (n_dir + 1) / 2 : n_dir) *
+                                ((d.n_fdot + rows - 1) / rows),
+                            p->n_sm);
+    }
     const size_t smem = transform_smem_bytes(tile, d.k_over, p->mode, nwarps, guard);
     int rc = prepare_transform(p, p->mode, smem);
     if (rc) return rc;
@@ -973,7 +996,8 @@ int fh_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *out_maps,
     if (rc) return rc;
     DeviceGuard g(p->device);
     return run_transform(p, dir_begin, n_dir, out_maps, p->tile_cells, p->block_warps,
-                         p->d.schedule, as_stream(stream), p->pair_pref, p->item_counter);
+                         p->d.schedule, as_stream(stream), p->pair_pref, p->item_counter,
+                         p->tile_auto && p->d.schedule == FH_SCHED_BATCHED);
 }
 
 int fh_copy_profile(fh_plan p, int32_t dir_begin, int32_t n_dir, uint64_t *out, void *stream)
@@ -1147,6 +1171,7 @@ int fh_autotune(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *tile_cells
                   p->n_fft, n_dir);
     auto apply = [&](const TuneChoice &c) {
         p->tile_cells = c.tile;
+        p->tile_auto = false;
         p->block_warps = c.warps;
         p->pair_pref = c.pairs ? 0 : 1;
         p->item_counter = c.counter;
@@ -1167,7 +1192,13 @@ int fh_autotune(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *tile_cells
     // fits with that choice's guard cells
     const int lim = max_optin_smem(p->device);
     std::vector<TuneChoice> cands;
-    const int32_t nt = std::min<int32_t>(n_dir, 8);
+    // timed on 8 of the directions, or as many as make four waves of items in
+    // pairs (fewer would rate a shape by how it fills one wave: 256 directions of
+    // 21 rows x 10240 cells, timed on 8, took the unpaired walk, 152 us against 90)
+    const int32_t items_dir = ((d.n_fdot + kRows - 1) / kRows) *
+                              std::max(1, d.n_f0 / default_tile(d, p->device, p->mode, 24,
+                                                                plan_guard(p, kPairDirs)));
+    const int32_t nt = std::min(n_dir, std::max(8, 8 * p->n_sm / items_dir + 2));
     const int32_t pair_kind = plan_pairs(p, nt, 0);
     const bool pairs_ok = pair_kind != kPairNone;
     for (int pr : {1, 0}) {
@@ -1177,8 +1208,19 @@ int fh_autotune(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *tile_cells
             // DIFF kernels: 512 / 1024 threads
             if ((nw == 24 || nw == 20) && p->mode == FH_MODE_DIFF) continue;
             const int32_t wmax = default_tile(d, p->device, p->mode, nw, guard);
-            for (int32_t w : {wmax, 1280, 1024, 768}) {
-                if (w > wmax || w > d.n_f0) continue;
+            std::vector<int32_t> widths{wmax, 1280, 1024, 768};
+            // few items: widths that make 1, 2 and 3 whole waves of them
+            const int64_t rows = pr && pair_kind == kPairRows ? 2 * kRows : kRows;
+            const int64_t stacks = (pr && pair_kind == kPairDirs ? (n_dir + 1) / 2 : n_dir) *
+                                   ((d.n_fdot + rows - 1) / rows);
+            if (stacks * (d.n_f0 / wmax + 1) < 8 * (int64_t)p->n_sm)
+                for (int64_t k = 1; k <= 3; ++k) {
+                    const int64_t tiles = k * p->n_sm / stacks;
+                    if (tiles > 0)
+                        widths.push_back((int32_t)(((d.n_f0 + tiles - 1) / tiles + 15) / 16 * 16));
+                }
+            for (int32_t w : widths) {
+                if (w < 64 || w > wmax || w > d.n_f0) continue;
                 if (transform_smem_bytes(w, d.k_over, p->mode, nw, guard) > (size_t)lim) continue;
                 bool dup = false;
                 for (const auto &c : cands) dup = dup || (c.tile == w && c.warps == nw && c.pairs == pr);
@@ -1187,8 +1229,6 @@ int fh_autotune(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *tile_cells
         }
     }
     if (cands.empty()) cands.push_back({p->tile_cells, p->block_warps, 0, 1, 0.0});
-    // timed on at most 8 of the directions (one window group): the per-item
-    // work, and so the best tile, does not depend on how many there are
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
