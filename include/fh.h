@@ -40,6 +40,10 @@
  * plan's internal buffers.  A plan is used by one host thread at a time, and
  * its work on one stream at a time (its buffers, the transform's item counter
  * among them, are shared by every call on the plan); a server is thread-safe.
+ * Calls without a plan's buffers (clustering, coincidences, peakmap steps,
+ * refinement) take their scratch stream-ordered from a pool of the library that
+ * keeps up to 256 MiB per device between calls and returns it when the process
+ * destroys its last plan.
  */
 #ifndef FH_H
 #define FH_H

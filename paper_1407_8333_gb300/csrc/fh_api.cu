@@ -80,6 +80,54 @@ int max_optin_smem(int device)
     return v > 0 ? v : 48 * 1024;
 }
 
+// One pool per device for the scratch of calls that hold no plan (clustering,
+// vetoes, refinement): memory freed by one call serves the next one, on any
+// thread or stream (the driver orders the reuse).  It keeps at most kScratchKeep
+// bytes across synchronisations, and nothing once the last plan of the process
+// is destroyed.  The default pool keeps nothing, so that every call mapped its
+// memory anew: about 100 us of each clustering, veto or refinement call.
+constexpr uint64_t kScratchKeep = uint64_t(256) << 20;
+constexpr int kMaxDevices = 64;
+static std::mutex g_pool_mu;
+static cudaMemPool_t g_pool[kMaxDevices] = {};
+static bool g_pool_tried[kMaxDevices] = {};
+static int64_t g_plans = 0;
+
+cudaMemPool_t scratch_pool()
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pool_tried[dev]) {
+        g_pool_tried[dev] = true;
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        uint64_t keep = kScratchKeep;
+        if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
+            if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) ==
+                cudaSuccess)
+                g_pool[dev] = pool;
+            else
+                cudaMemPoolDestroy(pool);
+        }
+        cudaGetLastError();
+    }
+    return g_pool[dev];
+}
+
+// plans alive in the process; the last one's destruction trims the pools
+static void count_plans(int change)
+{
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    g_plans += change;
+    if (change < 0 && g_plans == 0)
+        for (cudaMemPool_t pool : g_pool)
+            if (pool) cudaMemPoolTrimTo(pool, 0);
+}
+
 // the error word (bytes 0..3) and the largest |D| (bytes 16..23) of a plan,
 // one allocation cleared by one memset per call
 constexpr size_t kErrWordsBytes = 32;
@@ -508,6 +556,7 @@ int fh_create_plan(const fh_plan_desc *desc, fh_plan *out)
     }
     cudaMemset(p->err, 0, kErrWordsBytes);
     cudaMemset(p->sched, 0, 16);
+    count_plans(1);
     *out = p;
     return FH_OK;
 }
@@ -519,6 +568,7 @@ int fh_destroy_plan(fh_plan p)
         DeviceGuard g(p->device);
         cudaDeviceSynchronize();
         p->release();
+        count_plans(-1);
     }
     delete p;
     return FH_OK;

@@ -162,19 +162,26 @@ cudaError_t launch_fp64_bench(int32_t iters, int32_t grid, double *sink, cudaStr
 cudaError_t launch_smem_atomic_bench(int32_t variant, int32_t iters, int32_t grid,
                                      unsigned long long *sink, cudaStream_t s);
 
-// Device buffers of one call, taken stream-ordered (cudaMallocAsync) and
-// returned stream-ordered when the object goes out of scope.
+// The pool that calls take their scratch from on the current device (fh_api.cu;
+// null where it could not be made: the device's default pool serves then).
+cudaMemPool_t scratch_pool();
+
+// Device buffers of one call, taken stream-ordered and returned stream-ordered
+// when the object goes out of scope.
 struct Scratch {
     cudaStream_t s;
+    cudaMemPool_t pool;
     std::vector<void *> bufs;
-    explicit Scratch(cudaStream_t st) : s(st) {}
+    explicit Scratch(cudaStream_t st) : s(st), pool(scratch_pool()) {}
     Scratch(const Scratch &) = delete;
     Scratch &operator=(const Scratch &) = delete;
     template <typename T>
     cudaError_t get(T **p, size_t n)
     {
         void *q = nullptr;
-        const cudaError_t e = cudaMallocAsync(&q, (n ? n : 1) * sizeof(T), s);
+        const size_t bytes = (n ? n : 1) * sizeof(T);
+        const cudaError_t e = pool ? cudaMallocFromPoolAsync(&q, bytes, pool, s)
+                                   : cudaMallocAsync(&q, bytes, s);
         if (e == cudaSuccess) bufs.push_back(q);
         *p = static_cast<T *>(q);
         return e;

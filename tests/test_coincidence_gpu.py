@@ -207,3 +207,38 @@ def test_scan_tiles(fh, co, n):
     check_cluster(fh, co, a, 2.0)
     check_coinc(fh, co, a[:500], a, 0.0, 0.0, 0.0, (2, 2, 2, 2))
     check_coinc(fh, co, a, a[:300], 0.0, 0.0, 0.0, (2, 2, 2, 2))
+
+
+def test_scratch_shared_by_threads_and_streams(fh):
+    """Calls of several threads, each on its own stream, share the library's
+    scratch pool: every result is that of a call alone; the last plan's
+    destruction between calls (which empties the pool) changes nothing."""
+    import threading
+
+    import torch
+    sets = [dev(synth.candidate_set(60 + k, 0, 3000 + 500 * k, clusters=40)) for k in range(4)]
+    want = [fh.fh_cluster(c, 3.0)[0].clone() for c in sets]
+    torch.cuda.synchronize()
+    bad = []
+
+    def work(k):
+        try:
+            st = torch.cuda.Stream()
+            for r in range(12):
+                c = sets[(k + r) % 4]
+                lab, _ = fh.fh_cluster(c, 3.0, stream=st)
+                st.synchronize()
+                if not torch.equal(lab, want[(k + r) % 4]):
+                    bad.append((k, r))
+                if r == 5:
+                    _, pp = synth.random_case(3)
+                    fh.fh_destroy_plan(fh.fh_create_plan(fh.make_desc(pp, 20, 1, 100)))
+        except Exception as e:  # noqa: BLE001
+            bad.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
