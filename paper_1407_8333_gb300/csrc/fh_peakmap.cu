@@ -17,12 +17,18 @@
 // bins) and the segment's count; a single-block scan turns the counts into the
 // CSR offsets and per-segment bases; a second pass expands the bits into bin
 // indices.  Cleaning works on the peak lists: histograms by global atomics, a
-// warp per FFT for the keep/drop pass (ballot ranks keep the order), the same
-// scan for the new offsets.  The robust statistic needs only the histogram of
+// block per FFT for the passes that need the FFT (ballot ranks keep the order), the
+// same scan for the new offsets.  GB300's binary64 rate is a small fraction of its
+// integer rate, so no per-peak step uses binary64 where integers say the same:
+// gross columns come from integer column edges, the persistency threshold is
+// compared as an integer, and a power-of-two T_FFT gives a frequency's bits by
+// shifts.  The robust statistic needs only the histogram of
 // the per-bin counts (values 0 .. n_fft), so its medians are order statistics
 // found by one block scanning that histogram; every median is exact (integers
 // and half-integers), and m2 and the threshold are single binary64 operations
 // in the order written above.
+#include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdint>
 #include <vector>
@@ -39,16 +45,25 @@ constexpr int kSegWords = kSegBins / 32;
 constexpr int kScanThreads = 1024;
 
 // (k0 + b) / t_fft, the IEEE quotient.  When t_fft is a power of two the
-// quotient is the exact product with inv = 1 / t_fft (also exact), and a
-// binary64 multiply replaces the much slower division.
+// quotient of an integer x in [1, 2^53) is x itself with another exponent: its
+// bits come from integer shifts (a dozen integer instructions; a conversion and
+// a binary64 multiply cost several times that on GB300).
 struct FreqOf {
     int64_t k0;
-    double t_fft, inv;
+    double t_fft;
+    int32_t ex;     // t_fft = 2^ex where pow2
     bool pow2;
     __device__ __forceinline__ double operator()(int32_t b) const
     {
-        const double x = (double)(k0 + b);
-        return pow2 ? __dmul_rn(x, inv) : __ddiv_rn(x, t_fft);
+        const int64_t x = k0 + b;
+        if (pow2 && x > 0 && x < (int64_t(1) << 53)) {
+            const int lz = __clzll(x);
+            // the leading one at bit 52, then dropped (the hidden bit)
+            const uint64_t m = ((uint64_t)x << (lz - 11)) & 0xFFFFFFFFFFFFFull;
+            return __longlong_as_double(
+                (long long)(((uint64_t)(1023 + 63 - lz - ex) << 52) | m));
+        }
+        return __ddiv_rn((double)x, t_fft);
     }
 };
 
@@ -59,8 +74,8 @@ FreqOf make_freq_of(int64_t k0, double t_fft)
     FreqOf f;
     f.k0 = k0;
     f.t_fft = t_fft;
-    f.pow2 = m == 0.5 && ex > -1000 && ex < 1000;
-    f.inv = f.pow2 ? std::ldexp(1.0, 1 - ex) : 0.0;
+    f.ex = ex - 1;
+    f.pow2 = m == 0.5 && ex > -900 && ex < 900;  // every quotient is a normal number
     return f;
 }
 
@@ -72,7 +87,7 @@ struct SelArgs {
     float theta;
     uint32_t *mask;     // [fft][word]
     int32_t *seg_count; // [fft][seg]
-    int32_t *err;       // bulk-copy waits that ran out
+    int32_t *err;       // bulk-copy waits that ran out (Result)
 };
 
 __device__ __forceinline__ float ratio_at(const float *sp, const float *sa, int j, int n_bins)
@@ -335,7 +350,7 @@ tile_sums_kernel(const int32_t *cnt, int64_t n, int64_t *sums)
 template <typename T>
 __global__ void __launch_bounds__(kScanThreads)
 scan_counts_kernel(const int32_t *cnt, int64_t n, T *pref, int32_t stride, int64_t *strided,
-                   const int64_t *sums)
+                   const int64_t *sums, int64_t *total)
 {
     __shared__ int64_t part[kScanThreads / 32];
     __shared__ int64_t carry;
@@ -395,6 +410,7 @@ scan_counts_kernel(const int32_t *cnt, int64_t n, T *pref, int32_t stride, int64
             if (base + kScanTile >= n) {
                 if (pref) pref[n] = (T)run;
                 if (strided) strided[n / stride] = run;
+                if (total) *total = run;
             }
         }
         __syncthreads();
@@ -403,6 +419,14 @@ scan_counts_kernel(const int32_t *cnt, int64_t n, T *pref, int32_t stride, int64
 }
 
 // ---------------------------------------------------------------- cleaning
+// What a call reads back: one small copy at its end.
+struct Result {
+    int32_t err;       // kErr* bits
+    int32_t thr;       // persistency: a bin's count stays up to this
+    int64_t total;     // peaks selected or kept
+    double stats[3];   // persistency: m1, m2, threshold
+};
+
 // The peak range of FFT i, clamped into [0, n_peaks] whatever the offsets hold;
 // a CSR that is not one (o[0] != 0, o[n] != n_peaks or a decrease) is flagged.
 __device__ __forceinline__ void peak_range(const int64_t *o, int i, int64_t n_peaks, int64_t &lo,
@@ -412,9 +436,10 @@ __device__ __forceinline__ void peak_range(const int64_t *o, int i, int64_t n_pe
     hi = min(max(o[i + 1], lo), n_peaks);
 }
 
-__global__ void check_csr_kernel(const int64_t *o, int32_t n_fft, int64_t n_peaks, int32_t *err)
+__device__ __forceinline__ void check_csr(const int64_t *o, int32_t n_fft, int64_t n_peaks,
+                                          int64_t first, int64_t step, int32_t *err)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= n_fft; i += gridDim.x * blockDim.x) {
+    for (int64_t i = first; i <= n_fft; i += step) {
         bool bad = false;
         if (i == 0) bad = o[0] != 0;
         if (i == n_fft) bad = bad || o[n_fft] != n_peaks;
@@ -436,7 +461,7 @@ __device__ __forceinline__ double floor_quot(double num, double den, double inv)
     return floor(__ddiv_rn(num, den));
 }
 
-struct GrossCell {
+struct GrossGrid {
     const double *t;
     FreqOf fq;
     double t0_h, dt_h, f0_h, df_h, inv_df;
@@ -447,63 +472,124 @@ struct GrossCell {
         const double x = floor(__ddiv_rn(__dsub_rn(__ldg(t + i), t0_h), dt_h));
         return (x >= 0.0 && x < (double)n_th) ? (int64_t)x : -1;
     }
-    // gross cell of a peak of bin b in time cell it, or -1 off the grid
-    __device__ __forceinline__ int32_t cell(int64_t it, int32_t b) const
+    // frequency cell of bin b (may lie off the grid); non-decreasing in b, each
+    // of its operations being so
+    __device__ __forceinline__ double column(int64_t b) const
     {
-        if (it < 0) return -1;
-        const double y = floor_quot(__dsub_rn(fq(b), f0_h), df_h, inv_df);
-        return (y >= 0.0 && y < (double)n_fh) ? (int32_t)(it * n_fh + (int64_t)y) : -1;
+        return floor_quot(__dsub_rn(fq((int32_t)b), f0_h), df_h, inv_df);
     }
 };
 
-// warp per FFT: the gross cell of every peak (kept for the veto pass) and the
-// histogram (warp-aggregated atomics)
-__global__ void gross_hist_kernel(const int64_t *o, const int32_t *bins, int32_t n_fft,
-                                  int64_t n_peaks, GrossCell g, int32_t *cell, int32_t *hist)
+// Set-up of the gross veto: the CSR check, the cleared histogram and the column
+// edges: edge[y], y = 0 .. n_fh, the first bin whose frequency cell is y or more
+// (2^31 where no bin's is).  The bin that the grid names first, two to each side,
+// brackets nearly every edge; else the whole range of bins is searched.
+__global__ void __launch_bounds__(256)
+gross_setup_kernel(const int64_t *o, int32_t n_fft, int64_t n_peaks, GrossGrid g, int64_t *edge,
+                   int32_t *hist, int64_t cells, int32_t *err)
 {
-    const int lane = threadIdx.x & 31;
-    const int nw = gridDim.x * (blockDim.x >> 5);
-    for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n_fft; i += nw) {
-        int64_t lo, hi;
-        peak_range(o, i, n_peaks, lo, hi);
-        const int64_t it = g.it_of(i);
-        for (int64_t q0 = lo; q0 < hi; q0 += 32) {
-            const int64_t q = q0 + lane;
-            const int32_t c = q < hi ? g.cell(it, __ldg(bins + q)) : -1;
-            if (q < hi) cell[q] = c;
-            // neighbouring peaks of an FFT mostly share a cell: one atomic per
-            // distinct cell of the warp, adding its number of lanes
-            const unsigned same = __match_any_sync(kFull, c);
-            if (c >= 0 && lane == __ffs(same) - 1) atomicAdd(hist + c, __popc(same));
+    const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    check_csr(o, n_fft, n_peaks, first, step, err);
+    for (int64_t k = first; k < cells; k += step) hist[k] = 0;
+    for (int64_t y = first; y <= g.n_fh; y += step) {
+        const int64_t kmin = INT_MIN, kmax = (int64_t)INT_MAX + 1;
+        int64_t lo = kmin, hi = kmax;  // column(lo - 1) < y <= column(hi)
+        const double guess = (g.f0_h + (double)y * g.df_h) * g.fq.t_fft - (double)g.fq.k0;
+        if (guess > -2e9 && guess < 2e9) {
+            const int64_t c = (int64_t)guess;
+            if (g.column(c - 2) < (double)y && g.column(c + 2) >= (double)y) {
+                lo = c - 1;
+                hi = c + 2;
+            }
+        }
+        while (lo < hi) {
+            const int64_t m = (lo + hi) >> 1;  // m < hi <= 2^31
+            if (g.column(m) >= (double)y) hi = m; else lo = m + 1;
+        }
+        edge[y] = lo;
+    }
+}
+
+// a block per FFT: 620 peaks in 5 steps of 128 (a warp per FFT left two thirds of
+// the SMs' warps empty and every FFT a chain of 20 steps)
+constexpr int kFftThreads = 128;
+
+// The gross cell of every peak (kept for the veto pass) and the histogram: one
+// atomic per run of peaks in one cell of a warp (an FFT's peaks come in bin
+// order).  1.96 million peaks: 75 -> 17 us against a warp per FFT with each
+// column from binary64 and warp-wide matches.
+__global__ void __launch_bounds__(kFftThreads)
+gross_hist_kernel(const int64_t *o, const int32_t *bins, int64_t n_peaks, GrossGrid g,
+                  const int64_t *__restrict__ edge, int32_t *cell, int32_t *hist)
+{
+    __shared__ int64_t it_s;
+    const int i = blockIdx.x, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) it_s = g.it_of(i);
+    __syncthreads();
+    const int64_t it = it_s;
+    int64_t lo, hi;
+    peak_range(o, i, n_peaks, lo, hi);
+    const int64_t e0 = edge[0], e1 = edge[g.n_fh];
+    const float per_bin = (float)g.n_fh / fmaxf(1.0f, (float)(e1 - e0));
+    for (int64_t q0 = lo + (threadIdx.x & ~31); q0 < hi; q0 += kFftThreads) {
+        const int64_t q = q0 + lane;
+        int32_t c = -1;
+        if (q < hi && it >= 0) {
+            const int32_t b = __ldg(bins + q);
+            if (b >= e0 && b < e1) {
+                int32_t y = min((int32_t)((float)(b - e0) * per_bin), g.n_fh - 1);
+                // the edges are evenly spaced to a bin, so the estimate is off by one at
+                // most; a grid that is not takes the search
+                if (b < edge[y]) --y;
+                else if (b >= edge[y + 1]) ++y;
+                if (y < 0 || y >= g.n_fh || b < edge[y] || b >= edge[y + 1]) {
+                    int32_t a = 0, z = g.n_fh;  // edge[a] <= b < edge[z]
+                    while (z - a > 1) {
+                        const int32_t m = a + (z - a) / 2;
+                        if (edge[m] <= b) a = m; else z = m;
+                    }
+                    y = a;
+                }
+                c = (int32_t)(it * g.n_fh + y);
+            }
+        }
+        if (q < hi) cell[q] = c;
+        const int32_t left = __shfl_up_sync(kFull, c, 1);
+        const bool head = lane == 0 || c != left;
+        const unsigned heads = __ballot_sync(kFull, head);
+        if (head && c >= 0) {
+            const unsigned after = lane == 31 ? 0u : heads >> (lane + 1);
+            atomicAdd(hist + c, after ? __ffs(after) : 32 - lane);
         }
     }
 }
 
-// warp per FFT: FFTs with a peak in each bin (bins outside [0, n_bins) are flagged)
-__global__ void bin_hist_kernel(const int64_t *o, const int32_t *bins, int32_t n_fft,
-                                int64_t n_peaks, int32_t n_bins, int32_t *hist, int32_t *err)
+// FFTs with a peak in each bin (bins outside [0, n_bins) are flagged), a thread
+// per peak (1.9 million: 48 -> 20 us against a warp per FFT); the CSR check rides
+// along
+__global__ void __launch_bounds__(256)
+bin_hist_kernel(const int64_t *o, const int32_t *bins, int32_t n_fft, int64_t n_peaks,
+                int32_t n_bins, int32_t *hist, int32_t *err)
 {
-    const int lane = threadIdx.x & 31;
-    const int nw = gridDim.x * (blockDim.x >> 5);
-    for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n_fft; i += nw) {
-        int64_t lo, hi;
-        peak_range(o, i, n_peaks, lo, hi);
-        for (int64_t q = lo + lane; q < hi; q += 32) {
-            const int32_t b = __ldg(bins + q);
-            if (b >= 0 && b < n_bins)
-                atomicAdd(hist + b, 1);
-            else
-                atomicOr(err, kErrInvalid);
-        }
+    const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    check_csr(o, n_fft, n_peaks, first, step, err);
+    for (int64_t q = first; q < n_peaks; q += step) {
+        const int32_t b = __ldg(bins + q);
+        if (b >= 0 && b < n_bins)
+            atomicAdd(hist + b, 1);
+        else
+            atomicOr(err, kErrInvalid);
     }
 }
 
 // histogram of the per-bin counts: hc[v] = bins whose count is v (v <= vmax;
 // larger counts, possible only for an invalid CSR, go to vmax and are flagged)
-__global__ void count_hist_kernel(const int32_t *hist, int32_t n_bins, int32_t vmax, int32_t *hc,
-                                  int32_t *err)
+__device__ __forceinline__ void count_values(const int32_t *hist, int32_t n_bins, int32_t vmax,
+                                             int first, int step, int32_t *hc, int32_t *err)
 {
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < n_bins; b += gridDim.x * blockDim.x) {
+    for (int b = first; b < n_bins; b += step) {
         int32_t v = hist[b];
         if (v < 0 || v > vmax) {
             atomicOr(err, kErrInvalid);
@@ -512,11 +598,17 @@ __global__ void count_hist_kernel(const int32_t *hist, int32_t n_bins, int32_t v
         atomicAdd(hc + v, 1);
     }
 }
+__global__ void count_hist_kernel(const int32_t *hist, int32_t n_bins, int32_t vmax, int32_t *hc,
+                                  int32_t *err)
+{
+    count_values(hist, n_bins, vmax, blockIdx.x * blockDim.x + threadIdx.x,
+                 gridDim.x * blockDim.x, hc, err);
+}
 
-// the k-th smallest (0-based) of a multiset given by its value histogram
-// h[0 .. nv): one block; every thread scans a contiguous run of values
-__device__ int64_t kth_of_hist(const int32_t *h, int64_t nv, int64_t k, int64_t *part,
-                               int64_t *result)
+// the ka-th and kb-th smallest (0-based, ka <= kb) of a multiset given by its value
+// histogram h[0 .. nv): one block; every thread scans a contiguous run of values
+__device__ void kth_of_hist(const int32_t *h, int64_t nv, int64_t ka, int64_t kb, int64_t *part,
+                            int64_t (&result)[2])
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t per = (nv + blockDim.x - 1) / blockDim.x;
@@ -530,41 +622,51 @@ __device__ int64_t kth_of_hist(const int32_t *h, int64_t nv, int64_t k, int64_t 
         if (lane >= o) p += y;
     }
     if (lane == 31) part[warp] = p;
-    if (tid == 0) *result = nv - 1;
+    if (tid == 0) result[0] = result[1] = nv - 1;
     __syncthreads();
-    int64_t run = p - s;
-    for (int q = 0; q < warp; ++q) run += part[q];
-    if (run <= k && k < run + s) {
+    int64_t before = lane < warp ? part[lane] : 0;  // (at most 32 warps)
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
+    int64_t run = before + p - s;
+    if (run <= kb && ka < run + s) {
         for (int64_t v = lo; v < hi; ++v) {
-            run += h[v];
-            if (k < run) {
-                *result = v;
-                break;
-            }
+            const int64_t next = run + h[v];
+            if (run <= ka && ka < next) result[0] = v;
+            if (run <= kb && kb < next) result[1] = v;
+            run = next;
         }
     }
     __syncthreads();
-    const int64_t r = *result;
-    __syncthreads();
-    return r;
 }
 
 // App. "Robust statistic" on the per-bin counts, from their value histogram
 // hc (vmax + 1 values) and n_bins values in all: m1 = median, m2 =
 // median(|x - m1|) / 0.6745, thr = m1 + k m2.  The deviations are half-integers;
 // hd (2 vmax + 1 entries, zeroed) receives their doubled values.  One block.
+// With `counts` the block forms hc itself, and both histograms live in shared
+// memory (bands and FFT counts small enough: 8192 bins and 3164 FFTs take 10 us
+// against 14 us for the two kernels on global memory).
+constexpr int kSmallValues = 12000;  // words of shared memory for hc and hd
 __global__ void __launch_bounds__(kScanThreads)
-robust_stats_kernel(const int32_t *hc, int32_t vmax, int64_t n_bins, int32_t *hd, double k_sigma,
-                    double *stats)
+robust_stats_kernel(const int32_t *counts, int32_t *hc, int32_t vmax, int32_t n_bins, int32_t *hd,
+                    double k_sigma, Result *res_out)
 {
+    extern __shared__ int32_t small_s[];
     __shared__ int64_t part[kScanThreads / 32];
-    __shared__ int64_t res;
+    __shared__ int64_t res[2];
     const int64_t nv = (int64_t)vmax + 1;
+    const int64_t nd = 2 * nv + 1;
+    if (counts) {
+        hc = small_s;
+        hd = small_s + nv;
+        for (int64_t v = threadIdx.x; v < nv + nd; v += blockDim.x) small_s[v] = 0;
+        __syncthreads();
+        count_values(counts, n_bins, vmax, threadIdx.x, blockDim.x, hc, &res_out->err);
+        __syncthreads();
+    }
     // median of an even count: the mean of the two middle values
-    const int64_t ka = (n_bins - 1) / 2, kb = n_bins / 2;
-    const int64_t va = kth_of_hist(hc, nv, ka, part, &res);
-    const int64_t vb = kth_of_hist(hc, nv, kb, part, &res);
-    const int64_t m1x2 = va + vb;  // 2 m1, an integer
+    const int64_t ka = ((int64_t)n_bins - 1) / 2, kb = (int64_t)n_bins / 2;
+    kth_of_hist(hc, nv, ka, kb, part, res);
+    const int64_t m1x2 = res[0] + res[1];  // 2 m1, an integer
     for (int64_t v = threadIdx.x; v < nv; v += blockDim.x) {
         const int32_t c = hc[v];
         if (c) {
@@ -573,17 +675,19 @@ robust_stats_kernel(const int32_t *hc, int32_t vmax, int64_t n_bins, int32_t *hd
         }
     }
     __syncthreads();
-    const int64_t nd = 2 * nv + 1;
-    const int64_t da = kth_of_hist(hd, nd, ka, part, &res);
-    const int64_t db = kth_of_hist(hd, nd, kb, part, &res);
+    kth_of_hist(hd, nd, ka, kb, part, res);
     if (threadIdx.x == 0) {
         const double m1 = __ddiv_rn((double)m1x2, 2.0);
-        // median of |x - m1| = (da / 2 + db / 2) / 2, exact for these sizes
-        const double med = __ddiv_rn((double)(da + db), 4.0);
+        // median of |x - m1| = the mean of the two halves, exact for these sizes
+        const double med = __ddiv_rn((double)(res[0] + res[1]), 4.0);
         const double m2 = __ddiv_rn(med, 0.6745);
-        stats[0] = m1;
-        stats[1] = m2;
-        stats[2] = __dadd_rn(m1, __dmul_rn(k_sigma, m2));
+        const double thr = __dadd_rn(m1, __dmul_rn(k_sigma, m2));
+        res_out->stats[0] = m1;
+        res_out->stats[1] = m2;
+        res_out->stats[2] = thr;
+        // count > thr exactly when count > floor(thr), the counts being integers
+        const double f = floor(thr);
+        res_out->thr = f >= 2147483647.0 ? INT_MAX : f <= -2147483648.0 ? INT_MIN : (int32_t)f;
     }
 }
 
@@ -591,7 +695,7 @@ robust_stats_kernel(const int32_t *hc, int32_t vmax, int64_t n_bins, int32_t *hd
 struct KeepGross {
     const int32_t *cell, *hist;
     int32_t thr;
-    __device__ __forceinline__ bool operator()(int, int64_t q, int32_t) const
+    __device__ __forceinline__ bool operator()(int64_t q, int32_t) const
     {
         const int32_t c = cell[q];
         return c < 0 || hist[c] <= thr;
@@ -600,59 +704,65 @@ struct KeepGross {
 // which peaks stay: the bin's count is not above the persistency threshold
 struct KeepPersist {
     const int32_t *hist;
-    const double *stats;
+    const Result *res;
     int32_t n_bins;
-    __device__ __forceinline__ bool operator()(int, int64_t, int32_t b) const
+    __device__ __forceinline__ bool operator()(int64_t, int32_t b) const
     {
-        return b < 0 || b >= n_bins || !((double)hist[b] > stats[2]);
+        return b < 0 || b >= n_bins || hist[b] <= res->thr;
     }
 };
 
-// warp per FFT: kept peaks per FFT
+// a block per FFT: kept peaks of the FFT
 template <class Keep>
-__global__ void filter_count_kernel(const int64_t *o, const int32_t *bins, int32_t n_fft,
-                                    int64_t n_peaks, Keep keep, int32_t *cnt)
+__global__ void __launch_bounds__(kFftThreads)
+filter_count_kernel(const int64_t *o, const int32_t *bins, int64_t n_peaks, Keep keep,
+                    int32_t *cnt)
 {
-    const int lane = threadIdx.x & 31;
-    const int nw = gridDim.x * (blockDim.x >> 5);
-    for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n_fft; i += nw) {
-        int64_t lo, hi;
-        peak_range(o, i, n_peaks, lo, hi);
-        int c = 0;
-        for (int64_t q0 = lo; q0 < hi; q0 += 32) {
-            const int64_t q = q0 + lane;
-            const bool k = q < hi && keep(i, q, __ldg(bins + q));
-            c += __popc(__ballot_sync(kFull, k));
-        }
-        if (lane == 0) cnt[i] = c;
-    }
+    __shared__ int sum;
+    const int i = blockIdx.x;
+    if (threadIdx.x == 0) sum = 0;
+    __syncthreads();
+    int64_t lo, hi;
+    peak_range(o, i, n_peaks, lo, hi);
+    int c = 0;
+    for (int64_t q = lo + threadIdx.x; q < hi; q += kFftThreads) c += keep(q, __ldg(bins + q));
+    c = __reduce_add_sync(kFull, c);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&sum, c);
+    __syncthreads();
+    if (threadIdx.x == 0) cnt[i] = sum;
 }
 
-// warp per FFT: the kept peaks, in order, from the FFT's new offset
+// a block per FFT: the kept peaks, in order, from the FFT's new offset
 template <class Keep>
-__global__ void filter_write_kernel(const int64_t *o, const int32_t *bins, int32_t n_fft,
-                                    int64_t n_peaks, Keep keep, const int64_t *o_out,
-                                    int64_t capacity, FreqOf fq, int32_t *bins_out,
-                                    double *freq_out)
+__global__ void __launch_bounds__(kFftThreads)
+filter_write_kernel(const int64_t *o, const int32_t *bins, int64_t n_peaks, Keep keep,
+                    const int64_t *o_out, int64_t capacity, FreqOf fq, int32_t *bins_out,
+                    double *freq_out)
 {
-    const int lane = threadIdx.x & 31;
+    constexpr int kWarps = kFftThreads / 32;
+    __shared__ int kept[2][kWarps];
+    const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    const int nw = gridDim.x * (blockDim.x >> 5);
-    for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n_fft; i += nw) {
-        int64_t lo, hi;
-        peak_range(o, i, n_peaks, lo, hi);
-        int64_t pos = o_out[i];
-        for (int64_t q0 = lo; q0 < hi; q0 += 32) {
-            const int64_t q = q0 + lane;
-            const int32_t b = q < hi ? __ldg(bins + q) : 0;
-            const bool k = q < hi && keep(i, q, b);
-            const unsigned m = __ballot_sync(kFull, k);
-            const int64_t at = pos + __popc(m & lt);
-            if (k && at < capacity) {
-                bins_out[at] = b;
-                if (freq_out) freq_out[at] = fq(b);
-            }
-            pos += __popc(m);
+    int64_t lo, hi;
+    peak_range(o, i, n_peaks, lo, hi);
+    int64_t pos = o_out[i];
+    int turn = 0;
+    for (int64_t q0 = lo; q0 < hi; q0 += kFftThreads, turn ^= 1) {
+        const int64_t q = q0 + threadIdx.x;
+        const int32_t b = q < hi ? __ldg(bins + q) : 0;
+        const bool k = q < hi && keep(q, b);
+        const unsigned m = __ballot_sync(kFull, k);
+        if (lane == 0) kept[turn][warp] = __popc(m);
+        __syncthreads();  // (the other half is free: every thread is past its last use)
+        int64_t at = pos + __popc(m & lt);
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            at += w < warp ? kept[turn][w] : 0;
+            pos += kept[turn][w];
+        }
+        if (k && at < capacity) {
+            bins_out[at] = b;
+            if (freq_out) freq_out[at] = fq(b);
         }
     }
 }
@@ -670,7 +780,8 @@ cudaError_t scan_exclusive(const int32_t *cnt, int64_t n, T *pref, Scratch &sc, 
         tile_sums_kernel<<<(unsigned)tiles, kScanThreads, 0, s>>>(cnt, n, sums);
     }
     scan_counts_kernel<T><<<sums ? (unsigned)tiles : 1u, kScanThreads, 0, s>>>(cnt, n, pref, 1,
-                                                                              nullptr, sums);
+                                                                              nullptr, sums,
+                                                                              nullptr);
     return cudaGetLastError();
 }
 template cudaError_t scan_exclusive<int32_t>(const int32_t *, int64_t, int32_t *, Scratch &,
@@ -680,48 +791,42 @@ template cudaError_t scan_exclusive<int64_t>(const int32_t *, int64_t, int64_t *
 
 namespace {
 
-int warp_grid(int32_t n_fft)
-{
-    const int per_block = 8;  // warps of a 256-thread block
-    return (int)std::min<int64_t>(((int64_t)n_fft + per_block - 1) / per_block, 65535);
-}
-
-// kept peaks -> new CSR and lists; *n_out and the device error word on the host
+// kept peaks -> new CSR and lists; *n_out (and the statistics) on the host
 template <class Keep>
 int run_filter(const int64_t *o, const int32_t *bins, int32_t n_fft, int64_t n_peaks, Keep keep,
                int64_t k0, double t_fft, int64_t *o_out, int32_t *bins_out, double *freq_out,
-               int64_t capacity, int64_t *n_out, const int32_t *err, Scratch &sc, cudaStream_t s)
+               int64_t capacity, int64_t *n_out, Result *res, double *stats, Scratch &sc,
+               cudaStream_t s)
 {
     int32_t *cnt = nullptr;
     cudaError_t e = sc.get(&cnt, (size_t)n_fft);
-    const int grid = warp_grid(n_fft);
     if (e == cudaSuccess && n_fft > 0) {
-        filter_count_kernel<<<grid, 256, 0, s>>>(o, bins, n_fft, n_peaks, keep, cnt);
+        filter_count_kernel<<<n_fft, kFftThreads, 0, s>>>(o, bins, n_peaks, keep, cnt);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
         scan_counts_kernel<int64_t><<<1, kScanThreads, 0, s>>>(cnt, n_fft, o_out, 1, nullptr,
-                                                               nullptr);
+                                                               nullptr, &res->total);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && n_fft > 0) {
-        filter_write_kernel<<<grid, 256, 0, s>>>(o, bins, n_fft, n_peaks, keep, o_out, capacity,
-                                                 make_freq_of(k0, t_fft), bins_out, freq_out);
+        filter_write_kernel<<<n_fft, kFftThreads, 0, s>>>(o, bins, n_peaks, keep, o_out, capacity,
+                                                          make_freq_of(k0, t_fft), bins_out,
+                                                          freq_out);
         e = cudaGetLastError();
     }
-    int64_t total = 0;
-    int32_t h_err = 0;
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&total, o_out + n_fft, sizeof(total), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s);
+    Result h{};
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, res, sizeof h, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_error(e, "peakmap filter");
-    if (h_err & kErrCsr) return set_error(FH_ERR_INVALID_ARG, "offsets are not a CSR of n_peaks");
-    if (h_err & kErrInvalid)
+    if (stats)
+        for (int k = 0; k < 3; ++k) stats[k] = h.stats[k];
+    if (h.err & kErrCsr) return set_error(FH_ERR_INVALID_ARG, "offsets are not a CSR of n_peaks");
+    if (h.err & kErrInvalid)
         return set_error(FH_ERR_INVALID_ARG, "a bin index outside [0, n_bins)");
-    *n_out = total;
-    if (total > capacity)
-        return set_error(FH_ERR_CAPACITY, "%lld peaks kept, capacity %lld", (long long)total,
+    *n_out = h.total;
+    if (h.total > capacity)
+        return set_error(FH_ERR_CAPACITY, "%lld peaks kept, capacity %lld", (long long)h.total,
                          (long long)capacity);
     return FH_OK;
 }
@@ -780,8 +885,9 @@ int fh_peakmap_select(const float *s_p, const float *s_ar, int32_t n_fft, int32_
     if (n_fft > 65535) return set_error(FH_ERR_INVALID_ARG, "at most 65535 FFTs per call");
     Scratch sc(s);
     uint32_t *mask = nullptr;
-    int32_t *seg_count = nullptr, *err = nullptr;
+    int32_t *seg_count = nullptr;
     int64_t *seg_base = nullptr;
+    Result *res = nullptr;
     cudaError_t e = cudaSuccess;
     const int64_t need = fh_peakmap_select_workspace(n_fft, n_bins);
     if (workspace) {
@@ -794,18 +900,19 @@ int fh_peakmap_select(const float *s_p, const float *s_ar, int32_t n_fft, int32_
         seg_count = reinterpret_cast<int32_t *>(w + up(4 * (int64_t)n_fft * n_words));
         seg_base = reinterpret_cast<int64_t *>(w + up(4 * (int64_t)n_fft * n_words) +
                                                up(4 * (int64_t)n_fft * n_seg));
-        err = reinterpret_cast<int32_t *>(w + need - 256);
+        res = reinterpret_cast<Result *>(w + need - 256);
     } else {
         e = sc.get(&mask, (size_t)n_fft * n_words);
         if (e == cudaSuccess) e = sc.get(&seg_count, (size_t)n_fft * n_seg);
         if (e == cudaSuccess) e = sc.get(&seg_base, (size_t)n_fft * n_seg + 1);
-        if (e == cudaSuccess) e = sc.get(&err, 4);
+        if (e == cudaSuccess) e = sc.get(&res, 1);
         if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync (peakmap)");
     }
-    SelArgs a{s_p, s_ar, pitch, n_fft, n_bins, n_seg, n_words, theta, mask, seg_count, err};
+    SelArgs a{s_p, s_ar, pitch, n_fft, n_bins, n_seg, n_words, theta, mask, seg_count,
+              &res->err};
     const bool vec = ((reinterpret_cast<uintptr_t>(s_p) | reinterpret_cast<uintptr_t>(s_ar)) &
                       15u) == 0 && (pitch & 3) == 0;
-    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 4, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(res, 0, sizeof(Result), s);
     if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync (peakmap)");
     if (vec && (n_bins & 3) == 0)
         select_mask_bulk_kernel<<<dim3(n_seg, n_fft), kSegThreads, 0, s>>>(a);
@@ -816,7 +923,7 @@ int fh_peakmap_select(const float *s_p, const float *s_ar, int32_t n_fft, int32_
     e = cudaGetLastError();
     if (e == cudaSuccess) {
         scan_counts_kernel<int64_t><<<1, kScanThreads, 0, s>>>(
-            seg_count, (int64_t)n_fft * n_seg, seg_base, n_seg, offsets, nullptr);
+            seg_count, (int64_t)n_fft * n_seg, seg_base, n_seg, offsets, nullptr, &res->total);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
@@ -827,17 +934,15 @@ int fh_peakmap_select(const float *s_p, const float *s_ar, int32_t n_fft, int32_
     }
     if (e != cudaSuccess) return cuda_error(e, "peak selection");
     if (!n_peaks) return FH_OK;  // asynchronous: the total is offsets[n_fft]
-    int64_t total = 0;
-    int32_t h_err = 0;
-    e = cudaMemcpyAsync(&total, offsets + n_fft, sizeof(total), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s);
+    Result h{};
+    e = cudaMemcpyAsync(&h, res, sizeof h, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_error(e, "peak selection");
-    if (h_err) return set_error(FH_ERR_TIMEOUT, "peak selection: a bulk-copy wait ran out");
-    *n_peaks = total;
-    if (total > capacity)
-        return set_error(FH_ERR_CAPACITY, "%lld peaks selected, capacity %lld", (long long)total,
-                         (long long)capacity);
+    if (h.err) return set_error(FH_ERR_TIMEOUT, "peak selection: a bulk-copy wait ran out");
+    *n_peaks = h.total;
+    if (h.total > capacity)
+        return set_error(FH_ERR_CAPACITY, "%lld peaks selected, capacity %lld",
+                         (long long)h.total, (long long)capacity);
     return FH_OK;
 }
 
@@ -858,25 +963,30 @@ int fh_peakmap_gross_veto(const double *t, const int64_t *offsets, const int32_t
         return set_error(FH_ERR_INVALID_ARG, "bad gross grid (n_th, n_fh >= 1, steps > 0)");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     Scratch sc(s);
-    int32_t *err = nullptr;
-    cudaError_t e = sc.get(&err, 1);
-    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 4, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(hist, 0, sizeof(int32_t) * (size_t)n_th * n_fh, s);
+    Result *res = nullptr;
+    int32_t *cell = nullptr;
+    int64_t *edge = nullptr;
+    cudaError_t e = sc.get(&res, 1);
+    if (e == cudaSuccess) e = sc.get(&cell, (size_t)n_peaks);
+    if (e == cudaSuccess) e = sc.get(&edge, (size_t)n_fh + 1);
+    if (e == cudaSuccess) e = cudaMemsetAsync(res, 0, sizeof(Result), s);
+    const GrossGrid g{t, make_freq_of(k0, t_fft), t0_h, dt_h, f0_h, df_h, 1.0 / df_h, n_th, n_fh};
+    const int64_t cells = (int64_t)n_th * n_fh;
     if (e == cudaSuccess) {
-        check_csr_kernel<<<(n_fft + 256) / 256, 256, 0, s>>>(offsets, n_fft, n_peaks, err);
+        const int64_t work = std::max({cells, (int64_t)n_fh + 1, (int64_t)n_fft + 1});
+        const int grid = (int)std::min<int64_t>((work + 255) / 256, 4096);
+        gross_setup_kernel<<<grid, 256, 0, s>>>(offsets, n_fft, n_peaks, g, edge, hist, cells,
+                                                &res->err);
         e = cudaGetLastError();
     }
-    GrossCell g{t, make_freq_of(k0, t_fft), t0_h, dt_h, f0_h, df_h, 1.0 / df_h, n_th, n_fh};
-    int32_t *cell = nullptr;
-    if (e == cudaSuccess) e = sc.get(&cell, (size_t)n_peaks);
     if (e == cudaSuccess && n_fft > 0) {
-        gross_hist_kernel<<<warp_grid(n_fft), 256, 0, s>>>(offsets, bins, n_fft, n_peaks, g, cell,
-                                                           hist);
+        gross_hist_kernel<<<n_fft, kFftThreads, 0, s>>>(offsets, bins, n_peaks, g, edge, cell,
+                                                        hist);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return cuda_error(e, "gross histogram");
     return run_filter(offsets, bins, n_fft, n_peaks, KeepGross{cell, hist, threshold}, k0, t_fft,
-                      offsets_out, bins_out, freq_out, capacity, n_out, err, sc, s);
+                      offsets_out, bins_out, freq_out, capacity, n_out, res, nullptr, sc, s);
 }
 
 int fh_peakmap_persistency_veto(const int64_t *offsets, const int32_t *bins, int32_t n_fft,
@@ -893,41 +1003,38 @@ int fh_peakmap_persistency_veto(const int64_t *offsets, const int32_t *bins, int
         return set_error(FH_ERR_INVALID_ARG, "need n_bins >= 1, finite k_sigma, t_fft > 0");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     Scratch sc(s);
-    int32_t *err = nullptr, *hc = nullptr, *hd = nullptr;
-    double *d_stats = nullptr;
     // a bin's count is at most n_fft for a valid CSR; one more value catches the rest
     const int32_t vmax = n_fft + 1;
-    cudaError_t e = sc.get(&err, 1);
-    if (e == cudaSuccess) e = sc.get(&hc, (size_t)vmax + 1);
-    if (e == cudaSuccess) e = sc.get(&hd, 2 * ((size_t)vmax + 1) + 1);
-    if (e == cudaSuccess) e = sc.get(&d_stats, 3);
-    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 4, s);
+    const size_t nv = (size_t)vmax + 1, nd = 2 * nv + 1;
+    const bool small = nv + nd <= (size_t)kSmallValues && n_bins <= 65536;
+    Result *res = nullptr;
+    int32_t *hc = nullptr;
+    cudaError_t e = sc.get(&res, 1);
+    if (e == cudaSuccess && !small) e = sc.get(&hc, nv + nd);
+    if (e == cudaSuccess) e = cudaMemsetAsync(res, 0, sizeof(Result), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(hist, 0, sizeof(int32_t) * (size_t)n_bins, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(hc, 0, sizeof(int32_t) * ((size_t)vmax + 1), s);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(hd, 0, sizeof(int32_t) * (2 * ((size_t)vmax + 1) + 1), s);
+    if (e == cudaSuccess && !small)
+        e = cudaMemsetAsync(hc, 0, sizeof(int32_t) * (nv + nd), s);
     if (e == cudaSuccess) {
-        check_csr_kernel<<<(n_fft + 256) / 256, 256, 0, s>>>(offsets, n_fft, n_peaks, err);
+        const int64_t work = std::max(n_peaks, (int64_t)n_fft + 1);
+        const int grid = (int)std::min<int64_t>((work + 255) / 256, 8192);
+        bin_hist_kernel<<<grid, 256, 0, s>>>(offsets, bins, n_fft, n_peaks, n_bins, hist,
+                                             &res->err);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess && n_fft > 0) {
-        bin_hist_kernel<<<warp_grid(n_fft), 256, 0, s>>>(offsets, bins, n_fft, n_peaks, n_bins,
-                                                         hist, err);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) {
+    if (e == cudaSuccess && !small) {
         const int grid = (int)std::min<int64_t>(((int64_t)n_bins + 255) / 256, 4096);
-        count_hist_kernel<<<grid, 256, 0, s>>>(hist, n_bins, vmax, hc, err);
+        count_hist_kernel<<<grid, 256, 0, s>>>(hist, n_bins, vmax, hc, &res->err);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-        robust_stats_kernel<<<1, kScanThreads, 0, s>>>(hc, vmax, n_bins, hd, k_sigma, d_stats);
+        robust_stats_kernel<<<1, kScanThreads, small ? sizeof(int32_t) * (nv + nd) : 0, s>>>(
+            small ? hist : nullptr, hc, vmax, n_bins, hc ? hc + nv : nullptr, k_sigma, res);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(stats, d_stats, 24, cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return cuda_error(e, "persistency histogram");
-    return run_filter(offsets, bins, n_fft, n_peaks, KeepPersist{hist, d_stats, n_bins}, k0,
-                      t_fft, offsets_out, bins_out, freq_out, capacity, n_out, err, sc, s);
+    return run_filter(offsets, bins, n_fft, n_peaks, KeepPersist{hist, res, n_bins}, k0, t_fft,
+                      offsets_out, bins_out, freq_out, capacity, n_out, res, stats, sc, s);
 }
 
 }  // extern "C"

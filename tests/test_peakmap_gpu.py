@@ -270,3 +270,48 @@ def test_constant_lines_by_the_transform_without_doppler(fh, oracle_mod):
     for k in ("row", "cell", "count"):
         assert np.array_equal(cand[k][:2].astype(np.int64), o[k][0, 0, :2].astype(np.int64)), k
     assert list(cand["row"][:2]) == [1, 1]
+
+
+def _csr(counts, n_bins, seed):
+    """A peakmap with the given number of peaks per FFT."""
+    rng = np.random.RandomState(seed)
+    bins = [np.sort(rng.choice(n_bins, c, replace=False)) for c in counts]
+    o = np.zeros(len(counts) + 1, dtype=np.int64)
+    np.cumsum(counts, out=o[1:])
+    return o, np.concatenate(bins).astype(np.int32) if len(bins) else np.zeros(0, np.int32)
+
+
+# FFTs of 0, 1, 31 .. 129 and 1000 peaks (steps of 128, warps of 32); columns much
+# narrower than a bin, wider than the band, uneven against the bins, edges on bins
+# exactly (df a power of two), a grid below and above the band, k0 = 0, 2^40 bins
+@pytest.mark.parametrize("k0, t_fft, f0_h, df_h, n_fh", [
+    (409600, 8192.0, 50.0, 0.01, 12), (409600, 8192.0, 50.0, 1.0 / 8192, 2048),
+    (409600, 8192.0, 49.99, 1e-6, 40000), (409600, 8192.0, 50.0, 5.0, 3),
+    (0, 1024.0, 0.0, 0.25, 4), (90000, 1800.0, 50.0, 0.0123, 40),
+    (1 << 40, 8192.0, 134217728.0, 0.01, 9), (409600, 8192.0, 60.0, 0.01, 5),
+    (409600, 8192.0, 40.0, 0.01, 5)])
+def test_gross_columns_and_fft_sizes(fh, pm, k0, t_fft, f0_h, df_h, n_fh):
+    n_bins = 2048
+    o, b = _csr([0, 1, 31, 32, 33, 127, 128, 129, 1000, 0, 2048], n_bins, 5)
+    t = np.arange(len(o) - 1) * 0.5 * t_fft
+    grid = (0.0, 1.9 * t_fft, 5, f0_h, df_h, n_fh)
+    for thr in (0, 3, 40):
+        wo, wb, wh = pm.gross_veto(t, o, b, k0, t_fft, *grid, thr)
+        go, gb, gf, gh = fh.fh_peakmap_gross_veto(dev(t), dev(o), dev(b), k0, t_fft, *grid, thr)
+        assert np.array_equal(host(gh), wh)
+        assert np.array_equal(host(go), wo) and np.array_equal(host(gb), wb)
+        assert np.array_equal(host(gf).view(np.uint64),
+                              pm.peak_frequencies(wb, k0, t_fft).view(np.uint64))
+
+
+# the statistics in shared memory (up to 3997 FFTs and 65536 bins) and past it
+@pytest.mark.parametrize("n_fft, n_bins", [(3997, 40), (3998, 40), (9, 65536), (9, 65537), (1, 1),
+                                           (2, 2)])
+def test_persistency_in_and_out_of_shared_memory(fh, pm, n_fft, n_bins):
+    rng = np.random.RandomState(n_fft + n_bins)
+    o, b = _csr(rng.randint(0, min(n_bins, 30) + 1, n_fft), n_bins, 6)
+    for k in (0.0, 1.5):
+        wo, wb, wh, m1, m2, thr = pm.persistency_veto(o, b, n_bins, k)
+        go, gb, _, gh, st = fh.fh_peakmap_persistency_veto(dev(o), dev(b), n_bins, k, 0, 8192.0)
+        assert np.array_equal(host(gh), wh) and st == (m1, m2, thr)
+        assert np.array_equal(host(go), wo) and np.array_equal(host(gb), wb)
