@@ -25,6 +25,32 @@ constexpr uint32_t kWinLookup = 0xFFFFFFFFu;
 // error bits written by the device-side input checks
 enum : int32_t { kErrUnsorted = 1, kErrRange = 2, kErrInvalid = 4, kErrCsr = 8 };
 
+#ifdef __CUDACC__
+// floor(x 2^32) for |x| < 2^28, exactly: x = m 2^(e - 1075) with m the
+// significand (hidden bit included for normal numbers), so x 2^32 =
+// m 2^(e - 1043), a left shift by at most 7 bits, or a right shift whose
+// discarded bits round a negative value down.  Out-of-range inputs give some
+// value; the caller flags them.
+__device__ __forceinline__ int64_t floor_times_2p32(double x)
+{
+    const uint64_t bits = (uint64_t)__double_as_longlong(x);
+    const int ex = (int)((bits >> 52) & 0x7FF);
+    const uint64_t m = (bits & 0xFFFFFFFFFFFFFull) | (ex ? (uint64_t(1) << 52) : 0);
+    const int sh = (ex ? ex : 1) - 1043;
+    uint64_t q;
+    bool frac;
+    if (sh >= 0) {
+        q = m << (sh < 10 ? sh : 10);
+        frac = false;
+    } else {
+        const int rs = -sh;
+        q = rs < 64 ? m >> rs : 0;
+        frac = rs < 64 ? (m & ((uint64_t(1) << rs) - 1)) != 0 : m != 0;
+    }
+    return (bits >> 63) ? -(int64_t)q - (frac ? 1 : 0) : (int64_t)q;
+}
+#endif
+
 // One direction set of one plan, as the transform kernel sees it.
 struct TransformJob {
     const int64_t *A;        // positions, [dir][n_peaks] (absolute directions)
@@ -114,16 +140,6 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm, const dou
                 bool host_checks, cudaStream_t s);
 // the error of a device error word (0: FH_OK)
 int device_error_code(int32_t bits);
-// positions of n_batch peakmaps (refinement): batch c has offsets
-// offsets + c (n_fft + 1), source index src + c n_fft, sky + 3 c n_dir, its peak
-// count n_peaks[c] (device) and its positions at A + a_base[c] (device),
-// direction-major ([direction][peak] within each batch)
-cudaError_t launch_positions_batched(const double *freq, const int64_t *offsets,
-                                     const double *v, const double *sky, int32_t n_fft,
-                                     int32_t n_dir, int32_t n_batch, const int64_t *a_base,
-                                     const int64_t *n_peaks, double f0_min, double kt,
-                                     int32_t k_over, int64_t *A, int32_t *err, bool validate,
-                                     const int64_t *src, cudaStream_t s);
 cudaError_t launch_validate_device_inputs(const double *t, const double *freq,
                                           const int64_t *offsets, const double *v,
                                           const double *sky, int32_t n_fft, int32_t n_dir,

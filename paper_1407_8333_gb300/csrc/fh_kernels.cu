@@ -5,8 +5,6 @@
 //                                 and 32.32 fixed-point stripe start (Eq. fdopp;
 //                                 Sec. VI; Eq. freqres) of every direction
 //   prep_kernel          a3       the shift tables, CSR sanitising and checks alone
-//   positions_kernel     a1 + a2  the positions alone, also of several peakmaps
-//                                 (refined-grid search)
 //   windows_kernel       a4       which peaks can reach each tile; clears the profile
 //   transform_kernel     a4 + a5 + profile half of a6 (Eqs. due, ncount; Sec. VIII)
 //   select_kernel        a6       per-sub-band greedy picks (Sec. VIII; Eq. cr)
@@ -32,40 +30,10 @@ constexpr int kPosFfts = 8;
 constexpr int kPosThreads = 256;
 
 // ---------------------------------------------------------------- a1 + a2
-// several peakmaps in one launch (see positions_kernel); null a_base: one
-struct PosBatch {
-    const int64_t *a_base, *n_peaks;
-};
-
-// floor(x 2^32) for |x| < 2^28, exactly: x = m 2^(e - 1075) with m the
-// significand (hidden bit included for normal numbers), so x 2^32 =
-// m 2^(e - 1043), a left shift by at most 7 bits, or a right shift whose
-// discarded bits round a negative value down.  Out-of-range inputs give some
-// value; the caller flags them.
-__device__ __forceinline__ int64_t floor_times_2p32(double x)
-{
-    const uint64_t bits = (uint64_t)__double_as_longlong(x);
-    const int ex = (int)((bits >> 52) & 0x7FF);
-    const uint64_t m = (bits & 0xFFFFFFFFFFFFFull) | (ex ? (uint64_t(1) << 52) : 0);
-    const int sh = (ex ? ex : 1) - 1043;
-    uint64_t q;
-    bool frac;
-    if (sh >= 0) {
-        q = m << (sh < 10 ? sh : 10);
-        frac = false;
-    } else {
-        const int rs = -sh;
-        q = rs < 64 ? m >> rs : 0;
-        frac = rs < 64 ? (m & ((uint64_t(1) << rs) - 1)) != 0 : m != 0;
-    }
-    return (bits >> 63) ? -(int64_t)q - (frac ? 1 : 0) : (int64_t)q;
-}
-
 // grid (ceil(n_fft / 8), n_dir): the block computes r = 1 / (1 + v.n) for 8
 // FFTs of one direction, then the fixed-point position of each of their peaks
-// (a contiguous CSR range, so loads and stores are coalesced).  With `src`,
-// FFT i's peaks are read from freq[src[i] ...] (a sub-range of a larger
-// peakmap) and written compactly by `offsets`.  With `validate`, the blocks of
+// (a contiguous CSR range, so loads and stores are coalesced).  With `validate`,
+// the blocks of
 // direction 0 also flag frequencies that are not finite and positive
 // (kErrInvalid) or not strictly increasing within their FFT (kErrUnsorted).
 // The body of one positions block: group `group` of 8 FFTs, direction d.
@@ -77,11 +45,10 @@ __device__ __forceinline__ void positions_block(
     const double *__restrict__ freq, const int64_t *__restrict__ offsets, bool clamp_offsets,
     const double *__restrict__ v, const double *__restrict__ sky, int32_t n_fft, int64_t n_peaks,
     double f0_min, double kt, double cshift, int64_t *__restrict__ A, double *__restrict__ out_r,
-    int32_t *err, int32_t validate, const int64_t *__restrict__ src, int d, int group)
+    int32_t *err, int32_t validate, int d, int group)
 {
     __shared__ double r_s[kPosFfts];
     __shared__ int64_t off_s[kPosFfts + 1];
-    __shared__ int64_t src_s[kPosFfts];  // where each FFT's peaks start in freq
     const int i0 = group * kPosFfts;
     const int nf = min(kPosFfts, n_fft - i0);
     if (threadIdx.x < nf) {
@@ -100,15 +67,11 @@ __device__ __forceinline__ void positions_block(
         if (clamp_offsets) o = o < 0 ? 0 : (o > n_peaks ? n_peaks : o);
         off_s[threadIdx.x] = o;
     }
-    if (!clamp_offsets && threadIdx.x < nf)
-        src_s[threadIdx.x] = src ? src[i0 + threadIdx.x] : offsets[i0 + threadIdx.x];
     __syncthreads();
     if (clamp_offsets) {
         if (threadIdx.x == 0)
-            for (int k = 0; k <= nf; ++k) {
-                if (k > 0 && off_s[k] < off_s[k - 1]) off_s[k] = off_s[k - 1];
-                if (k < nf) src_s[k] = off_s[k];
-            }
+            for (int k = 1; k <= nf; ++k)
+                if (off_s[k] < off_s[k - 1]) off_s[k] = off_s[k - 1];
         __syncthreads();
     }
     const int64_t p_begin = off_s[0], p_end = off_s[nf];
@@ -126,13 +89,12 @@ __device__ __forceinline__ void positions_block(
             const int m = (lo + hi) >> 1;
             if (off_s[m] <= p) lo = m; else hi = m;
         }
-        const int64_t fp = src_s[lo] + (p - off_s[lo]);
-        const double f = in ? freq[fp] : 1.0;
+        const double f = in ? freq[p] : 1.0;
         if (check) {
             // positive finite doubles order like their bit patterns
             const int64_t fb = __double_as_longlong(f);
             int64_t prev = __shfl_up_sync(kFull, fb, 1);
-            if (lane == 0 && in && p > off_s[lo]) prev = __double_as_longlong(freq[fp - 1]);
+            if (lane == 0 && in && p > off_s[lo]) prev = __double_as_longlong(freq[p - 1]);
             if (in) {
                 if (!(fb > 0 && fb < 0x7FF0000000000000LL)) ev |= kErrInvalid;
                 if (p > off_s[lo] && !(fb > prev)) ev |= kErrUnsorted;
@@ -150,27 +112,6 @@ __device__ __forceinline__ void positions_block(
     }
     if (ev) atomicOr(err, ev);
     if (bad) atomicOr(err, kErrRange);
-}
-
-__global__ void __launch_bounds__(kPosThreads)
-positions_kernel(const double *__restrict__ freq, const int64_t *__restrict__ offsets,
-                 const double *__restrict__ v, const double *__restrict__ sky, int32_t n_fft,
-                 int64_t n_peaks, double f0_min, double kt, double cshift,
-                 int64_t *__restrict__ A, double *__restrict__ out_r, int32_t *err,
-                 int32_t validate, const int64_t *__restrict__ src, PosBatch batch)
-{
-    // batches (refinement): block z is one peakmap of several, each with its own
-    // offsets, source index, sky directions, output base and peak count
-    if (batch.a_base) {
-        const int c = blockIdx.z;
-        offsets += (int64_t)c * (n_fft + 1);
-        src += (int64_t)c * n_fft;
-        sky += 3 * (int64_t)c * gridDim.y;
-        A += batch.a_base[c];
-        n_peaks = batch.n_peaks[c];
-    }
-    positions_block(freq, offsets, false, v, sky, n_fft, n_peaks, f0_min, kt, cshift, A, out_r,
-                    err, validate, src, blockIdx.y, blockIdx.x);
 }
 
 // ---------------------------------------------------------------- a3 + per-call set-up
@@ -327,7 +268,7 @@ correct_kernel(const PrepArgs a, const double *__restrict__ freq, double f0_min,
     }
     const bool raw = a.offsets_in != nullptr;
     positions_block(freq, raw ? a.offsets_in : a.offsets_out, raw, a.v, a.sky, a.n_fft, a.n_peaks,
-                    f0_min, a.kt, cshift, A, out_r, a.err, a.validate, nullptr, d, group);
+                    f0_min, a.kt, cshift, A, out_r, a.err, a.validate, d, group);
 }
 
 
@@ -1965,28 +1906,6 @@ cudaError_t launch_correct(const PrepArgs &a, const double *freq, double f0_min,
     dim3 grid(1 + groups, std::max(1, a.n_dir));
     correct_kernel<<<grid, kPosThreads, 0, s>>>(a, freq, f0_min, cshift, A, out_r);
     return cudaGetLastError();
-}
-
-cudaError_t launch_positions_batched(const double *freq, const int64_t *offsets,
-                                     const double *v, const double *sky, int32_t n_fft,
-                                     int32_t n_dir, int32_t n_batch, const int64_t *a_base,
-                                     const int64_t *n_peaks, double f0_min, double kt,
-                                     int32_t k_over, int64_t *A, int32_t *err, bool validate,
-                                     const int64_t *src, cudaStream_t s)
-{
-    if (n_fft <= 0 || n_dir <= 0 || n_batch <= 0) return cudaSuccess;
-    const double cshift = 0.5 - 0.5 * (double)k_over;
-    for (int32_t b0 = 0; b0 < n_batch; b0 += 65535) {
-        const int32_t nb = std::min(65535, n_batch - b0);
-        dim3 grid((n_fft + kPosFfts - 1) / kPosFfts, n_dir, nb);
-        positions_kernel<<<grid, kPosThreads, 0, s>>>(
-            freq, offsets + (int64_t)b0 * (n_fft + 1), v, sky + 3 * (int64_t)b0 * n_dir, n_fft,
-            0, f0_min, kt, cshift, A, nullptr, err, validate ? 1 : 0, src + (int64_t)b0 * n_fft,
-            PosBatch{a_base + b0, n_peaks + b0});
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
 }
 
 cudaError_t launch_validate_device_inputs(const double *t, const double *freq,

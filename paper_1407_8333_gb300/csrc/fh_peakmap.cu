@@ -643,7 +643,7 @@ __device__ void kth_of_hist(const int32_t *h, int64_t nv, int64_t ka, int64_t kb
 // median(|x - m1|) / 0.6745, thr = m1 + k m2.  The deviations are half-integers;
 // hd (2 vmax + 1 entries, zeroed) receives their doubled values.  One block.
 // With `counts` the block forms hc itself, and both histograms live in shared
-// memory (bands and FFT counts small enough: 8192 bins and 3164 FFTs take 10 us
+// memory (bands and FFT counts small enough: 8192 bins and 3164 FFTs take 12 us
 // against 14 us for the two kernels on global memory).
 constexpr int kSmallValues = 12000;  // words of shared memory for hc and hd
 __global__ void __launch_bounds__(kScanThreads)

@@ -11,13 +11,23 @@
 // over all refined directions, rows and cells (ties: smallest direction, then
 // row, then cell).
 //
-// Per call: the coarse and refined shift tables (prep kernels); per
-// (candidate, FFT) the contiguous range of peaks that can reach the refined
-// band (a conservative frequency window, binary search); compact per-candidate
-// position arrays for those peaks only; peak windows and one batched transform
-// launch per group of candidates; a pick kernel per candidate.
+// Per call: the coarse shift tables (prep kernel) and, with device-side checks, the
+// frequencies' order; then one kernel over (candidate, share of the FFTs): per FFT the
+// contiguous range of peaks that can reach the refined band (a conservative
+// frequency window, two binary searches), and per (peak of a range, refined
+// direction) the position, exactly as the coarse correction forms it, and its
+// stripe start on every refined row, counted in a histogram of starts in shared
+// memory; last a kernel that sums the starts over K cells and picks.  A candidate's
+// ranges hold a few tenths of a peak per FFT, so what is left of the work is the
+// ranges themselves; positions are formed in lists of (peak, direction), a lane
+// each, because a lane per FFT would leave three quarters of a warp idle.
+// (The general transform on compacted peakmaps, which this replaces, needed a
+// host round trip for the compaction, 178,200 blocks of positions and a launch per
+// 12 candidates: 50 candidates x 9 directions on 3164 FFTs took
+// 460 us of kernels and as much again on the host.)
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "fh_internal.h"
@@ -28,16 +38,21 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-struct RangeArgs {
+struct RefineArgs {
     const double *t, *freq, *v, *sky;  // sky: [cand][n_ref][3]
-    const int64_t *offsets, *S0, *D, *Dr;
+    const int64_t *offsets, *S0, *D;   // sanitised CSR; coarse shift tables
     const int32_t *cell, *row;
-    int32_t n_fft, n_cand, k_over, n_rows, n_ref;
-    double f0_min, kt;
-    int64_t *start;   // [cand][fft]: first peak of the range
-    int32_t *count;   // [cand][fft]: peaks in the range
-    int64_t *S0r;     // [cand][fft]: refined row-0 shift, cell offset included
+    int32_t n_fft, k_over, n_rows, n_ref;
+    int32_t cand0, dir0, n_dir;        // the launch's first candidate and directions
+    int32_t dirs_per, rows_per;        // directions and rows of one block's histogram
+    int32_t ffts_per;                  // FFTs of one block
+    double f0_min, kt, t_ref, step_ref, cshift;
+    int32_t *starts;  // [cand][direction][row][3 K] of the launch: stripe starts, zeroed
+    int32_t *err;
 };
+
+constexpr int kRefThreads = 256;
+constexpr int kRefList = 64;  // (FFT, peak) entries a warp collects before it places them
 
 // Refined band of candidate c in refined cells [0, 2K + 1): a stripe starting at
 // s touches it iff s in [1 - K, 2K].  With the refined shifts X_j = S0r + j D'
@@ -46,97 +61,215 @@ struct RangeArgs {
 // is about ((f r - f0_min) KT + 0.5 - 0.5 K) 2^32 with r = 1 / (1 + v.n), so
 // the frequencies f = u (1 + v.n) of the peaks that can take part lie between
 // the extremes of that product over u in [u_lo, u_hi] and v.n between its
-// least and largest value over the candidate's refined directions (a bilinear
-// form: the extremes are at the corners).  The margin of a cell is far above
-// the rounding of these products; the transform decides exactly.
-__global__ void refine_ranges_kernel(const RangeArgs a)
+// least and largest value over the block's refined directions (a bilinear
+// form: the extremes are at the corners).  v.n is formed in binary32 and widened by
+// a bound of its error; the margin of a cell is far above the other roundings.
+// The exact position of each peak of the range then decides.
+//
+// grid (candidates, shares of ffts_per FFTs, (direction, row) groups of one
+// histogram).  A warp takes 32 FFTs at a time (lane <-> FFT), lists their peaks, and
+// places list x directions, a lane each.
+__global__ void __launch_bounds__(kRefThreads) refine_kernel(const RefineArgs a)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int c = blockIdx.y;
-    if (i >= a.n_fft) return;
-    const int K = a.k_over;
+    extern __shared__ int32_t hist[];  // [direction][row][3 K]
+    __shared__ int32_t list_fft[kRefThreads / 32][kRefList];
+    __shared__ int64_t list_peak[kRefThreads / 32][kRefList];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = a.cand0 + blockIdx.x;
+    const int row_groups = (a.n_rows + a.rows_per - 1) / a.rows_per;
+    const int d0 = (int)(blockIdx.z / row_groups) * a.dirs_per;
+    const int r0 = (int)(blockIdx.z % row_groups) * a.rows_per;
+    const int nd = min(a.dirs_per, a.n_dir - d0), nr = min(a.rows_per, a.n_rows - r0);
+    const int K = a.k_over, E = 3 * K;
+    const int words = nd * nr * E;
+    for (int w = threadIdx.x; w < words; w += kRefThreads) hist[w] = 0;
+    __syncthreads();
     const int64_t lo_cell = (int64_t)a.cell[c] - K;
-    const int64_t s0r = a.S0[i] + (int64_t)(a.row[c] - 2) * a.D[i] + lo_cell * 4294967296LL;
-    a.S0r[(int64_t)c * a.n_fft + i] = s0r;
-    const int64_t last = (int64_t)(a.n_rows - 1) * a.Dr[i];
-    const double xmin = ((double)s0r + (double)(last < 0 ? last : 0)) / 4294967296.0;
-    const double xmax = ((double)s0r + (double)(last > 0 ? last : 0)) / 4294967296.0;
-    const double c_off = 0.5 - 0.5 * (double)K;
-    const double u_lo = a.f0_min + (xmin + (double)(1 - K) - 1.0 - c_off) / a.kt;
-    const double u_hi = a.f0_min + (xmax + (double)(2 * K + 1) + 1.0 - c_off) / a.kt;
-    const double vx = a.v[3 * (int64_t)i], vy = a.v[3 * (int64_t)i + 1],
-                 vz = a.v[3 * (int64_t)i + 2];
-    double vn_lo = 0.0, vn_hi = 0.0;
-    const double *n = a.sky + 3 * (int64_t)c * a.n_ref;
-    for (int d = 0; d < a.n_ref; ++d, n += 3) {
-        const double vn = vx * n[0] + vy * n[1] + vz * n[2];
-        vn_lo = d ? fmin(vn_lo, vn) : vn;
-        vn_hi = d ? fmax(vn_hi, vn) : vn;
+    const int64_t j_off = (int64_t)a.row[c] - 2;
+    const double *sky = a.sky + 3 * ((int64_t)c * a.n_ref + a.dir0);
+    int32_t ev = 0;
+    const int f_begin = blockIdx.y * a.ffts_per;
+    const int f_end = min(a.n_fft, f_begin + a.ffts_per);
+
+    // the listed peaks in every direction of the group, a lane each
+    auto place = [&](int n) {
+        __syncwarp();
+        for (int q = lane; q < n * nd; q += 32) {
+            const int e = q / nd, d = q - e * nd;
+            const int i = list_fft[warp][e];
+            const double *n3 = sky + 3 * (d0 + d);
+            const double px = __dmul_rn(a.v[3 * (int64_t)i + 0], n3[0]);
+            const double py = __dmul_rn(a.v[3 * (int64_t)i + 1], n3[1]);
+            const double pz = __dmul_rn(a.v[3 * (int64_t)i + 2], n3[2]);
+            const double den = __dadd_rn(1.0, __dadd_rn(__dadd_rn(px, py), pz));
+            const double u = __dmul_rn(a.freq[list_peak[warp][e]], __ddiv_rn(1.0, den));
+            const double y = __dmul_rn(__dsub_rn(u, a.f0_min), a.kt);
+            const double x = __dadd_rn(y, a.cshift);
+            // |x| < 2^28 exactly when the biased exponent is below 1023 + 28
+            if (((__double_as_longlong(x) >> 52) & 0x7FF) >= 1051) ev |= kErrRange;
+            const double cc = __dmul_rn(__dsub_rn(a.t[i], a.t_ref), a.kt);
+            const int64_t dr = (int64_t)floor(__dmul_rn(__dmul_rn(a.step_ref, cc), 4294967296.0));
+            // start of the stripe on row r0, its cell 0 at start 1 - K
+            int64_t X = floor_times_2p32(x) - (a.S0[i] + j_off * a.D[i]) -
+                        (int64_t)r0 * dr + ((int64_t)(K - 1) - lo_cell) * 4294967296LL;
+            int32_t *h = hist + d * nr * E;
+            for (int r = 0; r < nr; ++r, X -= dr, h += E) {
+                const int32_t L = (int32_t)(X >> 32);
+                if ((uint32_t)L < (uint32_t)E) atomicAdd(h + L, 1);
+            }
+        }
+        __syncwarp();
+    };
+
+    const double absmax = fabs(__dmul_rn((double)(a.n_rows - 1), a.step_ref));
+    int listed = 0;
+    for (int base = f_begin + 32 * warp; base < f_end; base += kRefThreads) {
+        const int i = base + lane;
+        int64_t p = 0, p_end = 0;
+        if (i < f_end) {
+            // the refined drift and its range check, as the shift tables form them
+            const double cc = __dmul_rn(__dsub_rn(a.t[i], a.t_ref), a.kt);
+            if (!(fabs(cc) * absmax < (double)kFixedLimit)) ev |= kErrRange;
+            const int64_t dr = (int64_t)floor(__dmul_rn(__dmul_rn(a.step_ref, cc), 4294967296.0));
+            const int64_t s0r = a.S0[i] + j_off * a.D[i] + lo_cell * 4294967296LL;
+            const int64_t last = (int64_t)(a.n_rows - 1) * dr;
+            const double xmin = ((double)s0r + (double)(last < 0 ? last : 0)) / 4294967296.0;
+            const double xmax = ((double)s0r + (double)(last > 0 ? last : 0)) / 4294967296.0;
+            const double c_off = 0.5 - 0.5 * (double)K;
+            const double u_lo = a.f0_min + (xmin + (double)(1 - K) - 1.0 - c_off) / a.kt;
+            const double u_hi = a.f0_min + (xmax + (double)(2 * K + 1) + 1.0 - c_off) / a.kt;
+            const float vx = (float)a.v[3 * (int64_t)i], vy = (float)a.v[3 * (int64_t)i + 1],
+                        vz = (float)a.v[3 * (int64_t)i + 2];
+            float lo32 = 0.f, hi32 = 0.f;
+            const double *n = sky + 3 * d0;
+            for (int d = 0; d < nd; ++d, n += 3) {
+                const float vn = vx * (float)n[0] + vy * (float)n[1] + vz * (float)n[2];
+                lo32 = d ? fminf(lo32, vn) : vn;
+                hi32 = d ? fmaxf(hi32, vn) : vn;
+            }
+            // the sum of three products of rounded factors is off by less than
+            // 4 x 2^-23 of the sum of their magnitudes (|n| <= 1.000001)
+            const float wide = 5e-7f * (fabsf(vx) + fabsf(vy) + fabsf(vz)) + 1e-37f;
+            const double vn_lo = (double)(lo32 - wide), vn_hi = (double)(hi32 + wide);
+            const double f_lo = fmin(fmin(u_lo * (1.0 + vn_lo), u_lo * (1.0 + vn_hi)),
+                                     fmin(u_hi * (1.0 + vn_lo), u_hi * (1.0 + vn_hi)));
+            const double f_hi = fmax(fmax(u_lo * (1.0 + vn_lo), u_lo * (1.0 + vn_hi)),
+                                     fmax(u_hi * (1.0 + vn_lo), u_hi * (1.0 + vn_hi)));
+            p = a.offsets[i];
+            p_end = a.offsets[i + 1];
+            int64_t b = p_end;
+            while (p < b) {  // first peak with f >= f_lo
+                const int64_t m = (p + b) >> 1;
+                if (a.freq[m] < f_lo) p = m + 1; else b = m;
+            }
+            int64_t e = p;
+            b = p_end;
+            while (e < b) {  // first peak with f > f_hi
+                const int64_t m = (e + b) >> 1;
+                if (a.freq[m] <= f_hi) e = m + 1; else b = m;
+            }
+            p_end = e;
+        }
+        // every lane lists one peak per turn
+        for (;;) {
+            const unsigned have = __ballot_sync(kFull, p < p_end);
+            if (!have) break;
+            if (listed + 32 > kRefList) {
+                place(listed);
+                listed = 0;
+            }
+            if (p < p_end) {
+                const int k = listed + __popc(have & ((1u << lane) - 1u));
+                list_fft[warp][k] = i;
+                list_peak[warp][k] = p;
+                ++p;
+            }
+            listed += __popc(have);
+        }
     }
-    const double f_lo = fmin(fmin(u_lo * (1.0 + vn_lo), u_lo * (1.0 + vn_hi)),
-                             fmin(u_hi * (1.0 + vn_lo), u_hi * (1.0 + vn_hi)));
-    const double f_hi = fmax(fmax(u_lo * (1.0 + vn_lo), u_lo * (1.0 + vn_hi)),
-                             fmax(u_hi * (1.0 + vn_lo), u_hi * (1.0 + vn_hi)));
-    int64_t lo = a.offsets[i], hi = a.offsets[i + 1];
-    int64_t b = hi;
-    while (lo < b) {  // first peak with f >= f_lo
-        const int64_t m = (lo + b) >> 1;
-        if (a.freq[m] < f_lo) lo = m + 1; else b = m;
+    place(listed);
+    ev = (int32_t)__reduce_or_sync(kFull, (unsigned)ev);
+    if (lane == 0 && ev) atomicOr(a.err, ev);
+    __syncthreads();
+    // into the candidate's starts (other shares of the FFTs add theirs)
+    for (int w = threadIdx.x; w < words; w += kRefThreads) {
+        const int n = hist[w];
+        if (n) {
+            const int d = w / (nr * E), rest = w - d * nr * E;
+            atomicAdd(a.starts +
+                          (((int64_t)blockIdx.x * a.n_dir + d0 + d) * a.n_rows + r0) * E + rest,
+                      n);
+        }
     }
-    int64_t e = lo;
-    b = hi;
-    while (e < b) {  // first peak with f > f_hi
-        const int64_t m = (e + b) >> 1;
-        if (a.freq[m] <= f_hi) e = m + 1; else b = m;
-    }
-    a.start[(int64_t)c * a.n_fft + i] = lo;
-    a.count[(int64_t)c * a.n_fft + i] = (int32_t)(e - lo);
 }
 
 struct PickArgs {
-    const uint64_t *const *prof;  // [cand] -> [n_ref][n_f0r] profile keys
+    const int32_t *starts;        // [cand][direction][row][3 K]
     const int32_t *cell, *row;
-    int32_t n_cand, n_ref, n_f0r, k_over, n_fft;
+    int32_t n_rows, k_over, n_fft;
+    int32_t cand0, dir0, n_dir;   // the launch's first candidate and directions
+    int32_t *best;                // nullable: [cand] count, (direction, row), cell so far
+    int32_t last;                 // no further directions: write the candidate
     double f0_min, kt, fdot_min, fdot_step, fdot_step_ref, p0;
     fh_candidate *out;
 };
 
-// one warp per candidate: the best (count desc, direction asc, row asc, cell asc)
-// over the candidate's refined profile
-__global__ void refine_pick_kernel(const PickArgs a)
+// One block per candidate: the best (count desc, direction asc, row asc, cell asc)
+// of its refined maps.  A thread takes a (direction, row) at a time and slides a
+// K-cell window of starts along its 2K + 1 cells (cell b counts the starts at
+// b .. b + K - 1); later pairs and cells replace only by a larger count.
+constexpr int kPickThreads = 256;
+__global__ void __launch_bounds__(kPickThreads) refine_pick_kernel(const PickArgs a)
 {
-    const int c = blockIdx.x;
-    const int lane = threadIdx.x;
-    const uint64_t *pr = a.prof[c];
-    int bc = -1, bd = 0x7fffffff, bj = 0x7fffffff, bb = 0x7fffffff;
-    const int n = a.n_ref * a.n_f0r;
-    for (int k = lane; k < n; k += 32) {
-        const uint64_t key = pr[k];
-        const int cnt = (int)(uint32_t)(key >> 32);
-        const int j = (int)(0xFFFFFFFFu - (uint32_t)key);
-        const int d = k / a.n_f0r, b = k - d * a.n_f0r;
-        const bool better = cnt > bc || (cnt == bc && (d < bd || (d == bd && (j < bj ||
-                                                                   (j == bj && b < bb)))));
-        if (key != 0 && better) {
-            bc = cnt;
-            bd = d;
-            bj = j;
-            bb = b;
+    __shared__ int32_t best_s[kPickThreads / 32][3];  // count, (direction, row), cell
+    const int c = a.cand0 + blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int K = a.k_over, E = 3 * K, n = a.n_dir * a.n_rows;
+    const int32_t *st = a.starts + (int64_t)blockIdx.x * n * E;
+    int bc = -1, bq = 0x7fffffff, bb = 0x7fffffff;
+    for (int q = threadIdx.x; q < n; q += kPickThreads) {
+        const int32_t *h = st + (int64_t)q * E;
+        int cnt = 0;
+        for (int L = 0; L < K; ++L) cnt += h[L];
+        for (int b = 0;; ++b) {
+            if (cnt > bc) {
+                bc = cnt;
+                bq = a.dir0 * a.n_rows + q;
+                bb = b;
+            }
+            if (b == 2 * K) break;
+            cnt += h[b + K] - h[b];
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        const int c2 = __shfl_down_sync(kFull, bc, o), d2 = __shfl_down_sync(kFull, bd, o);
-        const int j2 = __shfl_down_sync(kFull, bj, o), b2 = __shfl_down_sync(kFull, bb, o);
-        const bool better = c2 > bc || (c2 == bc && (d2 < bd || (d2 == bd && (j2 < bj ||
-                                                                  (j2 == bj && b2 < bb)))));
-        if (better) {
+    auto take = [&](int c2, int q2, int b2) {
+        if (c2 > bc || (c2 == bc && (q2 < bq || (q2 == bq && b2 < bb)))) {
             bc = c2;
-            bd = d2;
-            bj = j2;
+            bq = q2;
             bb = b2;
         }
+    };
+    for (int o = 16; o > 0; o >>= 1) {
+        const int c2 = __shfl_down_sync(kFull, bc, o), q2 = __shfl_down_sync(kFull, bq, o),
+                  b2 = __shfl_down_sync(kFull, bb, o);
+        take(c2, q2, b2);
     }
-    if (lane != 0) return;
+    if (lane == 0) {
+        best_s[warp][0] = bc;
+        best_s[warp][1] = bq;
+        best_s[warp][2] = bb;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < kPickThreads / 32; ++w) take(best_s[w][0], best_s[w][1], best_s[w][2]);
+    if (a.best) {
+        int32_t *m = a.best + 3 * (int64_t)c;
+        if (a.dir0 > 0) take(m[0], m[1], m[2]);
+        m[0] = bc;
+        m[1] = bq;
+        m[2] = bb;
+    }
+    if (!a.last) return;
+    const int bd = bq / a.n_rows, bj = bq - bd * a.n_rows;
     fh_candidate r;
     r.subband = c;
     r.rank = 0;
@@ -173,7 +306,6 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
     const int32_t n = pm->n_fft;
     const int64_t np = pm->n_peaks;
     const int K = d.k_over;
-    const int32_t n_f0r = 2 * K + 1;
     const int32_t n_rows = 4 * k_fdot;
     const double step_ref = d.fdot_step / (double)k_fdot;
     // the inputs are checked on the host, or (FH_CHECKS_DEVICE) by the kernels
@@ -189,10 +321,8 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
 
     Scratch sc(s);
     double *t = nullptr, *freq = nullptr, *v = nullptr, *sky = nullptr;
-    int64_t *off = nullptr, *S0 = nullptr, *D = nullptr, *S0x = nullptr, *Dr = nullptr;
-    int64_t *start = nullptr, *S0r = nullptr;
-    int32_t *count = nullptr, *cc = nullptr, *cr = nullptr, *err = nullptr;
-    unsigned long long *dmax = nullptr;
+    int64_t *off = nullptr, *S0 = nullptr, *D = nullptr;
+    int32_t *cc = nullptr, *cr = nullptr;
     cudaError_t e = cudaSuccess;
     e = sc.get(&t, (size_t)n);
     if (e == cudaSuccess) e = sc.get(&freq, (size_t)np);
@@ -203,16 +333,36 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
     if (e == cudaSuccess && !host_checks) e = sc.get(&off_raw, (size_t)n + 1);
     if (e == cudaSuccess) e = sc.get(&S0, (size_t)n);
     if (e == cudaSuccess) e = sc.get(&D, (size_t)n);
-    if (e == cudaSuccess) e = sc.get(&S0x, (size_t)n);
-    if (e == cudaSuccess) e = sc.get(&Dr, (size_t)n);
-    if (e == cudaSuccess) e = sc.get(&start, (size_t)n_cand * n);
-    if (e == cudaSuccess) e = sc.get(&S0r, (size_t)n_cand * n);
-    if (e == cudaSuccess) e = sc.get(&count, (size_t)n_cand * n);
     if (e == cudaSuccess) e = sc.get(&cc, (size_t)n_cand);
     if (e == cudaSuccess) e = sc.get(&cr, (size_t)n_cand);
-    if (e == cudaSuccess) e = sc.get(&err, 4);
-    if (e == cudaSuccess) e = sc.get(&dmax, 2);
+    // A block's histogram of starts in shared memory: all directions and rows where
+    // they fit in 40 KB, else groups of directions, else of rows.  In memory, the
+    // starts of as many candidates and directions at a time as 1 GiB holds (and as
+    // give a grid at most 65535 groups).
+    const int32_t E = 3 * K;
+    const int64_t per_dir = (int64_t)n_rows * E, most = (int64_t)1 << 28, room = 40 * 1024 / 4;
+    RefineArgs ra{};
+    ra.rows_per = (int32_t)std::max<int64_t>(1, std::min<int64_t>(n_rows, room / E));
+    const int64_t row_groups = (n_rows + ra.rows_per - 1) / ra.rows_per;
+    const int32_t dir_batch = (int32_t)std::max<int64_t>(
+        1, std::min<int64_t>({n_ref, most / per_dir, 65535 / row_groups}));
+    ra.dirs_per = (int32_t)std::max<int64_t>(
+        1, std::min<int64_t>(dir_batch, room / ((int64_t)ra.rows_per * E)));
+    const int32_t cand_batch = (int32_t)std::max<int64_t>(
+        1, std::min<int64_t>(n_cand, most / (per_dir * dir_batch)));
+    const size_t n_starts = (size_t)cand_batch * dir_batch * per_dir;
+    // what is read back (the candidates, then the error word) and what starts at zero
+    // beside it (largest |D|, stripe starts), in one block
+    const size_t out_bytes = sizeof(fh_candidate) * (size_t)n_cand;
+    char *zero = nullptr;
+    int32_t *best = nullptr;
+    if (e == cudaSuccess) e = sc.get(&zero, out_bytes + 64 + 4 * n_starts);
+    if (e == cudaSuccess && dir_batch < n_ref) e = sc.get(&best, 3 * (size_t)n_cand);
     if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync (refinement)");
+    fh_candidate *d_out = reinterpret_cast<fh_candidate *>(zero);
+    int32_t *err = reinterpret_cast<int32_t *>(zero + out_bytes);
+    unsigned long long *dmax = reinterpret_cast<unsigned long long *>(zero + out_bytes + 16);
+    int32_t *starts = reinterpret_cast<int32_t *>(zero + out_bytes + 64);
     struct {
         void *dst;
         const void *src;
@@ -227,9 +377,8 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
     for (auto &x : cp)
         if (x.bytes && e == cudaSuccess)
             e = cudaMemcpyAsync(x.dst, x.src, x.bytes, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 4, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dmax, 0, 16, s);
-    // coarse shift tables, then the refined step D' (and its largest |D'|)
+    if (e == cudaSuccess) e = cudaMemsetAsync(zero, 0, out_bytes + 64 + 4 * n_starts, s);
+    // coarse shift tables
     PrepArgs pa{};
     pa.offsets_in = host_checks ? nullptr : off_raw;  // sanitised into off by the checks
     pa.offsets_out = off;
@@ -247,173 +396,61 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
     pa.fdot_step = d.fdot_step;
     pa.S0 = S0;
     pa.D = D;
-    pa.dmax = dmax + 1;  // the coarse drift is not needed
+    pa.dmax = dmax;  // (not needed here)
     pa.err = err;
     if (e == cudaSuccess) e = launch_prep(pa, s);
     // device checks: every peak's frequency too (the positions below cover only
     // the peaks near each candidate, and the range searches need sorted FFTs)
     if (e == cudaSuccess && !host_checks)
         e = launch_validate_device_inputs(t, freq, off, v, sky, n, n_cand * n_ref, err, s);
-    PrepArgs pr = pa;
-    pr.offsets_in = nullptr;  // sanitised and checked by the first launch
-    pr.validate = 0;
-    pr.n_fdot = n_rows;
-    pr.fdot_min = 0.0;
-    pr.fdot_step = step_ref;
-    pr.S0 = S0x;
-    pr.D = Dr;
-    pr.dmax = dmax;
-    if (e == cudaSuccess) e = launch_prep(pr, s);
-    // the peaks of every (candidate, FFT) that can reach the refined band
-    RangeArgs ra{};
+    if (e != cudaSuccess) return cuda_error(e, "refinement set-up");
+    // Refined maps are refused where a tile of 2 K + 1 cells with the guard of the
+    // refined drift exceeds a block's shared memory.
+    {
+        double m = 0.0;
+        for (int32_t i = 0; i < n; ++i) {
+            const double x = std::fabs(step_ref * ((pm->t_fft[i] - d.t_ref) * kt));
+            if (x > m && x < 1e9) m = x;  // non-finite times are left to the checks
+        }
+        const int32_t guard = guard_for((unsigned long long)(m * 4294967296.0) + 4);
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (transform_smem_bytes(2 * K + 1, K, FH_MODE_START, 16, guard) >
+            (size_t)max_optin_smem(dev))
+            return cuda_error(cudaErrorInvalidValue, "refined map in shared memory");
+    }
+    const size_t smem = 4 * (size_t)ra.dirs_per * ra.rows_per * E;
+    // shares of the FFTs: two waves of four blocks per SM, at least a block's 256 each
+    const int64_t blocks = (int64_t)std::min(n_cand, cand_batch) * row_groups *
+                           ((dir_batch + ra.dirs_per - 1) / ra.dirs_per);
+    const int64_t shares = std::max<int64_t>(
+        1, std::min<int64_t>(8 * (int64_t)n_sm / blocks, (n + kRefThreads - 1) / kRefThreads));
+    ra.ffts_per = (int32_t)(((n + shares - 1) / shares + 31) / 32 * 32);
     ra.t = t;
     ra.freq = freq;
     ra.v = v;
     ra.sky = sky;
-    ra.n_ref = n_ref;
     ra.offsets = off;
     ra.S0 = S0;
     ra.D = D;
-    ra.Dr = Dr;
     ra.cell = cc;
     ra.row = cr;
     ra.n_fft = n;
-    ra.n_cand = n_cand;
     ra.k_over = K;
     ra.n_rows = n_rows;
+    ra.n_ref = n_ref;
     ra.f0_min = d.f0_min;
     ra.kt = kt;
-    ra.start = start;
-    ra.count = count;
-    ra.S0r = S0r;
-    if (e == cudaSuccess && n > 0 && n_cand > 0) {
-        dim3 grid((n + 255) / 256, n_cand);
-        refine_ranges_kernel<<<grid, 256, 0, s>>>(ra);
-        e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) return cuda_error(e, "refinement set-up");
-    // per-candidate compact offsets (host prefix sums)
-    std::vector<int32_t> h_count((size_t)n_cand * n);
-    if (!h_count.empty())
-        e = cudaMemcpyAsync(h_count.data(), count, 4 * h_count.size(), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_error(e, "refinement ranges");
-    std::vector<int64_t> h_off((size_t)n_cand * (n + 1));
-    std::vector<int64_t> n_sub(n_cand);
-    for (int32_t c = 0; c < n_cand; ++c) {
-        int64_t acc = 0;
-        int64_t *o = &h_off[(size_t)c * (n + 1)];
-        for (int32_t i = 0; i < n; ++i) {
-            o[i] = acc;
-            acc += h_count[(size_t)c * n + i];
-        }
-        o[n] = acc;
-        n_sub[c] = acc;
-    }
-    int64_t *sub_off = nullptr;
-    e = sc.get(&sub_off, h_off.size());
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(sub_off, h_off.data(), 8 * h_off.size(), cudaMemcpyHostToDevice, s);
-    // positions, profiles and windows of every candidate
-    // one allocation each for all candidates' positions and profiles
-    std::vector<int64_t *> A(n_cand, nullptr);
-    std::vector<uint64_t *> prof(n_cand, nullptr);
-    const int32_t n_slabs = (n_rows + kRows - 1) / kRows;
-    size_t a_total = 0;
-    for (int32_t c = 0; c < n_cand; ++c)
-        a_total += (size_t)n_ref * std::max<int64_t>(1, n_sub[c]);
-    const size_t prof_each = (size_t)n_ref * n_f0r;
-    int64_t *a_all = nullptr;
-    uint64_t *prof_all = nullptr;
-    if (e == cudaSuccess) e = sc.get(&a_all, a_total);
-    if (e == cudaSuccess) e = sc.get(&prof_all, prof_each * n_cand);
-    if (e == cudaSuccess) e = cudaMemsetAsync(prof_all, 0, 8 * prof_each * n_cand, s);
-    size_t a_at = 0;
-    for (int32_t c = 0; c < n_cand; ++c) {
-        A[c] = a_all + a_at;
-        a_at += (size_t)n_ref * std::max<int64_t>(1, n_sub[c]);
-        prof[c] = prof_all + prof_each * c;
-    }
-    // every candidate's positions in one launch
-    std::vector<int64_t> h_batch(2 * (size_t)n_cand);
-    for (int32_t c = 0; c < n_cand; ++c) {
-        h_batch[c] = A[c] - a_all;
-        h_batch[n_cand + c] = n_sub[c];
-    }
-    int64_t *d_batch = nullptr;
-    if (e == cudaSuccess) e = sc.get(&d_batch, h_batch.size());
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_batch, h_batch.data(), 8 * h_batch.size(), cudaMemcpyHostToDevice,
-                            s);
-    if (e == cudaSuccess)
-        e = launch_positions_batched(freq, sub_off, v, sky, n, n_ref, n_cand, d_batch,
-                                     d_batch + n_cand, d.f0_min, kt, K, a_all, err, !host_checks,
-                                     start, s);
-    if (e != cudaSuccess) return cuda_error(e, "refinement positions");
-    // the refined drift on the host, for the guard cells (as the device's D')
-    double m = 0.0;
-    for (int32_t i = 0; i < n; ++i) {
-        const double x = std::fabs(step_ref * ((pm->t_fft[i] - d.t_ref) * kt));
-        if (x > m && x < 1e9) m = x;  // non-finite times are left to the checks
-    }
-    const int32_t guard = guard_for((unsigned long long)(m * 4294967296.0) + 4);
-    const int nwarps = 16;
-    const size_t smem = transform_smem_bytes(n_f0r, K, FH_MODE_START, nwarps, guard);
-    e = transform_prepare(FH_MODE_START, smem);
-    if (e != cudaSuccess) return cuda_error(e, "transform_prepare");
-    const int bps = std::max(1, transform_blocks_per_sm(FH_MODE_START, nwarps, smem));
-    for (int32_t g = 0; g < n_cand; g += kMaxBatchJobs) {
-        JobTable tbl{};
-        int64_t items = 0;
-        for (int32_t c = g; c < std::min(n_cand, g + kMaxBatchJobs); ++c) {
-            TransformJob &j = tbl.job[tbl.n_jobs++];
-            j.A = A[c];
-            j.offsets = sub_off + (size_t)c * (n + 1);
-            j.S0 = S0r + (size_t)c * n;
-            j.D = Dr;
-            j.profile = prof[c];
-            j.maps = nullptr;
-            j.dmax = dmax;
-            j.err = err;
-            j.weights = nullptr;
-            j.count_bound = n_sub[c];
-            // no window table: a candidate's ranges hold a few peaks per FFT, so
-            // the transform's own binary search per FFT costs less than a pre-pass
-            j.windows = nullptr;
-            j.n_peaks = n_sub[c];
-            j.n_fft = n;
-            j.n_f0 = n_f0r;
-            j.n_fdot = n_rows;
-            j.k_over = K;
-            j.tile_cells = n_f0r;
-            j.n_slabs = n_slabs;
-            j.n_tiles = 1;
-            j.dir_begin = 0;
-            j.n_dir = n_ref;
-            j.item_begin = items;
-            j.n_items = (int64_t)n_slabs * n_ref;
-            items += j.n_items;
-
-        }
-        const int32_t grid = (int32_t)std::min<int64_t>(items, (int64_t)n_sm * bps);
-        e = launch_transform(FH_MODE_START, tbl, items, grid, nwarps, smem, guard, s);
-        if (e != cudaSuccess) return cuda_error(e, "refinement transform");
-    }
-    // the pick of every candidate
-    uint64_t **d_prof = nullptr;
-    fh_candidate *d_out = nullptr;
-    e = sc.get(&d_prof, (size_t)n_cand);
-    if (e == cudaSuccess) e = sc.get(&d_out, (size_t)n_cand);
-    if (e == cudaSuccess && n_cand > 0)
-        e = cudaMemcpyAsync(d_prof, prof.data(), sizeof(uint64_t *) * (size_t)n_cand,
-                            cudaMemcpyHostToDevice, s);
+    ra.t_ref = d.t_ref;
+    ra.step_ref = step_ref;
+    ra.cshift = 0.5 - 0.5 * (double)K;
+    ra.starts = starts;
+    ra.err = err;
     PickArgs pk{};
-    pk.prof = d_prof;
+    pk.starts = starts;
     pk.cell = cc;
     pk.row = cr;
-    pk.n_cand = n_cand;
-    pk.n_ref = n_ref;
-    pk.n_f0r = n_f0r;
+    pk.n_rows = n_rows;
     pk.k_over = K;
     pk.n_fft = n;
     pk.f0_min = d.f0_min;
@@ -423,17 +460,34 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
     pk.fdot_step_ref = step_ref;
     pk.p0 = d.p0;
     pk.out = d_out;
-    if (e == cudaSuccess && n_cand > 0) {
-        refine_pick_kernel<<<n_cand, 32, 0, s>>>(pk);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess && n_cand > 0)
-        e = cudaMemcpyAsync(out, d_out, sizeof(fh_candidate) * (size_t)n_cand,
-                            cudaMemcpyDeviceToHost, s);
-    int32_t h_err = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h_err, err, 4, cudaMemcpyDeviceToHost, s);
+    pk.best = best;
+    for (int32_t c0 = 0; c0 < n_cand; c0 += cand_batch)
+        for (int32_t b0 = 0; b0 < n_ref; b0 += dir_batch) {
+            const int32_t nc = std::min(cand_batch, n_cand - c0);
+            if (c0 > 0 || b0 > 0) e = cudaMemsetAsync(starts, 0, 4 * n_starts, s);
+            if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync (refinement)");
+            ra.cand0 = pk.cand0 = c0;
+            ra.dir0 = pk.dir0 = b0;
+            ra.n_dir = pk.n_dir = std::min(dir_batch, n_ref - b0);
+            pk.last = b0 + ra.n_dir == n_ref;
+            if (n > 0) {
+                const unsigned groups =
+                    (unsigned)((ra.n_dir + ra.dirs_per - 1) / ra.dirs_per * row_groups);
+                dim3 grid(nc, (n + ra.ffts_per - 1) / ra.ffts_per, groups);
+                refine_kernel<<<grid, kRefThreads, smem, s>>>(ra);
+            }
+            refine_pick_kernel<<<nc, kPickThreads, 0, s>>>(pk);
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return cuda_error(e, "refinement");
+        }
+    std::vector<char> back(out_bytes + 4);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(back.data(), zero, back.size(), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_error(e, "refinement pick");
+    std::memcpy(out, back.data(), out_bytes);
+    int32_t h_err = 0;
+    std::memcpy(&h_err, back.data() + out_bytes, 4);
     if (h_err) return device_error_code(h_err);
     return FH_OK;
 }

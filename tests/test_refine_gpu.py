@@ -154,3 +154,21 @@ def test_refine_with_device_checks(fh, oracle_mod):
         assert ei.value.code == fh.FH_ERR_UNSORTED
     finally:
         fh.fh_destroy_plan(plan)
+
+
+# histograms of all directions and rows, of groups of directions (40 of them), of one
+# direction (256 rows), of groups of rows (K = 16: 213 of 256); K = 1; FFT shares
+# around a block's 256 FFTs; directions taken in two turns (12,000 of them)
+@pytest.mark.parametrize("k_over, k_fdot, n_fft, n_cand, n_ref", [
+    (10, 4, 255, 6, 9), (10, 4, 257, 3, 40), (10, 64, 40, 2, 3), (16, 64, 30, 2, 2),
+    (1, 2, 300, 5, 4), (3, 1, 2049, 1, 1), (30, 64, 4, 1, 12000)])
+def test_groups_and_shares(fh, oracle_mod, k_over, k_fdot, n_fft, n_cand, n_ref):
+    inp, pp = synth.random_case(700 + n_fft + k_over, n_fft=n_fft, n_bins=24, k_over=k_over,
+                                n_fdot=9, n_dir=1, p=0.3)
+    cu = synth.uniform(800 + n_fft, 3, np.arange(2 * n_cand)).reshape(2, n_cand)
+    cells = (cu[0] * pp["n_f0"]).astype(np.int32)
+    rows = (cu[1] * pp["n_fdot"]).astype(np.int32)
+    sky = random_sky_ref(900 + n_fft, n_cand, n_ref)
+    g = gpu_refine(fh, inp, pp, cells, rows, sky, k_fdot)
+    o = oracle_mod.refine(inp, pp, cells, rows, sky, k_fdot)
+    check(g, o, n_cand)
