@@ -307,7 +307,7 @@ struct fh_plan_s {
     int64_t n_peaks = 0;
     int32_t n_dir = 0;
     int64_t launches = 0;
-    size_t prepared_smem[3] = {0, 0, 0};
+    LaunchCache launch;
     // adaptive weights (Eq. ncountadap), set by fh_set_weights until the next
     // fh_correct_doppler: W [max_dir][max_fft] and per-direction sums S1, S2
     int32_t *wq = nullptr;
@@ -345,15 +345,6 @@ struct fh_plan_s {
 };
 
 namespace {
-
-int prepare_transform(fh_plan p, int32_t mode, size_t smem)
-{
-    if (p->prepared_smem[mode] >= smem) return FH_OK;
-    cudaError_t e = transform_prepare(mode, smem);
-    if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(transform)");
-    p->prepared_smem[mode] = smem;
-    return FH_OK;
-}
 
 int check_dirs(fh_plan p, int32_t dir_begin, int32_t n_dir)
 {
@@ -935,8 +926,6 @@ static int run_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *o
                             p->n_sm);
     }
     const size_t smem = transform_smem_bytes(tile, d.k_over, p->mode, nwarps, guard);
-    int rc = prepare_transform(p, p->mode, smem);
-    if (rc) return rc;
     // the window pre-pass clears each direction's profile before the transform
     // merges into it; without FFTs there is no pre-pass, so clear it here
     cudaError_t e = cudaSuccess;
@@ -969,7 +958,9 @@ static int run_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *o
     job.n_slabs = (d.n_fdot + slab_rows - 1) / slab_rows;
     job.n_tiles = (d.n_f0 + tile - 1) / tile;
     const int64_t per_dir = (int64_t)job.n_slabs * job.n_tiles;
-    int bps = transform_blocks_per_sm(p->mode, nwarps, smem);
+    const int bps = transform_blocks_per_sm(p->launch, p->mode, nwarps, p->weighted,
+                                            kind == kPairDirs ? 1 : kind == kPairRows ? 2 : 0,
+                                            out_maps != nullptr, smem);
     if (bps < 1) return set_error(FH_ERR_CUDA, "transform kernel cannot be resident");
     // peak windows of a group of directions (bounded table), then the transform;
     // with direction pairs the table and the work items are per pair, and a group
@@ -990,7 +981,15 @@ static int run_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *o
         if (p->win) cudaFree(p->win);
         p->win = nullptr;
         p->win_bytes = 0;
-        e = cudaMalloc(&p->win, need);
+        // from the scratch pool, which has kept memory at hand (a mapping of its own
+        // costs the first transform of a plan about 100 us), except under capture,
+        // where the graph would own it
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        cudaStreamIsCapturing(s, &capturing);
+        cudaMemPool_t pool =
+            capturing == cudaStreamCaptureStatusNone ? scratch_pool() : nullptr;
+        e = pool ? cudaMallocFromPoolAsync(reinterpret_cast<void **>(&p->win), need, pool, s)
+                 : cudaMalloc(&p->win, need);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return set_error(FH_ERR_NOMEM, "cudaMalloc of %zu bytes (peak windows) failed", need);

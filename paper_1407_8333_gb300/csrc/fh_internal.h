@@ -153,7 +153,20 @@ __host__ __device__ int32_t guard_for(unsigned long long dmax, int32_t span_rows
 // smem bytes the transform needs for tile width W (and mode)
 size_t transform_smem_bytes(int32_t tile_cells, int32_t k_over, int32_t mode, int32_t nwarps,
                             int32_t guard);
-cudaError_t transform_prepare(int32_t mode, size_t smem);  // opt-in dynamic smem
+// How many blocks of the transform kernel of a launch shape fit an SM with `smem`
+// bytes each (below 1: not launchable).  The first use of a shape opts its kernel
+// in to the device's largest dynamic shared memory (never less: other plans may be
+// using the same kernel with more).  The cache belongs to one plan or server; it
+// saves the driver calls of the shapes used last.
+struct LaunchCache {
+    struct Entry {
+        int32_t shape = -1, blocks = 0;
+        size_t smem = 0;
+    } entry[8];
+    int32_t next = 0;
+};
+int transform_blocks_per_sm(LaunchCache &cache, int32_t mode, int32_t nwarps, bool weighted,
+                            int pack, bool maps, size_t smem);
 // sched: null (every block takes every grid-th item) or two device words that
 // are zero at the launch (a counter handing out items after each block's
 // first, and a count of finished blocks); the kernel's last block zeroes them
@@ -161,7 +174,6 @@ cudaError_t transform_prepare(int32_t mode, size_t smem);  // opt-in dynamic sme
 cudaError_t launch_transform(int32_t mode, const JobTable &tbl, int64_t total_items,
                              int32_t grid, int32_t nwarps, size_t smem, int32_t guard,
                              cudaStream_t s, unsigned int *sched = nullptr);
-int transform_blocks_per_sm(int32_t mode, int32_t nwarps, size_t smem);
 // Peak windows of every (direction, slab, tile, FFT) of a job, written to
 // job.windows (the job's other fields as for the transform).
 cudaError_t launch_windows(const TransformJob &job, uint32_t *windows, cudaStream_t s);

@@ -887,7 +887,11 @@ __device__ __forceinline__ void diff_steps(std::integer_sequence<int, Ts...>, in
 // with the other segments' totals as carry-in.  The count goes to the map
 // (optional) and the warp's max over rows (smallest row on ties) to the
 // direction's profile by a 64-bit atomicMax, which is order-independent.
-template <int MODE, int MAXT, bool WEIGHTED, int PACK>
+//
+// MAPS: the counts also go to J->maps.  An instantiation of its own: the walk
+// shares its registers with the emit, and carrying the map's code cost the
+// kernels without maps 1 %.
+template <int MODE, int MAXT, bool WEIGHTED, int PACK, bool MAPS>
 __global__ void __launch_bounds__(MAXT, 1)
 transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int32_t hist_words,
                  int32_t guard, uint32_t cell_stride, unsigned int *__restrict__ sched)
@@ -1331,6 +1335,39 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
             }
 
             // emit counts, map and profile
+            // A group of 16 cells x 32 rows of the map leaves through 2 KB of the guard
+            // cells per warp (free now; where they hold one for every emitting warp): lane = row
+            // writes its 16 counts, then four lanes write a row's 64 bytes, two whole
+            // sectors, eight rows per 16-byte store.  A word of (cell m, row r) lies at
+            // m 32 + (r + 8 (m / 4)) mod 32, on its own bank in both directions.  (With
+            // each lane storing its own row a store touched 32 lines and half a sector
+            // of each: the 383 MB map of the 50 Hz workload cost 150 us of the kernel, now
+            // 40 us.)
+            int32_t *stage = nullptr;
+            if (MAPS && J->maps != nullptr) {
+                const int n_low = guard >> 4;  // in cells -guard .. -1, the rest above E
+                const int n_high = (hist_words / kRows - guard - (E + 1)) >> 4;
+                // (the warps that emit: segments of whole groups, as below)
+                const int seg = (((Wt + nwarps - 1) / nwarps) + 15) & ~15;
+                if (n_low + max(n_high, 0) >= (Wt + seg - 1) / seg)
+                    stage = warp < n_low ? Hlo + warp * (16 * kRows)
+                                         : H + (E + 1 + (warp - n_low) * 16) * kRows;
+            }
+            auto store16 = [&](const auto &v, int32_t *row0, int rows) {
+#pragma unroll
+                for (int m = 0; m < 16; ++m)
+                    stage[m * kRows + ((lane + 8 * (m >> 2)) & 31)] = v[m];
+                __syncwarp();
+                const int g = lane & 3;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int r = 8 * j + (lane >> 2);
+                    const int32_t *x = stage + 4 * g * kRows + ((r + 8 * g) & 31);
+                    const int4 w = make_int4(x[0], x[kRows], x[2 * kRows], x[3 * kRows]);
+                    if (r < rows) *reinterpret_cast<int4 *>(row0 + (int64_t)r * n_f0 + 4 * g) = w;
+                }
+                __syncwarp();
+            };
             unsigned long long *prof = reinterpret_cast<unsigned long long *>(J->profile) +
                                        (int64_t)(d_abs + dsel) * n_f0 + b0;
             if constexpr (QUAD) {
@@ -1346,7 +1383,10 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                 const bool ok_a = lane < min(R, kRows);
                 const bool ok_b = ROWQ ? lane < R - kRows : ok_a;
                 int32_t *map_a = nullptr, *map_b = nullptr;
-                if (J->maps != nullptr) {
+                int32_t *rows_a = nullptr, *rows_b = nullptr;  // row j0 of each
+                if (MAPS && J->maps != nullptr) {
+                    rows_a = J->maps + ((int64_t)d_rel * n_fdot + j0) * n_f0 + b0;
+                    rows_b = rows_a + (ROWQ ? (int64_t)kRows * n_f0 : (int64_t)n_fdot * n_f0);
                     int32_t *const m0 = J->maps + ((int64_t)d_rel * n_fdot + j0 + lane) * n_f0 + b0;
                     if (ok_a) map_a = m0;
                     if (ok_b) map_b = m0 + (ROWQ ? (int64_t)kRows * n_f0 : (int64_t)n_fdot * n_f0);
@@ -1378,6 +1418,9 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                 const bool vec_map = map_a != nullptr && map_b != nullptr &&
                                      (((uintptr_t)map_a & 15u) == 0) &&
                                      (((uintptr_t)map_b & 15u) == 0);
+                // (both row 0s aligned and whole rows a multiple of 16 bytes: every row)
+                const bool staged = stage != nullptr && (n_f0 & 3) == 0 &&
+                                    (((uintptr_t)rows_a | (uintptr_t)rows_b) & 15u) == 0;
                 auto run = [&](auto map_tag) {
                     constexpr bool kMap = decltype(map_tag)::value;
                     int c = c0;
@@ -1404,7 +1447,10 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                             }
                         }
                         if constexpr (kMap) {
-                            if (vec_map) {
+                            if (staged) {
+                                store16(ca, rows_a + c, min(R, kRows));
+                                store16(cbn, rows_b + c, ROWQ ? R - kRows : R);
+                            } else if (vec_map) {
                                 int4 *da = reinterpret_cast<int4 *>(map_a + c);
                                 int4 *db = reinterpret_cast<int4 *>(map_b + c);
 #pragma unroll
@@ -1452,14 +1498,18 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                         }
                     }
                 };
-                if (J->maps != nullptr)
-                    run(std::true_type{});
+                if (MAPS && J->maps != nullptr)
+                    run(std::integral_constant<bool, MAPS>{});
                 else
                     run(std::false_type{});
             } else {
-                int32_t *maprow = nullptr;
-                if (J->maps != nullptr && row_ok)
-                    maprow = J->maps + ((int64_t)(d_rel + dsel) * n_fdot + j0 + lane) * n_f0 + b0;
+                int32_t *maprow = nullptr, *row0 = nullptr;
+                if (MAPS && J->maps != nullptr) {
+                    row0 = J->maps + ((int64_t)(d_rel + dsel) * n_fdot + j0) * n_f0 + b0;
+                    if (row_ok) maprow = row0 + (int64_t)lane * n_f0;
+                }
+                const bool staged = stage != nullptr && (n_f0 & 3) == 0 &&
+                                    ((uintptr_t)row0 & 15u) == 0;
                 // Per cell the profile takes the warp's max over its rows, smallest row
                 // on ties.  Counts below 2^26 fit one packed signed reduction
                 // 32 count + (31 - lane); rows beyond the pass start their window at
@@ -1503,7 +1553,9 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                                 if (lane == m) myv = v;
                             }
                             if constexpr (kMap) {
-                                if (vec_map) {
+                                if (staged) {
+                                    store16(cnts, row0 + c, R);
+                                } else if (vec_map) {
                                     int4 *d4 = reinterpret_cast<int4 *>(maprow + c);
 #pragma unroll
                                     for (int q = 0; q < 4; ++q)
@@ -1525,8 +1577,8 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                             if (lane == 0) atomicMax(prof + c, key_of(v));
                         }
                     };
-                    if (J->maps != nullptr)
-                        run(std::true_type{});
+                    if (MAPS && J->maps != nullptr)
+                        run(std::integral_constant<bool, MAPS>{});
                     else
                         run(std::false_type{});
                 } else {
@@ -1536,7 +1588,7 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                     const int c0 = min(Wt, warp * seg);
                     const int c1 = min(Wt, c0 + seg);
                     auto emit = [&](int c, int count) {
-                        if (maprow) maprow[c] = count;
+                        if (MAPS && maprow) maprow[c] = count;
                         const int m = __reduce_max_sync(kFull, row_ok ? count : INT_MIN);
                         const unsigned rm =
                             __reduce_min_sync(kFull, (row_ok && count == m) ? (unsigned)lane : 32u);
@@ -1943,56 +1995,68 @@ size_t transform_smem_bytes(int32_t tile_cells, int32_t k_over, int32_t mode, in
 // Kernel instantiation for a counting mode and block size: blocks of up to 512
 // threads get up to 128 registers per thread, of up to 640 threads (START
 // mode) 102, of up to 768 threads 80, of 1024 threads 64.
-template <bool WEIGHTED, int PACK, typename F>
+template <bool WEIGHTED, int PACK, bool MAPS, typename F>
 static auto with_transform_kernel_w(int32_t mode, int32_t nwarps, F &&f)
 {
     if constexpr (!PACK) {
         if (mode == FH_MODE_DIFF)
-            return nwarps > 16 ? f(transform_kernel<FH_MODE_DIFF, 1024, WEIGHTED, false>)
-                               : f(transform_kernel<FH_MODE_DIFF, 512, WEIGHTED, false>);
+            return nwarps > 16 ? f(transform_kernel<FH_MODE_DIFF, 1024, WEIGHTED, 0, MAPS>)
+                               : f(transform_kernel<FH_MODE_DIFF, 512, WEIGHTED, 0, MAPS>);
     }
-    return nwarps > 24   ? f(transform_kernel<FH_MODE_START, 1024, WEIGHTED, PACK>)
-           : nwarps > 20 ? f(transform_kernel<FH_MODE_START, 768, WEIGHTED, PACK>)
-           : nwarps > 16 ? f(transform_kernel<FH_MODE_START, 640, WEIGHTED, PACK>)
-                         : f(transform_kernel<FH_MODE_START, 512, WEIGHTED, PACK>);
+    if constexpr (MAPS)  // two sizes are enough: the emit weighs more there
+        return nwarps > 24 ? f(transform_kernel<FH_MODE_START, 1024, WEIGHTED, PACK, true>)
+                           : f(transform_kernel<FH_MODE_START, 768, WEIGHTED, PACK, true>);
+    else
+        return nwarps > 24   ? f(transform_kernel<FH_MODE_START, 1024, WEIGHTED, PACK, false>)
+               : nwarps > 20 ? f(transform_kernel<FH_MODE_START, 768, WEIGHTED, PACK, false>)
+               : nwarps > 16 ? f(transform_kernel<FH_MODE_START, 640, WEIGHTED, PACK, false>)
+                             : f(transform_kernel<FH_MODE_START, 512, WEIGHTED, PACK, false>);
 }
 // weighted: instantiation that adds per-FFT weights (adaptive map); plain: +1;
-// pack: direction pairs with two 16-bit counts per word (plain START map only)
+// pack: direction pairs (1) or row pairs (2) with two 16-bit counts per word (plain
+// START map only); maps: the counts are written out
+template <bool MAPS, typename F>
+static auto with_transform_kernel_m(int32_t mode, int32_t nwarps, bool weighted, int pack, F &&f)
+{
+    if (pack == 1) return with_transform_kernel_w<false, 1, MAPS>(FH_MODE_START, nwarps, f);
+    if (pack == 2) return with_transform_kernel_w<false, 2, MAPS>(FH_MODE_START, nwarps, f);
+    return weighted ? with_transform_kernel_w<true, 0, MAPS>(mode, nwarps, f)
+                    : with_transform_kernel_w<false, 0, MAPS>(mode, nwarps, f);
+}
 template <typename F>
-static auto with_transform_kernel(int32_t mode, int32_t nwarps, bool weighted, int pack, F &&f)
+static auto with_transform_kernel(int32_t mode, int32_t nwarps, bool weighted, int pack, bool maps,
+                                  F &&f)
 {
-    if (pack == 1) return with_transform_kernel_w<false, 1>(FH_MODE_START, nwarps, f);
-    if (pack == 2) return with_transform_kernel_w<false, 2>(FH_MODE_START, nwarps, f);
-    return weighted ? with_transform_kernel_w<true, 0>(mode, nwarps, f)
-                    : with_transform_kernel_w<false, 0>(mode, nwarps, f);
+    return maps ? with_transform_kernel_m<true>(mode, nwarps, weighted, pack, f)
+                : with_transform_kernel_m<false>(mode, nwarps, weighted, pack, f);
 }
 
-cudaError_t transform_prepare(int32_t mode, size_t smem)
+int transform_blocks_per_sm(LaunchCache &cache, int32_t mode, int32_t nwarps, bool weighted,
+                            int pack, bool maps, size_t smem)
 {
-    cudaError_t e = cudaSuccess;
-    for (int nw : {16, 20, 24, 32})
-        for (int v = 0; v < 4; ++v) {
-            const bool wt = v == 1;
-            const int pk = v >= 2 ? v - 1 : 0;
-            if (pk && mode != FH_MODE_START) continue;
-            const cudaError_t r = with_transform_kernel(mode, nw, wt, pk, [&](auto k) {
-                return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)smem);
-            });
-            if (r != cudaSuccess) e = r;
-        }
-    return e;
-}
-
-int transform_blocks_per_sm(int32_t mode, int32_t nwarps, size_t smem)
-{
-    int n = 0;
-    // (both instantiations are bounded to one block of nwarps warps per SM by
-    // their launch bounds; shared memory decides the rest)
-    const cudaError_t e = with_transform_kernel(mode, nwarps, false, 0, [&](auto k) {
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, nwarps * 32, smem);
+    const int32_t shape = mode | nwarps << 4 | (weighted ? 1 : 0) << 12 | pack << 13 |
+                          (maps ? 1 : 0) << 16;
+    for (const auto &x : cache.entry)
+        if (x.shape == shape && x.smem == smem) return x.blocks;
+    int n = 0, dev = 0;
+    cudaGetDevice(&dev);
+    const cudaError_t e = with_transform_kernel(mode, nwarps, weighted, pack, maps, [&](auto k) {
+        const cudaError_t r = cudaFuncSetAttribute(
+            k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_optin_smem(dev));
+        return r != cudaSuccess
+                   ? r
+                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, nwarps * 32, smem);
     });
-    return e == cudaSuccess ? n : 0;
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    auto &x = cache.entry[cache.next];
+    cache.next = (cache.next + 1) % 8;
+    x.shape = shape;
+    x.smem = smem;
+    x.blocks = n;
+    return n;
 }
 
 cudaError_t launch_transform(int32_t mode, const JobTable &tbl, int64_t total_items,
@@ -2009,14 +2073,16 @@ cudaError_t launch_transform(int32_t mode, const JobTable &tbl, int64_t total_it
     }
     // the launch's packing: every job with direction pairs (1), or with row pairs (2)
     bool weighted = false, dirs = mode == FH_MODE_START && tbl.n_jobs > 0, rows = dirs;
+    bool maps = false;
     for (int j = 0; j < tbl.n_jobs; ++j) {
+        maps = maps || tbl.job[j].maps != nullptr;
         weighted = weighted || tbl.job[j].weights != nullptr;
         dirs = dirs && tbl.job[j].dir_pairs != 0;
         rows = rows && tbl.job[j].row_pairs != 0;
     }
     const int pack = dirs ? 1 : rows ? 2 : 0;
     if (weighted && pack) return cudaErrorInvalidValue;  // packed counters hold plain counts only
-    with_transform_kernel(mode, nwarps, weighted, pack, [&](auto k) {
+    with_transform_kernel(mode, nwarps, weighted, pack, maps, [&](auto k) {
         k<<<grid, nwarps * 32, smem, s>>>(tbl, total_items, hist_words, guard, kRows * 4u, sched);
         return cudaSuccess;
     });

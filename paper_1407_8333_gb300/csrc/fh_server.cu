@@ -157,7 +157,7 @@ struct fh_server_s {
     int32_t next_batch = 0;
     int64_t pending = 0;  // jobs not yet DONE/FAILED/CANCELLED
     Clock::time_point t0 = Clock::now();
-    size_t prepared_smem = 0;
+    LaunchCache launch;
     std::string fatal;
 
     double now() const
@@ -309,12 +309,9 @@ int fh_server_s::launch_batch(Slot &slot, std::vector<Job *> &batch)
             e = launch_windows(t, j->d_win, s);
             if (e != cudaSuccess) return cuda_error(e, "windows launch");
         }
-        if (smem > prepared_smem) {
-            e = transform_prepare(FH_MODE_START, smem);
-            if (e != cudaSuccess) return cuda_error(e, "transform_prepare");
-            prepared_smem = smem;
-        }
-        const int bps = std::max(1, transform_blocks_per_sm(FH_MODE_START, nwarps, smem));
+        const int bps = transform_blocks_per_sm(launch, FH_MODE_START, nwarps, false, kind, false,
+                                                smem);
+        if (bps < 1) return set_error(FH_ERR_CUDA, "transform kernel cannot be resident");
         const int32_t grid = (int32_t)std::min<int64_t>(items, (int64_t)n_sm * bps);
         e = launch_transform(FH_MODE_START, tbl, items, grid, nwarps, smem, guard, s, slot.sched);
         if (e != cudaSuccess) return cuda_error(e, "transform launch");

@@ -156,8 +156,6 @@ int fh_search_static(const fh_plan_desc *desc, const fh_peakmap *pm, const doubl
     const size_t smem = transform_smem_bytes(tile, d.k_over, mode, nwarps, guard);
     if (smem > (size_t)max_optin_smem(dev))
         return set_error(FH_ERR_INVALID_ARG, "tile_cells too wide for shared memory");
-    e = transform_prepare(mode, smem);
-    if (e != cudaSuccess) return cuda_error(e, "transform_prepare");
     JobTable tbl{};
     tbl.n_jobs = 1;
     TransformJob &job = tbl.job[0];
@@ -184,7 +182,8 @@ int fh_search_static(const fh_plan_desc *desc, const fh_peakmap *pm, const doubl
     job.dir_begin = 0;
     job.n_dir = 1;
     job.n_items = (int64_t)job.n_slabs * job.n_tiles;
-    const int bps = transform_blocks_per_sm(mode, nwarps, smem);
+    LaunchCache launch;
+    const int bps = transform_blocks_per_sm(launch, mode, nwarps, false, 0, false, smem);
     if (bps < 1) return set_error(FH_ERR_CUDA, "transform kernel cannot be resident");
     const int64_t cap = (int64_t)n_sm * bps;
     const int32_t grid = (int32_t)(job.n_items < cap ? job.n_items : cap);

@@ -85,3 +85,41 @@ def test_selection_block_sizes(fh, subband_bins, k_over):
                                 n_dir=2, p=0.1, subband_bins=subband_bins, top_k=4,
                                 excl_cells=2 * k_over, sep_cells=3 * k_over)
     check(fh, inp, pp)
+
+
+# maps staged through the guard cells: 16-cell groups with rows of 16 bytes (n_f0 a
+# multiple of 4), written row by row where they are not (odd K and bins), more warps
+# than the guard cells hold a stage for; ragged last groups, tiles and slabs
+@pytest.mark.parametrize("n_bins, k_over", [(40, 4), (33, 4), (41, 3), (100, 10), (64, 1)])
+@pytest.mark.parametrize("n_dir, n_fdot", [(1, 5), (1, 45), (1, 70), (2, 33), (3, 31)])
+def test_written_maps(fh, n_bins, k_over, n_dir, n_fdot):
+    for warps, tile in ((4, 64), (16, 0), (24, 0), (32, 0)):
+        inp, pp = synth.random_case(400 + n_bins + n_fdot, n_fft=50, n_bins=n_bins, k_over=k_over,
+                                    n_fdot=n_fdot, n_dir=n_dir, p=0.2, vmax=2e-6)
+        check(fh, inp, pp, block_warps=warps, tile_cells=min(tile, pp["n_f0"]))
+    w = 0.5 + np.arange(n_dir * 50).reshape(n_dir, 50) % 3
+    check(fh, inp, pp, weights=w)
+
+
+def test_plans_of_different_shapes_take_turns(fh):
+    """A plan with small tiles between two passes of one with the largest."""
+    import torch
+    import oracle
+    big, pb = synth.random_case(81, n_fft=40, n_bins=400, n_fdot=40, n_dir=2, p=0.1, vmax=2e-6)
+    small, ps = synth.random_case(82, n_fft=40, n_bins=20, n_fdot=40, n_dir=2, p=0.1, vmax=2e-6)
+    plans, want = [], []
+    for inp, pp, tile in ((big, pb, 0), (small, ps, 32)):
+        plan = fh.fh_create_plan(fh.make_desc(pp, 40, 2, inp.n_peaks, tile_cells=tile))
+        dev = [torch.from_numpy(np.ascontiguousarray(x)).cuda()
+               for x in (inp.t, inp.offsets, inp.freq, inp.v, inp.sky)]
+        fh.fh_correct_doppler(plan, *dev)
+        plans.append((plan, dev))
+        want.append(oracle.search(inp, pp))
+    try:
+        for k in (0, 1, 0, 1):
+            fh.fh_transform(plans[k][0], 0, 2)
+            c = fh.fh_select_candidates(plans[k][0], 0, 2)
+            assert np.array_equal(c["count"].ravel(), want[k]["count"].ravel())
+    finally:
+        for plan, _ in plans:
+            fh.fh_destroy_plan(plan)
