@@ -123,3 +123,45 @@ def test_plans_of_different_shapes_take_turns(fh):
     finally:
         for plan, _ in plans:
             fh.fh_destroy_plan(plan)
+
+
+# positions formed in integers and, where their bounds fail, in binary64: band edges
+# at and around powers of two, T_FFT that is not one (K T odd up to 675), K up to
+# 40, frequencies on and off the bin grid, far above and below the band, r on both
+# sides of 1, f0 of 0 and below
+@pytest.mark.parametrize("f0", [0.0, -3.0, 1e-3, 63.75, 64.0, 127.999, 900.0, 903.21, 1999.3])
+@pytest.mark.parametrize("t_fft, k_over", [(1024.0, 10), (8192.0, 7), (1800.0, 12), (4096.0, 40),
+                                           (3.0, 1), (1000.1, 1)])
+def test_positions_in_integers(fh, f0, t_fft, k_over):
+    import torch
+    import oracle
+    rng = np.random.RandomState(int(t_fft) + k_over)
+    n_fft, base = 17, max(abs(f0), 1.0)
+    parts = [np.round((base + rng.uniform(-0.2, 9.0, 40)) * t_fft) / t_fft,
+             base + rng.uniform(-0.3, 12.0, 40), base * rng.uniform(0.3, 3.0, 10),
+             np.nextafter(base, 1e9) * np.ones(1), np.array([base, base / 2, base * 2])]
+    f = np.unique(np.abs(np.concatenate(parts)) + 1e-9)
+    f[:20] = np.round(f[:20] * 1024) / 1024
+    f = np.unique(f[f > 0])
+    offsets = np.arange(n_fft + 1, dtype=np.int64) * len(f)
+    freq = np.tile(f, n_fft)
+    t = np.arange(n_fft) * 0.5 * t_fft
+    v = rng.uniform(-1, 1, (n_fft, 3)) * np.array([0.0, 1e-9, 1e-4, 0.05])[np.arange(n_fft) % 4, None]
+    sky = np.array([[0.6, 0.0, 0.8], [-0.6, 0.64, 0.48]])
+    pp = dict(t_fft=t_fft, k_over=k_over, f0_min=f0, n_f0=50, fdot_min=0.0, fdot_step=1e-12,
+              n_fdot=1, t_ref=0.0, subband_cells=50, top_k=1, excl_cells=0, sep_cells=0, n_thr=0,
+              p0=0.1)
+    plan = fh.fh_create_plan(fh.make_desc(pp, n_fft, 2, len(freq)))
+    try:
+        A = torch.empty((2, len(freq)), dtype=torch.int64, device="cuda")
+        dev = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (t, offsets, freq, v, sky)]
+        fh.fh_correct_doppler(plan, *dev, out_A=A)
+        got = A.cpu().numpy()
+    finally:
+        fh.fh_destroy_plan(plan)
+    kt = float(k_over) * t_fft
+    r = oracle.doppler_factor(v, sky)
+    x = (freq[None, :] * np.repeat(r, len(f), axis=1) - f0) * kt + (0.5 - 0.5 * k_over)
+    near = np.abs(x) < 2.0 ** 28   # beyond that a call is refused
+    want = np.floor(x * 2.0 ** 32)[near].astype(np.int64)
+    assert near.sum() > 1000 and np.array_equal(got[near], want)
