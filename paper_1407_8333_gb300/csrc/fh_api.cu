@@ -131,6 +131,11 @@ static void count_plans(int change)
 // the error word (bytes 0..3) and the largest |D| (bytes 16..23) of a plan,
 // one allocation cleared by one memset per call
 constexpr size_t kErrWordsBytes = 32;
+// with the pair distances of n_dir directions behind them
+constexpr int64_t err_block_bytes(int32_t n_dir)
+{
+    return (int64_t)kErrWordsBytes + 4 * (int64_t)n_dir;
+}
 
 // Device address of a page-locked (pinned or registered, mapped) host array,
 // which kernels can read in place; nullptr for pageable or unknown memory.
@@ -291,7 +296,7 @@ struct fh_plan_s {
     unsigned long long *dmax = nullptr;  // largest |D_i| of the current peakmap (in err's block)
     int32_t *dense = nullptr;            // set by the window pre-pass: an FFT with two peaks
                                          // in one cell (in err's block)
-    int32_t *unit_delta = nullptr;       // per direction pair of a group: the largest distance
+    int32_t *unit_delta = nullptr;       // (in err's block) per pair's first direction: the largest distance
                                          // between a peak's two cells (window pre-pass)
     unsigned int *sched = nullptr;       // the batched transform's item counter (2 words,
                                          // zero between launches)
@@ -325,7 +330,7 @@ struct fh_plan_s {
         for (cudaEvent_t ev : tev) cudaEventDestroy(ev);
         tev.clear();
         void *bufs[] = {t,    freq, v,   sky,  offsets, offsets_raw, S0, D,
-                        A,    profile, cand, err, win,  wq,  ws, unit_delta, sched};  // dmax: in err's block
+                        A,    profile, cand, err, win,  wq,  ws, sched};  // dmax, unit_delta: in err's block
         for (void *b : bufs)
             if (b) cudaFree(b);
         if (h_err) cudaFreeHost(h_err);
@@ -521,8 +526,7 @@ int fh_create_plan(const fh_plan_desc *desc, fh_plan *out)
                   {(void **)&p->freq, s.freq},     {(void **)&p->v, s.v},
                   {(void **)&p->sky, s.sky},       {(void **)&p->A, s.A},
                   {(void **)&p->profile, s.profile}, {(void **)&p->cand, s.cand},
-                  {(void **)&p->err, kErrWordsBytes},
-                  {(void **)&p->unit_delta, 4 * ((int64_t)desc->max_dir / 2 + 1)},
+                  {(void **)&p->err, err_block_bytes(desc->max_dir)},
                   {(void **)&p->sched, 16}};
     for (auto &a : allocs) {
         e = cudaMalloc(a.ptr, (size_t)std::max<int64_t>(a.bytes, 16));
@@ -545,7 +549,8 @@ int fh_create_plan(const fh_plan_desc *desc, fh_plan *out)
         delete p;
         return set_error(FH_ERR_NOMEM, "cudaMallocHost failed");
     }
-    cudaMemset(p->err, 0, kErrWordsBytes);
+    p->unit_delta = reinterpret_cast<int32_t *>(reinterpret_cast<char *>(p->err) + kErrWordsBytes);
+    cudaMemset(p->err, 0, err_block_bytes(desc->max_dir));
     cudaMemset(p->sched, 0, 16);
     count_plans(1);
     *out = p;
@@ -769,7 +774,7 @@ int fh_correct_doppler(fh_plan p, const fh_peakmap *pm, const double *v_over_c,
     const bool host_checks = p->input_checks == FH_CHECKS_HOST;
     p->weighted = false;  // a new peakmap starts with unit weights
     // the error word and the largest |D| share one allocation: one memset
-    cudaError_t e = cudaMemsetAsync(p->err, 0, kErrWordsBytes, s);
+    cudaError_t e = cudaMemsetAsync(p->err, 0, err_block_bytes(n_dir), s);
     if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync");
     if (pm->mem_kind == FH_MEM_HOST) {
         if (!pm->offsets || (n > 0 && !pm->t_fft) || (np > 0 && !pm->freq))
@@ -1006,10 +1011,6 @@ static int run_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *o
         job.item_begin = 0;
         job.n_items = per_dir * ((gn + per_unit - 1) / per_unit);
         job.windows = p->win;
-        if (pairs) {
-            e = cudaMemsetAsync(p->unit_delta, 0, sizeof(int32_t) * (size_t)((gn + 1) / 2), s);
-            if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync(pair distances)");
-        }
         cudaEvent_t *ev = nullptr;
         if (p->timing && !p->tev.empty()) {
             ev = &p->tev[3 * (size_t)(p->tev_next % kTimingSlots)];

@@ -49,6 +49,38 @@ __device__ __forceinline__ int64_t floor_times_2p32(double x)
     }
     return (bits >> 63) ? -(int64_t)q - (frac ? 1 : 0) : (int64_t)q;
 }
+
+// Programmatic dependent launch: a kernel launched by launch_after may be set up, and
+// its blocks become resident, while the kernel before it on the stream drains; its
+// first statement, wait_for_previous(), holds it until that one has completed
+// (and so, as every kernel of a chain waits, all before it).  A kernel that calls
+// let_next_start() allows its successor in once all its own blocks have started.
+// Without a kernel before it, or in a plain launch, both do nothing.  Worth 1 - 2 us
+// per launch of a chain: a step of four kernels on 200 FFTs 45.2 -> 42.6 us.
+__device__ __forceinline__ void wait_for_previous()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void let_next_start()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... Q>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                         Q &&...args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
 #endif
 
 // One direction set of one plan, as the transform kernel sees it.
@@ -76,8 +108,9 @@ struct TransformJob {
     int32_t dir_pairs;       // 1: items cover directions 2u and 2u + 1 with two 16-bit
                              // counts per shared word (plain START map, every job of a
                              // launch alike); the window table is per pair
-    int32_t *unit_delta;     // (dir_pairs) per pair, the largest cell distance between a
-                             // peak's two positions (+2), from the window pre-pass
+    int32_t *unit_delta;     // (dir_pairs) per absolute index of a pair's first direction, the
+                             // largest cell distance between a peak's two positions (+2),
+                             // from the window pre-pass (zeroed with the positions)
     int32_t delta_alloc;     // (dir_pairs) the part of the guard that holds that distance;
                              // a pair beyond it takes the clamped walk
     int32_t row_pairs;       // 1 (plain START map of one direction, not with dir_pairs):

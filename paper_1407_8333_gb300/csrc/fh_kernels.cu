@@ -347,6 +347,7 @@ __global__ void __launch_bounds__(kPosThreads)
 correct_kernel(const PrepArgs a, const double *__restrict__ freq, double f0_min, double cshift,
                const PosGrid G, int64_t *__restrict__ A, double *__restrict__ out_r)
 {
+    let_next_start();
     int32_t e = 0;
     unsigned long long amax = 0;
     if (blockIdx.x == 0) {
@@ -547,6 +548,8 @@ windows_kernel(const TransformJob J, uint32_t *__restrict__ windows)
     constexpr int kPeaks = PAIR ? 736 : 1024;
     // rows padded by one word: lanes on different FFTs fall on different banks
     __shared__ int32_t cell_s[NR][8][kPeaks + 1];
+    let_next_start();
+    wait_for_previous();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int unit = blockIdx.y;
     const int nd = PAIR ? min(2, J.n_dir - 2 * unit) : 1;  // directions of the unit
@@ -621,7 +624,7 @@ windows_kernel(const TransformJob J, uint32_t *__restrict__ windows)
             const int64_t d0 = (int64_t)global_cell(Ab, 0) - global_cell(Aa, 0);
             const int64_t d1 = (int64_t)global_cell(Ab, ns - 1) - global_cell(Aa, ns - 1);
             const int64_t dm = max(d0 < 0 ? -d0 : d0, d1 < 0 ? -d1 : d1) + 2;
-            atomicMax(J.unit_delta + unit, (int32_t)min(dm, (int64_t)INT_MAX));
+            atomicMax(J.unit_delta + d_first, (int32_t)min(dm, (int64_t)INT_MAX));
         }
     }
     __syncthreads();
@@ -996,6 +999,8 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
     // PACK: 0 full-word counters; 1 direction pairs; 2 row pairs (one direction)
     static_assert(!PACK || (MODE == FH_MODE_START && !WEIGHTED), "packed counters: plain START");
     extern __shared__ __align__(16) int32_t smem_raw[];
+    let_next_start();
+    wait_for_previous();
     const int lane = threadIdx.x & 31;
     // (out of a shuffle: known to be uniform in the warp)
     const int warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
@@ -1088,7 +1093,7 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
         // a pair whose positions lie further apart than the job allows walks clamped
         const bool fast = MODE == FH_MODE_START && ((job_fast >> jb) & 1u) &&
                           (!has_b || J->unit_delta == nullptr ||
-                           J->unit_delta[unit] <= J->delta_alloc);
+                           J->unit_delta[d_abs] <= J->delta_alloc);
         const int64_t base_shift = (int64_t)(b0 - K + 1) * 4294967296LL;
         const int64_t e_fixed = (int64_t)E * 4294967296LL;
         const int nchunks = (n_fft + 31) >> 5;
@@ -1804,6 +1809,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectArgs a)
     __shared__ unsigned long long wkey[kSelThreads / 32];
     __shared__ int wcell[kSelThreads / 32];
     __shared__ int npick, stop;
+    wait_for_previous();
     const int q = blockIdx.x, d_rel = blockIdx.y;
     const int lo = q * a.subband_cells;
     const int hi = min(a.n_f0, lo + a.subband_cells);
@@ -2187,11 +2193,10 @@ cudaError_t launch_transform(int32_t mode, const JobTable &tbl, int64_t total_it
     }
     const int pack = dirs ? 1 : rows ? 2 : 0;
     if (weighted && pack) return cudaErrorInvalidValue;  // packed counters hold plain counts only
-    with_transform_kernel(mode, nwarps, weighted, pack, maps, [&](auto k) {
-        k<<<grid, nwarps * 32, smem, s>>>(tbl, total_items, hist_words, guard, kRows * 4u, sched);
-        return cudaSuccess;
+    return with_transform_kernel(mode, nwarps, weighted, pack, maps, [&](auto k) {
+        return launch_after(k, grid, nwarps * 32, smem, s, tbl, total_items, hist_words, guard,
+                            kRows * 4u, sched);
     });
-    return cudaGetLastError();
 }
 
 cudaError_t launch_windows(const TransformJob &job, uint32_t *windows, cudaStream_t s)
@@ -2202,18 +2207,12 @@ cudaError_t launch_windows(const TransformJob &job, uint32_t *windows, cudaStrea
     const int m = std::min(kWinMaxM, std::max(1, (job.n_tiles + 31) / 32));
     auto go = [&](auto pair_tag) {
         constexpr bool P = decltype(pair_tag)::value;
-        if (m == 1)
-            windows_kernel<1, P><<<grid, 256, 0, s>>>(job, windows);
-        else if (m == 2)
-            windows_kernel<2, P><<<grid, 256, 0, s>>>(job, windows);
-        else
-            windows_kernel<3, P><<<grid, 256, 0, s>>>(job, windows);
+        auto *k = m == 1   ? windows_kernel<1, P>
+                  : m == 2 ? windows_kernel<2, P>
+                           : windows_kernel<3, P>;
+        return launch_after(k, grid, 256, 0, s, job, windows);
     };
-    if (job.dir_pairs)
-        go(std::true_type{});
-    else
-        go(std::false_type{});
-    return cudaGetLastError();
+    return job.dir_pairs ? go(std::true_type{}) : go(std::false_type{});
 }
 
 cudaError_t launch_select(const SelectArgs &a, cudaStream_t s)
@@ -2224,8 +2223,7 @@ cudaError_t launch_select(const SelectArgs &a, cudaStream_t s)
     const int cells = std::min(a.subband_cells, a.n_f0);
     const int threads = (int)std::min<int64_t>(kSelThreads, ((int64_t)cells + 32 * kSelPer - 1) /
                                                                 (32 * kSelPer) * 32);
-    select_kernel<<<grid, threads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_after(select_kernel, grid, threads, 0, s, a);
 }
 
 cudaError_t launch_weight_bound(const int64_t *A, const int64_t *offsets, const int32_t *W,

@@ -104,7 +104,7 @@ struct Job {
         const size_t a_win = take(sizeof(uint32_t) * (size_t)units() * (size_t)n_slabs() *
                                   (size_t)n_tiles() * (size_t)std::max(1, n_fft));
         const size_t a_dmax = take(16);
-        const size_t a_ud = take(pairs == 1 ? sizeof(int32_t) * (size_t)units() : 0);
+        const size_t a_ud = take(pairs == 1 ? sizeof(int32_t) * (size_t)n_dir : 0);
         if (carve) {
             d_udelta = pairs == 1 ? (int32_t *)(dbuf + a_ud) : nullptr;
             d_dmax = (unsigned long long *)(dbuf + a_dmax);
@@ -300,7 +300,7 @@ int fh_server_s::launch_batch(Slot &slot, std::vector<Job *> &batch)
             t.item_begin = items;
             t.n_items = (int64_t)t.n_slabs * t.n_tiles * j->units();
             if (j->d_udelta) {
-                e = cudaMemsetAsync(j->d_udelta, 0, sizeof(int32_t) * (size_t)j->units(), s);
+                e = cudaMemsetAsync(j->d_udelta, 0, sizeof(int32_t) * (size_t)j->n_dir, s);
                 if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync(pair distances)");
             }
             items += t.n_items;
