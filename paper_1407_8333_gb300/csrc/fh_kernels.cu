@@ -27,7 +27,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr double kTwo32 = 4294967296.0;
-constexpr int kPosFfts = 8;
 constexpr int kPosThreads = 256;
 
 // ---------------------------------------------------------------- a1 + a2
@@ -110,7 +109,7 @@ __device__ __forceinline__ bool integer_position(const PosGrid &G, double f, dou
     return (unsigned)d <= 9u && (uint64_t)(X + G.x_max) <= 2 * (uint64_t)G.x_max;
 }
 
-// The body of one positions block: r = 1 / (1 + v.n) for group `group` of 8 FFTs and
+// The body of one positions block: r = 1 / (1 + v.n) for group `group` of NF FFTs and
 // directions d0 .. d0 + ND - 1 (below n_dir), then the fixed-point position of each
 // of their peaks in each of the directions (a contiguous CSR range, so loads and
 // stores are coalesced; ND directions share a peak's load, its FFT and the
@@ -121,20 +120,20 @@ __device__ __forceinline__ bool integer_position(const PosGrid &G, double f, dou
 // [0, n_peaks] and made non-decreasing within the block, which keeps every
 // access in bounds (a valid CSR is unchanged; an invalid one is flagged by the
 // global CSR pass).
-template <int ND>
+template <int ND, int NF>
 __device__ __forceinline__ void positions_block(
     const double *__restrict__ freq, const int64_t *__restrict__ offsets, bool clamp_offsets,
     const double *__restrict__ v, const double *__restrict__ sky, int32_t n_fft, int64_t n_peaks,
     double f0_min, double kt, double cshift, const PosGrid &G, int64_t *__restrict__ A,
     double *__restrict__ out_r, int32_t *err, int32_t validate, int d0, int n_dir, int group)
 {
-    __shared__ double r_s[ND][kPosFfts];
-    __shared__ int32_t kd_s[ND][kPosFfts];
-    __shared__ int64_t off_s[kPosFfts + 1];
-    const int i0 = group * kPosFfts;
-    const int nf = min(kPosFfts, n_fft - i0);
+    __shared__ double r_s[ND][NF];
+    __shared__ int32_t kd_s[ND][NF];
+    __shared__ int64_t off_s[NF + 1];
+    const int i0 = group * NF;
+    const int nf = min(NF, n_fft - i0);
     const int nd = ND == 1 ? 1 : min(ND, n_dir - d0);
-    const int li = threadIdx.x % kPosFfts, ld = threadIdx.x / kPosFfts;
+    const int li = threadIdx.x % NF, ld = threadIdx.x / NF;
     if (ld < nd && li < nf) {
         const int i = i0 + li, d = d0 + ld;
         const double px = __dmul_rn(v[3 * (int64_t)i + 0], sky[3 * (int64_t)d + 0]);
@@ -332,17 +331,17 @@ __global__ void __launch_bounds__(1024, 1) prep_kernel(const PrepArgs a)
     flush_prep(a, e, amax);
 }
 
-// a1 - a3 in one launch (fh_correct_doppler): grid (1 + ceil(n_fft / 8),
+// a1 - a3 in one launch (fh_correct_doppler): grid (1 + ceil(n_fft / NF),
 // ceil(n_dir / ND)), kPosThreads threads.  Block (0, 0) sanitises the CSR for the later kernels
 // and checks the sky directions; block (x, d), x >= 1, computes the positions
-// of FFTs 8 (x - 1) .. 8 (x - 1) + 7 for direction d (clamping the raw CSR
+// of FFTs NF (x - 1) .. NF x - 1 for ND directions (clamping the raw CSR
 // entries it reads when they still need sanitising, so it does not wait for
 // block (0, 0)), and the blocks of direction 0 also the shift tables and
 // per-FFT checks of their FFTs.
 // Bound by instructions: 64 directions x 26.5 M peaks (900 Hz workload) 13.3 ms with
 // the binary64 operations, at their issue rate; 9.0 ms in integers, a direction
 // per block; 5.8 ms with four.
-template <int ND>
+template <int ND, int NF>
 __global__ void __launch_bounds__(kPosThreads)
 correct_kernel(const PrepArgs a, const double *__restrict__ freq, double f0_min, double cshift,
                const PosGrid G, int64_t *__restrict__ A, double *__restrict__ out_r)
@@ -358,13 +357,14 @@ correct_kernel(const PrepArgs a, const double *__restrict__ freq, double f0_min,
         return;
     }
     const int group = (int)blockIdx.x - 1, d0 = ND * (int)blockIdx.y;
-    if (d0 == 0) {
-        const int i = group * kPosFfts + (int)threadIdx.x;
-        if (threadIdx.x < kPosFfts && i < a.n_fft) fft_tables(a, i, e, amax);
-        if (threadIdx.x < 32) flush_prep(a, e, amax);
+    if (d0 == 0 && threadIdx.x >= kPosThreads - 32) {
+        // (the last warp, beside the first one's Doppler factors)
+        const int k = (int)threadIdx.x - (kPosThreads - 32), i = group * NF + k;
+        if (k < NF && i < a.n_fft) fft_tables(a, i, e, amax);
+        flush_prep(a, e, amax);
     }
     const bool raw = a.offsets_in != nullptr;
-    positions_block<ND>(freq, raw ? a.offsets_in : a.offsets_out, raw, a.v, a.sky, a.n_fft,
+    positions_block<ND, NF>(freq, raw ? a.offsets_in : a.offsets_out, raw, a.v, a.sky, a.n_fft,
                         a.n_peaks, f0_min, a.kt, cshift, G, A, out_r, a.err, a.validate, d0,
                         a.n_dir, group);
 }
@@ -479,7 +479,7 @@ __device__ __forceinline__ void lookup_window(const int64_t *__restrict__ Ad,
 // A warp's 32 entries of a slab are 4 tiles x 8 consecutive FFTs, i.e. four
 // 32-byte runs of the [slab][tile][FFT] table, so each warp writes its own
 // runs and the slab loop has no barrier.
-// grid (ceil(n_fft / 8), units), 256 threads.
+// grid (ceil(n_fft / 8), units, shares of the tile passes), 256 threads.
 constexpr int kWinPad = 1;
 constexpr int kWinMaxM = 3;
 __device__ __forceinline__ int lower_bound_cell(const int32_t *a, int n, int x)
@@ -558,7 +558,7 @@ windows_kernel(const TransformJob J, uint32_t *__restrict__ windows)
     const int64_t *A1 = nd == 2 ? A0 + J.n_peaks : A0;  // the pair's second direction
     // the transform merges into each direction's profile by atomicMax from 0:
     // the blocks of the unit clear it here, a strided slice each
-    for (int di = 0; di < nd; ++di) {
+    for (int di = 0; di < nd && blockIdx.z == 0; ++di) {
         uint64_t *pr = J.profile + (int64_t)(d_first + di) * J.n_f0;
         for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < J.n_f0;
              k += (int64_t)gridDim.x * blockDim.x)
@@ -575,7 +575,8 @@ windows_kernel(const TransformJob J, uint32_t *__restrict__ windows)
         const int ns = ls ? (int)(J.offsets[is + 1] - os) : 0;
         const bool stage = ns + 2 * kWinPad <= kPeaks;
         bool close = false;
-        if (stage || J.dense != nullptr) {
+        const bool first = blockIdx.z == 0;  // (the flags once per FFT)
+        if (stage || (first && J.dense != nullptr)) {
             const int64_t *Aa = A0 + os, *Ab = A1 + os;
             int32_t *c0 = &cell_s[0][warp][kWinPad];
             int32_t *c1 = &cell_s[NR - 1][warp][kWinPad];
@@ -613,9 +614,10 @@ windows_kernel(const TransformJob J, uint32_t *__restrict__ windows)
                 c1[-1 - lane] = INT_MIN;
                 c1[ns + lane] = INT_MAX;
             }
-            if (J.dense != nullptr && __any_sync(kFull, close) && lane == 0) atomicOr(J.dense, 1);
+            if (first && J.dense != nullptr && __any_sync(kFull, close) && lane == 0)
+                atomicOr(J.dense, 1);
         }
-        if (PAIR && nd == 2 && J.unit_delta != nullptr && lane == 0 && ns > 0) {
+        if (PAIR && first && nd == 2 && J.unit_delta != nullptr && lane == 0 && ns > 0) {
             // the pair's largest distance between a peak's two cells: the positions
             // differ by f (r_b - r_a) KT (+ rounding), linear in f, so it is largest
             // at the FFT's first or last peak (ascending frequencies); 2 cells of
@@ -648,7 +650,7 @@ windows_kernel(const TransformJob J, uint32_t *__restrict__ windows)
     // every FFT of the block staged (the usual case): the slab loop reads shared
     // memory only; else the whole block takes the global-memory searches
     const bool all_staged = __syncthreads_and(staged ? 1 : 0) != 0;
-    for (int t0 = 0; t0 < J.n_tiles; t0 += kTiles) {
+    for (int t0 = blockIdx.z * kTiles; t0 < J.n_tiles; t0 += kTiles * gridDim.z) {
         const int nt = min(kTiles, J.n_tiles - t0);
         // the lane's tiles: lower bound = Lc + b0 - K + 1, upper bound = Hc + b0 + Wt
         int blo[M], bhi[M], qa[M], qb[M];
@@ -2057,16 +2059,22 @@ cudaError_t launch_correct(const PrepArgs &a, const double *freq, double f0_min,
 {
     if (a.n_fft <= 0 && !a.offsets_in && !(a.validate && a.n_dir > 0)) return cudaSuccess;
     const double cshift = 0.5 - 0.5 * (double)k_over;
-    const unsigned groups = (unsigned)((std::max(0, a.n_fft) + kPosFfts - 1) / kPosFfts);
     const PosGrid G = make_pos_grid(f0_min, a.kt, k_over);
-    // four directions per block, while that leaves every SM blocks
-    const int32_t n_dir = std::max(1, a.n_dir);
-    if (n_dir >= 4 && (int64_t)groups * ((n_dir + 3) / 4) >= 1024) {
-        dim3 grid(1 + groups, (n_dir + 3) / 4);
-        correct_kernel<4><<<grid, kPosThreads, 0, s>>>(a, freq, f0_min, cshift, G, A, out_r);
+    // Four directions per block while that leaves every SM blocks; 8 FFTs, or 2 where
+    // even that leaves few, so that a block's chain of loads is short (one direction
+    // of 3164 FFTs: 19.5 -> 15.3 us, of 200: 8.9 -> 6.2; but 3 x 5003 FFTs of 83 peaks,
+    // 1881 blocks of 8: 14.5 us, 21.5 with 2).
+    const int32_t n_dir = std::max(1, a.n_dir), n = std::max(0, a.n_fft);
+    const int64_t g8 = (n + 7) / 8;
+    if (n_dir >= 4 && g8 * ((n_dir + 3) / 4) >= 1024) {
+        dim3 grid(1 + g8, (n_dir + 3) / 4);
+        correct_kernel<4, 8><<<grid, kPosThreads, 0, s>>>(a, freq, f0_min, cshift, G, A, out_r);
+    } else if (g8 * n_dir >= 600) {
+        dim3 grid(1 + g8, n_dir);
+        correct_kernel<1, 8><<<grid, kPosThreads, 0, s>>>(a, freq, f0_min, cshift, G, A, out_r);
     } else {
-        dim3 grid(1 + groups, n_dir);
-        correct_kernel<1><<<grid, kPosThreads, 0, s>>>(a, freq, f0_min, cshift, G, A, out_r);
+        dim3 grid(1 + (n + 1) / 2, n_dir);
+        correct_kernel<1, 2><<<grid, kPosThreads, 0, s>>>(a, freq, f0_min, cshift, G, A, out_r);
     }
     return cudaGetLastError();
 }
@@ -2203,8 +2211,14 @@ cudaError_t launch_windows(const TransformJob &job, uint32_t *windows, cudaStrea
 {
     if (job.n_fft <= 0 || job.n_dir <= 0) return cudaSuccess;
     dim3 grid((job.n_fft + 7) / 8, job.dir_pairs ? (job.n_dir + 1) / 2 : job.n_dir);
-    // tiles per lane and pass: enough for all tiles in one pass, at most kWinMaxM
-    const int m = std::min(kWinMaxM, std::max(1, (job.n_tiles + 31) / 32));
+    // tiles per lane and pass: enough for all tiles in one pass, at most kWinMaxM; where
+    // there are too few blocks to fill the SMs, one tile per lane and the passes side by
+    // side, each staging the peaks again (200 FFTs x 72 tiles: 7.1 -> 5.0 us; 3164 FFTs x
+    // 82 tiles x 19 slabs: 30.3 -> 28.4 us)
+    const int passes = std::max(1, (job.n_tiles + 31) / 32);
+    const bool few = (int64_t)grid.x * grid.y < 600;
+    const int m = few ? 1 : std::min(kWinMaxM, passes);
+    if (few) grid.z = std::min(passes, 64);
     auto go = [&](auto pair_tag) {
         constexpr bool P = decltype(pair_tag)::value;
         auto *k = m == 1   ? windows_kernel<1, P>

@@ -165,3 +165,13 @@ def test_positions_in_integers(fh, f0, t_fft, k_over):
     near = np.abs(x) < 2.0 ** 28   # beyond that a call is refused
     want = np.floor(x * 2.0 ** 32)[near].astype(np.int64)
     assert near.sum() > 1000 and np.array_equal(got[near], want)
+
+
+# correction blocks of 2 and of 8 FFTs (4800 FFT-directions), of one and of four
+# directions, and window passes side by side (up to 600 blocks of 8 FFTs) or not
+@pytest.mark.parametrize("n_fft, n_dir", [(1, 1), (2, 1), (9, 3), (1599, 3), (1601, 3), (2049, 7),
+                                          (17, 5)])
+def test_correction_and_window_blocks(fh, n_fft, n_dir):
+    inp, pp = synth.random_case(500 + n_fft, n_fft=n_fft, n_bins=110, n_fdot=4, n_dir=n_dir, p=0.05,
+                                vmax=2e-6)
+    check(fh, inp, pp, tile_cells=32)
