@@ -181,9 +181,9 @@ range_kernel(CandSet a, CandSet b, double reach_f, double reach_d, int32_t max_c
 #pragma unroll
     for (int q = 0; q < kStats; ++q) st[q] = 0ull;
     bool bad = false;
-    const int n = a.n + b.n;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const bool in_b = k >= a.n;
+    const unsigned n = (unsigned)a.n + (unsigned)b.n;  // at most 2^31
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const bool in_b = k >= (unsigned)a.n;
         const fh_cand_params x = in_b ? b.c[k - a.n] : a.c[k];
         bad = bad || !cand_ok(x);
         if (in_b) {
@@ -192,7 +192,7 @@ range_kernel(CandSet a, CandSet b, double reach_f, double reach_d, int32_t max_c
             st[kMaxF] = max(st[kMaxF], f);
             st[kMinD] = max(st[kMinD], ~d);
             st[kMaxD] = max(st[kMaxD], d);
-            if (label) label[k - a.n] = k - a.n;
+            if (label) label[k - a.n] = (int32_t)(k - a.n);
         }
         st[kWidF] = max(st[kWidF], okey(x.df));
         st[kWidD] = max(st[kWidD], okey(x.dfdot));
@@ -242,9 +242,9 @@ cell_count_kernel(CandSet a, CandSet b, const Head *hp, int32_t max_cells, int32
                   int2 *at)
 {
     const Head h = *hp;
-    const int n = a.n + b.n;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const bool in_b = k >= a.n;
+    const unsigned n = (unsigned)a.n + (unsigned)b.n;  // at most 2^31
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const bool in_b = k >= (unsigned)a.n;
         const fh_cand_params *p = in_b ? b.c + (k - a.n) : a.c + k;
         const double2 q = *reinterpret_cast<const double2 *>(&p->f);  // f, fdot
         const CandSet &s = in_b ? b : a;
@@ -267,14 +267,14 @@ cell_scatter_kernel(CandSet a, CandSet b, const Head *hp, int32_t max_cells, con
                     const int2 *at, Sorted o)
 {
     const double f0 = hp->f0, d0 = hp->d0;
-    const int n = a.n + b.n;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const bool in_b = k >= a.n;
-        const int i = in_b ? k - a.n : k;
+    const unsigned n = (unsigned)a.n + (unsigned)b.n;  // at most 2^31
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const bool in_b = k >= (unsigned)a.n;
+        const int i = (int)(in_b ? k - a.n : k);
         const int2 w = at[k];
         if (w.x < 0) continue;
         const fh_cand_params x = in_b ? b.c[i] : a.c[i];
-        const int t = start[(in_b ? max_cells : 0) + w.x] + w.y;
+        const unsigned t = (unsigned)start[(in_b ? max_cells : 0) + w.x] + (unsigned)w.y;
         o.index[t] = i;
         o.cell[t] = w.x;
         o.x[t] = make_float4((float)x.lam, (float)x.beta,
@@ -288,7 +288,7 @@ cell_scatter_kernel(CandSet a, CandSet b, const Head *hp, int32_t max_cells, con
 // The cells around a candidate's cell with frequency index shifted by k, as one
 // range [lo, hi) of sorted positions (empty where the index is off the grid).
 __device__ __forceinline__ void cell_range(const int32_t *start, int32_t cell, int32_t nbf,
-                                           int32_t nbd, int k, int &lo, int &hi)
+                                           int32_t nbd, int k, unsigned &lo, unsigned &hi)
 {
     const int i = cell / nbd + k, j = cell % nbd;
     if (i < 0 || i >= nbf) {
@@ -360,53 +360,96 @@ __device__ __forceinline__ void uf_union(int32_t *parent, int32_t a, int32_t b, 
     atomicOr(err, kErrRange);
 }
 
-// Threads take the candidates in sorted order; each looks at those behind it: the
-// rest of its own and the next spin-down cell, and the three cells of the next
-// frequency index.  So every pair is looked at once, neighbouring lanes read
-// neighbouring (or the same) records, and the distance is formed in binary32 with
-// its error bound; only pairs whose distance lies within the bound of d_max
-// take the binary64 divisions and square root (GB300's binary64 rate is a small
-// fraction of its binary32 one).  10^5 candidates of one 1 Hz band: 4.0 -> 0.14 ms
-// against buckets of frequency alone with the binary64 records gathered per
-// pair (117 -> 7 million pairs looked at); 10^6 over 10 Hz: 25.4 -> 0.69 ms.
-__global__ void __launch_bounds__(256)
+// The scan of clustering and coincidences.  Four lanes share a candidate and step
+// through its ranges of sorted positions (neighbouring lanes read neighbouring
+// records); pairs that the rejects leave go to the warp's list, and 32 of them at a
+// time are decided, a lane each.  (Decided where they are found, one lane in four was
+// busy and the scan of 10^5 candidates took 144 us, link, and 98 us, coincidences;
+// a thread per candidate also left three quarters of the warps empty.)
+//   range(t, k, lo, hi): the k-th of `ranges` ranges of position t
+//   decide(t, u): what to do with the pair of positions t and u
+constexpr int kScanLanes = 4;
+constexpr int kPairThreads = 256;
+constexpr int kPairCands = kPairThreads / kScanLanes;  // candidates of a block
+template <typename R, typename D>
+__device__ __forceinline__ void scan_pairs(const Sorted &o, unsigned n, int ranges, const float4 &hi_lim,
+                                           const float4 &tol, R &&range, D &&decide)
+{
+    __shared__ uint2 list_s[kPairThreads / 32][64];
+    uint2 *list = list_s[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31, sub = lane % kScanLanes;
+    const unsigned lt = (1u << lane) - 1u;
+    int listed = 0;
+    const unsigned t = blockIdx.x * kPairCands + threadIdx.x / kScanLanes;
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 xa = t < n ? o.x[t] : none, ha = t < n ? o.h[t] : none;
+    for (int k = 0; k < ranges; ++k) {
+        unsigned lo = 0, hi = 0;
+        if (t < n) range(t, k, lo, hi);
+        for (unsigned u = lo + sub; __any_sync(kFull, u < hi); u += kScanLanes) {
+            bool near = false;
+            if (u < hi)
+                near = !far_apart(apart(xa, o.x[u]), wid(ha, o.h[u]), hi_lim, tol);
+            const unsigned m = __ballot_sync(kFull, near);
+            if (m == 0) continue;
+            if (near) list[listed + __popc(m & lt)] = make_uint2(t, u);
+            listed += __popc(m);
+            if (listed >= 32) {
+                __syncwarp();
+                listed -= 32;
+                const uint2 q = list[listed + lane];
+                decide(q.x, q.y);
+                __syncwarp();
+            }
+        }
+    }
+    __syncwarp();
+    if (lane < listed) {
+        const uint2 q = list[lane];
+        decide(q.x, q.y);
+    }
+}
+
+// Every pair is looked at once, from its first candidate in the sorted order: the rest
+// of that one's own and the next spin-down cell, and the three cells of the next
+// frequency index.  The distance is formed in binary32 with its error bound; only pairs
+// whose distance lies within the bound of d_max take the binary64 divisions and
+// square root (GB300's binary64 rate is a small fraction of its binary32 one).
+// 10^5 candidates of one 1 Hz band: 4.0 ms with buckets of frequency alone and the
+// binary64 records gathered per pair (117 million pairs looked at, now 7), 59 us
+// now; 10^6 over 10 Hz: 25.4 -> 0.41 ms.
+__global__ void __launch_bounds__(kPairThreads)
 link_kernel(const fh_cand_params *c, int32_t max_cells, double d_max, Limits lim, const Head *hp,
             const int32_t *start, Sorted o, int32_t *parent, int32_t *err)
 {
     const int32_t nbf = hp->nbf, nbd = hp->nbd;
-    const int n = start[max_cells];  // placed candidates
     const float4 tol = hp->tol;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        const float4 xa = o.x[t], ha = o.h[t];
-        const int32_t cell = o.cell[t];
-        for (int k = 0; k < 2; ++k) {
-            int lo, hi;
-            cell_range(start, cell, nbf, nbd, k, lo, hi);
+    scan_pairs(
+        o, (unsigned)start[max_cells], 2, lim.hi, tol,
+        [&](unsigned t, int k, unsigned &lo, unsigned &hi) {
+            cell_range(start, o.cell[t], nbf, nbd, k, lo, hi);
             if (k == 0) lo = t + 1;
-            for (int u = lo; u < hi; ++u) {
-                const float4 d = apart(xa, o.x[u]), w = wid(ha, o.h[u]);
-                if (far_apart(d, w, lim.hi, tol)) continue;
-                bool in = false, sure = false;
-                if (!lim.exact && ordinary(d, w)) {
-                    const float ax = fabsf(d.x);
-                    const float p0 = (ax + tol.x) / w.x, p1 = (d.y + tol.y) / w.y,
-                                p2 = (d.z + tol.z) / w.z, p3 = (d.w + tol.w) / w.w;
-                    const float m0 = fmaxf(ax - tol.x, 0.f) / w.x,
-                                m1 = fmaxf(d.y - tol.y, 0.f) / w.y,
-                                m2 = fmaxf(d.z - tol.z, 0.f) / w.z,
-                                m3 = fmaxf(d.w - tol.w, 0.f) / w.w;
-                    in = p0 * p0 + p1 * p1 + p2 * p2 + p3 * p3 < lim.d2_lo;
-                    sure = in || m0 * m0 + m1 * m1 + m2 * m2 + m3 * m3 > lim.d2_hi;
-                }
-                const int32_t i = o.index[t], j = o.index[u];
-                if (!sure) {
-                    const fh_cand_params a = c[i], b = c[j];
-                    in = norm_distance(a, b, a.f, b.f) <= d_max;
-                }
-                if (in) uf_union(parent, i, j, err);
+        },
+        [&](unsigned t, unsigned u) {
+            const float4 d = apart(o.x[t], o.x[u]), w = wid(o.h[t], o.h[u]);
+            bool in = false, sure = false;
+            if (!lim.exact && ordinary(d, w)) {
+                const float ax = fabsf(d.x);
+                const float p0 = (ax + tol.x) / w.x, p1 = (d.y + tol.y) / w.y,
+                            p2 = (d.z + tol.z) / w.z, p3 = (d.w + tol.w) / w.w;
+                const float m0 = fmaxf(ax - tol.x, 0.f) / w.x, m1 = fmaxf(d.y - tol.y, 0.f) / w.y,
+                            m2 = fmaxf(d.z - tol.z, 0.f) / w.z, m3 = fmaxf(d.w - tol.w, 0.f) / w.w;
+                in = p0 * p0 + p1 * p1 + p2 * p2 + p3 * p3 < lim.d2_lo;
+                sure = in || m0 * m0 + m1 * m1 + m2 * m2 + m3 * m3 > lim.d2_hi;
             }
-        }
-    }
+            if (sure && !in) return;
+            const int32_t i = o.index[t], j = o.index[u];
+            if (!sure) {
+                const fh_cand_params a = c[i], b = c[j];
+                in = norm_distance(a, b, a.f, b.f) <= d_max;
+            }
+            if (in) uf_union(parent, i, j, err);
+        });
 }
 
 // every candidate's root, in place (roots only ever move to ancestors, so a
@@ -429,7 +472,7 @@ __global__ void __launch_bounds__(256) finish_labels_kernel(int32_t *label, int3
 }
 
 // ---------------------------------------------------------------- coincidences
-constexpr int kKeep = 4;  // partners of a candidate kept from the count for the write
+constexpr int kKeep = 8;  // partners of a candidate kept from the count for the write
 struct CoinArgs {
     CandSet s1, s2;
     double w[4];          // windows: lam, beta, f, fdot
@@ -451,45 +494,52 @@ __device__ bool coincide(const CoinArgs &a, int32_t i, int32_t j)
            bins_apart(x.lam, y.lam, x.dlam, y.dlam, true) <= a.w[0];
 }
 
-// the partners of set 1's candidate at sorted position t: f(index in set 2)
-template <typename F>
-__device__ __forceinline__ void for_partners(const CoinArgs &a, int t, F &&f)
+// whether the records at sorted positions t (set 1) and u coincide, after the rejects:
+// clearly inside every window in binary32, else the exact test
+__device__ __forceinline__ bool inside(const CoinArgs &a, unsigned t, unsigned u, const float4 &tol)
+{
+    const float4 d = apart(a.o.x[t], a.o.x[u]), w = wid(a.o.h[t], a.o.h[u]);
+    const bool in = !a.lim.exact && ordinary(d, w) && d.x + tol.x < a.lim.lo.x * w.x &&
+                    d.y + tol.y < a.lim.lo.y * w.y && d.z + tol.z < a.lim.lo.z * w.z &&
+                    d.w + tol.w < a.lim.lo.w * w.w;
+    return in || coincide(a, a.o.index[t], a.o.index[u]);
+}
+
+// Partners of every set-1 candidate, counted, the first kKeep found kept (in any
+// order; the write sorts them).  10^5 x 10^5 candidates of one 1 Hz band: 1.20 ms -> 55 us
+// for the count and 1.45 ms -> 36 us for the write; 10^6 x 10^6 over 10 Hz: 9.7 -> 0.35 ms
+// and 11.4 ms -> 61 us.  cnt1 starts at zero.
+__global__ void __launch_bounds__(kPairThreads) coin_count_kernel(const CoinArgs a, int32_t *cnt1,
+                                                                  int32_t *cnt2)
 {
     const int32_t nbf = a.h->nbf, nbd = a.h->nbd;
     const float4 tol = a.h->tol;
-    const float4 xa = a.o.x[t], ha = a.o.h[t];
-    const int32_t cell = a.o.cell[t], i = a.o.index[t];
-    for (int k = -1; k <= 1; ++k) {
-        int lo, hi;
-        cell_range(a.start + a.max_cells, cell, nbf, nbd, k, lo, hi);
-        for (int u = lo; u < hi; ++u) {
-            const float4 d = apart(xa, a.o.x[u]), w = wid(ha, a.o.h[u]);
-            if (far_apart(d, w, a.lim.hi, tol)) continue;
-            // clearly inside every window in binary32, else the exact test
-            const bool in = !a.lim.exact && ordinary(d, w) && d.x + tol.x < a.lim.lo.x * w.x &&
-                            d.y + tol.y < a.lim.lo.y * w.y && d.z + tol.z < a.lim.lo.z * w.z &&
-                            d.w + tol.w < a.lim.lo.w * w.w;
+    scan_pairs(
+        a.o, (unsigned)a.start[a.max_cells], 3, a.lim.hi, tol,
+        [&](unsigned t, int k, unsigned &lo, unsigned &hi) {
+            cell_range(a.start + a.max_cells, a.o.cell[t], nbf, nbd, k - 1, lo, hi);
+        },
+        [&](unsigned t, unsigned u) {
+            if (!inside(a, t, u, tol)) return;
             const int32_t j = a.o.index[u];
-            if (in || coincide(a, i, j)) f(j);
-        }
-    }
-}
-
-// 10^5 x 10^5 candidates of one 1 Hz band: 1.20 -> 0.10 ms for the count and 1.45 ->
-// 0.05 ms for the write (which reads the kept partners instead of searching
-// again); 10^6 x 10^6 over 10 Hz: 9.7 -> 0.56 ms and 11.4 -> 0.09 ms.
-__global__ void __launch_bounds__(256) coin_count_kernel(const CoinArgs a, int32_t *cnt1,
-                                                         int32_t *cnt2)
-{
-    const int n = a.start[a.max_cells];  // placed candidates of set 1
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-        int c = 0;
-        for_partners(a, t, [&](int32_t j) {
+            const int c = atomicAdd(cnt1 + a.o.index[t], 1);
             if (c < kKeep) a.keep[(int64_t)t * kKeep + c] = j;
-            ++c;
             if (cnt2) atomicAdd(cnt2 + j, 1);
         });
-        cnt1[a.o.index[t]] = c;
+}
+
+// the partners of set 1's candidate at sorted position t, one thread: f(index in set 2)
+template <typename F>
+__device__ __forceinline__ void for_partners(const CoinArgs &a, unsigned t, F &&f)
+{
+    const float4 tol = a.h->tol;
+    for (int k = -1; k <= 1; ++k) {
+        unsigned lo, hi;
+        cell_range(a.start + a.max_cells, a.o.cell[t], a.h->nbf, a.h->nbd, k, lo, hi);
+        for (unsigned u = lo; u < hi; ++u)
+            if (!far_apart(apart(a.o.x[t], a.o.x[u]), wid(a.o.h[t], a.o.h[u]), a.lim.hi, tol) &&
+                inside(a, t, u, tol))
+                f(a.o.index[u]);
     }
 }
 
@@ -636,6 +686,8 @@ __global__ void cc_write_kernel(const CCArgs a, const int64_t *off, int64_t capa
 
 int grid_for(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 4096)); }
 
+unsigned pair_grid(int64_t n) { return (unsigned)((n + kPairCands - 1) / kPairCands); }
+
 // reach per parameter -> binary32 bounds (see Limits)
 Limits make_limits(const double *reach, double d_max)
 {
@@ -734,9 +786,9 @@ int fh_cluster(const fh_cand_params *cands, int32_t n, double d_max, int32_t *la
     cudaError_t e = build_cells(none, set, d_max, d_max, label, g, sc, s);
     if (e == cudaSuccess) {
         // (with no set a the starts of the second half are the set's own)
-        link_kernel<<<grid_for(n), 256, 0, s>>>(cands, g.max_cells, d_max,
-                                                make_limits(reach, d_max), g.head,
-                                                g.start + g.max_cells, g.o, label, &g.head->err);
+        link_kernel<<<pair_grid(n), kPairThreads, 0, s>>>(
+            cands, g.max_cells, d_max, make_limits(reach, d_max), g.head, g.start + g.max_cells,
+            g.o, label, &g.head->err);
         finish_labels_kernel<<<grid_for(n), 256, 0, s>>>(label, n, g.head);
         e = cudaGetLastError();
     }
@@ -793,7 +845,7 @@ int fh_coincidences(const fh_cand_params *c1, int32_t n1, double t_ref1,
     a.start = g.start;
     a.max_cells = g.max_cells;
     a.o = g.o;
-    coin_count_kernel<<<grid_for(n1), 256, 0, s>>>(a, cnt1, n_match2);
+    coin_count_kernel<<<pair_grid(n1), kPairThreads, 0, s>>>(a, cnt1, n_match2);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = scan_exclusive(cnt1, n1, off, sc, s);
     if (e == cudaSuccess && capacity > 0) {

@@ -209,6 +209,19 @@ def test_scan_tiles(fh, co, n):
     check_coinc(fh, co, a, a[:300], 0.0, 0.0, 0.0, (2, 2, 2, 2))
 
 
+@pytest.mark.parametrize("n", [1, 8, 63, 64, 65, 257])
+@pytest.mark.parametrize("shape", [(1, 1, 1, 1), (2, 1, 3, 2), (40, 20, 30, 10)])
+def test_lists_of_pairs(fh, co, n, shape):
+    """Set sizes at the edges of a block's and a warp's candidates, with all,
+    many or few pairs left to decide, and more and fewer partners than the
+    count keeps."""
+    a = synth.candidates_on_grid(54, 1, n, shape)
+    b = synth.candidates_on_grid(54, 2, 90, shape)
+    check_cluster(fh, co, a, 1.0)
+    check_coinc(fh, co, a, b, 0.0, 0.0, 0.0, (1, 1, 1, 1))
+    check_coinc(fh, co, b, a, 0.0, 0.0, 0.0, (0, 1, 1, 2))
+
+
 def test_scratch_shared_by_threads_and_streams(fh):
     """Calls of several threads, each on its own stream, share the library's
     scratch pool: every result is that of a call alone; the last plan's
