@@ -47,6 +47,7 @@ struct RefineArgs {
     int32_t dirs_per, rows_per;        // directions and rows of one block's histogram
     int32_t ffts_per;                  // FFTs of one block
     double f0_min, kt, t_ref, step_ref, cshift;
+    double half_inv_kt;                // 0.5 / kt
     int32_t *starts;  // [cand][direction][row][3 K] of the launch: stripe starts, zeroed
     int32_t *err;
 };
@@ -66,12 +67,17 @@ constexpr int kRefList = 64;  // (FFT, peak) entries a warp collects before it p
 // a bound of its error; the margin of a cell is far above the other roundings.
 // The exact position of each peak of the range then decides.
 //
+// The binary64 pipe (1.68 results per SM and clock) bounds the kernel, so the ranges
+// leave it what they must: the shifts in integers, the sky rounded to binary32 once
+// per block, no division, the searches on the frequencies' bits.  50 candidates x 9
+// directions on 3164 FFTs: 67 us with all of that in binary64, 43 us now.
+//
 // grid (candidates, shares of ffts_per FFTs, (direction, row) groups of one
 // histogram).  A warp takes 32 FFTs at a time (lane <-> FFT), lists their peaks, and
 // places list x directions, a lane each.
 __global__ void __launch_bounds__(kRefThreads) refine_kernel(const RefineArgs a)
 {
-    extern __shared__ int32_t hist[];  // [direction][row][3 K]
+    extern __shared__ int32_t hist[];  // [direction][row][3 K], then the sky
     __shared__ int32_t list_fft[kRefThreads / 32][kRefList];
     __shared__ int64_t list_peak[kRefThreads / 32][kRefList];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -83,10 +89,12 @@ __global__ void __launch_bounds__(kRefThreads) refine_kernel(const RefineArgs a)
     const int K = a.k_over, E = 3 * K;
     const int words = nd * nr * E;
     for (int w = threadIdx.x; w < words; w += kRefThreads) hist[w] = 0;
-    __syncthreads();
     const int64_t lo_cell = (int64_t)a.cell[c] - K;
     const int64_t j_off = (int64_t)a.row[c] - 2;
     const double *sky = a.sky + 3 * ((int64_t)c * a.n_ref + a.dir0);
+    float *sky32 = reinterpret_cast<float *>(hist + a.dirs_per * a.rows_per * E);
+    for (int w = threadIdx.x; w < 3 * nd; w += kRefThreads) sky32[w] = (float)sky[3 * d0 + w];
+    __syncthreads();
     int32_t ev = 0;
     const int f_begin = blockIdx.y * a.ffts_per;
     const int f_end = min(a.n_fft, f_begin + a.ffts_per);
@@ -102,13 +110,13 @@ __global__ void __launch_bounds__(kRefThreads) refine_kernel(const RefineArgs a)
             const double py = __dmul_rn(a.v[3 * (int64_t)i + 1], n3[1]);
             const double pz = __dmul_rn(a.v[3 * (int64_t)i + 2], n3[2]);
             const double den = __dadd_rn(1.0, __dadd_rn(__dadd_rn(px, py), pz));
-            const double u = __dmul_rn(a.freq[list_peak[warp][e]], __ddiv_rn(1.0, den));
+            const double u = __dmul_rn(a.freq[list_peak[warp][e]], __drcp_rn(den));
             const double y = __dmul_rn(__dsub_rn(u, a.f0_min), a.kt);
             const double x = __dadd_rn(y, a.cshift);
             // |x| < 2^28 exactly when the biased exponent is below 1023 + 28
             if (((__double_as_longlong(x) >> 52) & 0x7FF) >= 1051) ev |= kErrRange;
             const double cc = __dmul_rn(__dsub_rn(a.t[i], a.t_ref), a.kt);
-            const int64_t dr = (int64_t)floor(__dmul_rn(__dmul_rn(a.step_ref, cc), 4294967296.0));
+            const int64_t dr = floor_times_2p32(__dmul_rn(a.step_ref, cc));
             // start of the stripe on row r0, its cell 0 at start 1 - K
             int64_t X = floor_times_2p32(x) - (a.S0[i] + j_off * a.D[i]) -
                         (int64_t)r0 * dr + ((int64_t)(K - 1) - lo_cell) * 4294967296LL;
@@ -130,43 +138,51 @@ __global__ void __launch_bounds__(kRefThreads) refine_kernel(const RefineArgs a)
             // the refined drift and its range check, as the shift tables form them
             const double cc = __dmul_rn(__dsub_rn(a.t[i], a.t_ref), a.kt);
             if (!(fabs(cc) * absmax < (double)kFixedLimit)) ev |= kErrRange;
-            const int64_t dr = (int64_t)floor(__dmul_rn(__dmul_rn(a.step_ref, cc), 4294967296.0));
+            const int64_t dr = floor_times_2p32(__dmul_rn(a.step_ref, cc));
             const int64_t s0r = a.S0[i] + j_off * a.D[i] + lo_cell * 4294967296LL;
             const int64_t last = (int64_t)(a.n_rows - 1) * dr;
-            const double xmin = ((double)s0r + (double)(last < 0 ? last : 0)) / 4294967296.0;
-            const double xmax = ((double)s0r + (double)(last > 0 ? last : 0)) / 4294967296.0;
-            const double c_off = 0.5 - 0.5 * (double)K;
-            const double u_lo = a.f0_min + (xmin + (double)(1 - K) - 1.0 - c_off) / a.kt;
-            const double u_hi = a.f0_min + (xmax + (double)(2 * K + 1) + 1.0 - c_off) / a.kt;
+            // the band's two ends in half cells from f0_min: the cells below and above
+            // the extreme shifts, (1 - K) - 1 and (2 K + 1) + 1, less 0.5 - 0.5 K
+            const int32_t x_lo = (int32_t)((s0r + (last < 0 ? last : 0)) >> 32);
+            const int32_t x_hi = (int32_t)((s0r + (last > 0 ? last : 0)) >> 32) + 1;
+            const double u_lo = __fma_rn((double)(2 * x_lo - K - 1), a.half_inv_kt, a.f0_min);
+            const double u_hi = __fma_rn((double)(2 * x_hi + 5 * K + 3), a.half_inv_kt, a.f0_min);
             const float vx = (float)a.v[3 * (int64_t)i], vy = (float)a.v[3 * (int64_t)i + 1],
                         vz = (float)a.v[3 * (int64_t)i + 2];
             float lo32 = 0.f, hi32 = 0.f;
-            const double *n = sky + 3 * d0;
-            for (int d = 0; d < nd; ++d, n += 3) {
-                const float vn = vx * (float)n[0] + vy * (float)n[1] + vz * (float)n[2];
+            for (int d = 0; d < nd; ++d) {
+                const float vn =
+                    vx * sky32[3 * d] + vy * sky32[3 * d + 1] + vz * sky32[3 * d + 2];
                 lo32 = d ? fminf(lo32, vn) : vn;
                 hi32 = d ? fmaxf(hi32, vn) : vn;
             }
             // the sum of three products of rounded factors is off by less than
             // 4 x 2^-23 of the sum of their magnitudes (|n| <= 1.000001)
             const float wide = 5e-7f * (fabsf(vx) + fabsf(vy) + fabsf(vz)) + 1e-37f;
-            const double vn_lo = (double)(lo32 - wide), vn_hi = (double)(hi32 + wide);
-            const double f_lo = fmin(fmin(u_lo * (1.0 + vn_lo), u_lo * (1.0 + vn_hi)),
-                                     fmin(u_hi * (1.0 + vn_lo), u_hi * (1.0 + vn_hi)));
-            const double f_hi = fmax(fmax(u_lo * (1.0 + vn_lo), u_lo * (1.0 + vn_hi)),
-                                     fmax(u_hi * (1.0 + vn_lo), u_hi * (1.0 + vn_hi)));
+            const double g_lo = 1.0 + (double)(lo32 - wide), g_hi = 1.0 + (double)(hi32 + wide);
+            double f_lo, f_hi;
+            if (__double2hiint(u_lo) > 0 && __double2hiint(g_lo) > 0) {  // all positive
+                f_lo = u_lo * g_lo;
+                f_hi = u_hi * g_hi;
+            } else {
+                f_lo = fmin(fmin(u_lo * g_lo, u_lo * g_hi), fmin(u_hi * g_lo, u_hi * g_hi));
+                f_hi = fmax(fmax(u_lo * g_lo, u_lo * g_hi), fmax(u_hi * g_lo, u_hi * g_hi));
+            }
+            // (frequencies are positive: their bits order as they do)
+            const long long b_lo = __double_as_longlong(f_lo), b_hi = __double_as_longlong(f_hi);
+            const long long *fb = reinterpret_cast<const long long *>(a.freq);
             p = a.offsets[i];
             p_end = a.offsets[i + 1];
             int64_t b = p_end;
             while (p < b) {  // first peak with f >= f_lo
                 const int64_t m = (p + b) >> 1;
-                if (a.freq[m] < f_lo) p = m + 1; else b = m;
+                if (fb[m] < b_lo) p = m + 1; else b = m;
             }
             int64_t e = p;
             b = p_end;
             while (e < b) {  // first peak with f > f_hi
                 const int64_t m = (e + b) >> 1;
-                if (a.freq[m] <= f_hi) e = m + 1; else b = m;
+                if (fb[m] <= b_hi) e = m + 1; else b = m;
             }
             p_end = e;
         }
@@ -347,7 +363,7 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
     const int32_t dir_batch = (int32_t)std::max<int64_t>(
         1, std::min<int64_t>({n_ref, most / per_dir, 65535 / row_groups}));
     ra.dirs_per = (int32_t)std::max<int64_t>(
-        1, std::min<int64_t>(dir_batch, room / ((int64_t)ra.rows_per * E)));
+        1, std::min<int64_t>(dir_batch, room / ((int64_t)ra.rows_per * E + 3)));  // + its sky
     const int32_t cand_batch = (int32_t)std::max<int64_t>(
         1, std::min<int64_t>(n_cand, most / (per_dir * dir_batch)));
     const size_t n_starts = (size_t)cand_batch * dir_batch * per_dir;
@@ -419,7 +435,7 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
             (size_t)max_optin_smem(dev))
             return cuda_error(cudaErrorInvalidValue, "refined map in shared memory");
     }
-    const size_t smem = 4 * (size_t)ra.dirs_per * ra.rows_per * E;
+    const size_t smem = 4 * (size_t)ra.dirs_per * ((size_t)ra.rows_per * E + 3);
     // shares of the FFTs: two waves of four blocks per SM, at least a block's 256 each
     const int64_t blocks = (int64_t)std::min(n_cand, cand_batch) * row_groups *
                            ((dir_batch + ra.dirs_per - 1) / ra.dirs_per);
@@ -444,6 +460,7 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
     ra.t_ref = d.t_ref;
     ra.step_ref = step_ref;
     ra.cshift = 0.5 - 0.5 * (double)K;
+    ra.half_inv_kt = 0.5 / kt;
     ra.starts = starts;
     ra.err = err;
     PickArgs pk{};
