@@ -222,6 +222,35 @@ def test_lists_of_pairs(fh, co, n, shape):
     check_coinc(fh, co, b, a, 0.0, 0.0, 0.0, (0, 1, 1, 2))
 
 
+@pytest.mark.parametrize("n", [7, 8, 9, 8191, 8200])
+@pytest.mark.parametrize("skip", [0, 1, 3])
+def test_counts_of_any_alignment(fh, co, n, skip):
+    """The scan moves 16 bytes at a time where its arrays start on 16: a
+    caller's partner counts may start on any 4."""
+    import ctypes
+
+    import torch
+    a = synth.candidate_set(55, 1, n, clusters=3, cluster_size=4)
+    b = synth.candidate_set(55, 2, 200, clusters=3, cluster_size=4)
+    win = (2, 2, 2, 2)
+    want, w1, _ = co.coincidences(a, b, 0.0, 0.0, 0.0, win)
+    m1 = torch.full((n + 8,), -7, dtype=torch.int32, device="cuda")
+    pairs = torch.empty((max(1, len(want)), 2), dtype=torch.int32, device="cuda")
+    da, db = dev(a), dev(b)
+    w = (ctypes.c_double * 4)(*win)
+    k = ctypes.c_int64(0)
+    rc = fh.load().fh_coincidences(
+        ctypes.c_void_p(da.data_ptr()), n, 0.0, ctypes.c_void_p(db.data_ptr()), 200, 0.0, 0.0,
+        ctypes.cast(w, ctypes.c_void_p), ctypes.c_void_p(pairs.data_ptr()), pairs.shape[0],
+        ctypes.byref(k), ctypes.c_void_p(m1.data_ptr() + 4 * skip), None,
+        ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == 0 and k.value == len(want)
+    got = m1.cpu().numpy()
+    assert np.array_equal(got[skip:skip + n], w1)
+    assert (got[:skip] == -7).all() and (got[skip + n:] == -7).all()
+    assert np.array_equal(pairs.cpu().numpy()[:len(want)], want.reshape(-1, 2))
+
+
 def test_scratch_shared_by_threads_and_streams(fh):
     """Calls of several threads, each on its own stream, share the library's
     scratch pool: every result is that of a call alone; the last plan's
