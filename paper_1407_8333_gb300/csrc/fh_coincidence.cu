@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(kRangeThreads)
 range_kernel(CandSet a, CandSet b, double reach_f, double reach_d, int32_t max_cells, Head *h,
              int32_t *label)
 {
+    let_next_start();
     unsigned long long st[kStats];
 #pragma unroll
     for (int q = 0; q < kStats; ++q) st[q] = 0ull;
@@ -262,6 +263,8 @@ __global__ void __launch_bounds__(256)
 cell_count_kernel(CandSet a, CandSet b, const Head *hp, int32_t max_cells, int32_t *cnt,
                   int2 *at)
 {
+    let_next_start();
+    wait_for_previous();
     const Head h = *hp;
     const unsigned n = (unsigned)a.n + (unsigned)b.n;  // at most 2^31
     for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -292,6 +295,8 @@ __global__ void __launch_bounds__(256)
 cell_scatter_kernel(CandSet a, CandSet b, const Head *hp, int32_t max_cells, const int32_t *start,
                     const int2 *at, Sorted o)
 {
+    let_next_start();
+    wait_for_previous();
     const double f0 = hp->f0, d0 = hp->d0;
     const unsigned n = (unsigned)a.n + (unsigned)b.n;  // at most 2^31
     for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
@@ -449,6 +454,8 @@ __global__ void __launch_bounds__(kPairThreads)
 link_kernel(const fh_cand_params *c, int32_t max_cells, double d_max, Limits lim, const Head *hp,
             const int32_t *start, Sorted o, int32_t *parent, int32_t *err)
 {
+    let_next_start();
+    wait_for_previous();
     const int32_t nbf = hp->nbf, nbd = hp->nbd;
     const float4 tol = hp->tol;
     scan_pairs(
@@ -483,6 +490,8 @@ link_kernel(const fh_cand_params *c, int32_t max_cells, double d_max, Limits lim
 // concurrent find still ends at the same root), and the number of roots
 __global__ void __launch_bounds__(256) finish_labels_kernel(int32_t *label, int32_t n, Head *h)
 {
+    let_next_start();
+    wait_for_previous();
     int roots = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int32_t r = uf_find(label, i, &h->err);
@@ -539,6 +548,8 @@ __device__ __forceinline__ bool inside(const CoinArgs &a, unsigned t, unsigned u
 __global__ void __launch_bounds__(kPairThreads) coin_count_kernel(const CoinArgs a, int32_t *cnt1,
                                                                   int32_t *cnt2)
 {
+    let_next_start();
+    wait_for_previous();
     const int32_t nbf = a.h->nbf, nbd = a.h->nbd;
     const float4 tol = a.h->tol;
     scan_pairs(
@@ -574,6 +585,8 @@ __global__ void __launch_bounds__(256)
 coin_write_kernel(const CoinArgs a, const int32_t *cnt1, const int64_t *off, int64_t capacity,
                   int32_t *pairs)
 {
+    let_next_start();
+    wait_for_previous();
     const int n = a.start[a.max_cells];
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
         const int32_t i = a.o.index(t);
@@ -633,6 +646,8 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z)
 
 __global__ void cc_insert_kernel(const CCArgs a)
 {
+    let_next_start();
+    wait_for_previous();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < a.n_pairs;
          p += (int64_t)gridDim.x * blockDim.x) {
         const int32_t i = a.pairs[2 * p], j = a.pairs[2 * p + 1];
@@ -676,6 +691,8 @@ __global__ void cc_insert_kernel(const CCArgs a)
 
 __global__ void cc_best_kernel(const CCArgs a)
 {
+    let_next_start();
+    wait_for_previous();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < a.n_pairs;
          p += (int64_t)gridDim.x * blockDim.x) {
         const int32_t h = a.slot[p];
@@ -687,6 +704,8 @@ __global__ void cc_best_kernel(const CCArgs a)
 
 __global__ void cc_flag_kernel(const CCArgs a)
 {
+    let_next_start();
+    wait_for_previous();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < a.n_pairs;
          p += (int64_t)gridDim.x * blockDim.x) {
         const int32_t h = a.slot[p];
@@ -697,6 +716,8 @@ __global__ void cc_flag_kernel(const CCArgs a)
 __global__ void cc_write_kernel(const CCArgs a, const int64_t *off, int64_t capacity,
                                 int32_t *out, double *out_d)
 {
+    let_next_start();
+    wait_for_previous();
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < a.n_pairs;
          p += (int64_t)gridDim.x * blockDim.x) {
         if (!a.flag[p]) continue;
@@ -770,11 +791,12 @@ cudaError_t build_cells(const CandSet &a, const CandSet &b, double reach_f, doub
     const int grid = grid_for((int64_t)n);
     range_kernel<<<std::min(grid, 608), kRangeThreads, 0, s>>>(a, b, reach_f, reach_d,
                                                                g.max_cells, g.head, label);
-    cell_count_kernel<<<grid, 256, 0, s>>>(a, b, g.head, g.max_cells, cnt, where);
+    launch_after(cell_count_kernel, grid, 256, 0, s, a, b, g.head, g.max_cells, cnt, where);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = scan_exclusive(cnt, (int64_t)cells, g.start, sc, s);
     if (e == cudaSuccess) {
-        cell_scatter_kernel<<<grid, 256, 0, s>>>(a, b, g.head, g.max_cells, g.start, where, g.o);
+        launch_after(cell_scatter_kernel, grid, 256, 0, s, a, b, g.head, g.max_cells, g.start,
+                     where, g.o);
         e = cudaGetLastError();
     }
     return e;
@@ -811,10 +833,10 @@ int fh_cluster(const fh_cand_params *cands, int32_t n, double d_max, int32_t *la
     cudaError_t e = build_cells(none, set, d_max, d_max, label, g, sc, s);
     if (e == cudaSuccess) {
         // (with no set a the starts of the second half are the set's own)
-        link_kernel<<<pair_grid(n), kPairThreads, 0, s>>>(
-            cands, g.max_cells, d_max, make_limits(reach, d_max), g.head, g.start + g.max_cells,
-            g.o, label, &g.head->err);
-        finish_labels_kernel<<<grid_for(n), 256, 0, s>>>(label, n, g.head);
+        launch_after(link_kernel, pair_grid(n), kPairThreads, 0, s, cands, g.max_cells, d_max,
+                     make_limits(reach, d_max), g.head, g.start + g.max_cells, g.o, label,
+                     &g.head->err);
+        launch_after(finish_labels_kernel, grid_for(n), 256, 0, s, label, n, g.head);
         e = cudaGetLastError();
     }
     Head h{};
@@ -870,11 +892,11 @@ int fh_coincidences(const fh_cand_params *c1, int32_t n1, double t_ref1,
     a.start = g.start;
     a.max_cells = g.max_cells;
     a.o = g.o;
-    coin_count_kernel<<<pair_grid(n1), kPairThreads, 0, s>>>(a, cnt1, n_match2);
+    launch_after(coin_count_kernel, pair_grid(n1), kPairThreads, 0, s, a, cnt1, n_match2);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = scan_exclusive(cnt1, n1, off, sc, s);
     if (e == cudaSuccess && capacity > 0) {
-        coin_write_kernel<<<grid_for(n1), 256, 0, s>>>(a, cnt1, off, capacity, pairs);
+        launch_after(coin_write_kernel, grid_for(n1), 256, 0, s, a, cnt1, off, capacity, pairs);
         e = cudaGetLastError();
     }
     int64_t total = 0;
@@ -933,14 +955,14 @@ int fh_cluster_coincidences(const fh_cand_params *c1, int32_t n1, double t_ref1,
              keys, dmin, best, tsize - 1, slot, flag, dist, err};
     const int grid = grid_for(n_pairs);
     if (e == cudaSuccess) {
-        cc_insert_kernel<<<grid, 256, 0, s>>>(a);
-        cc_best_kernel<<<grid, 256, 0, s>>>(a);
-        cc_flag_kernel<<<grid, 256, 0, s>>>(a);
+        launch_after(cc_insert_kernel, grid, 256, 0, s, a);
+        launch_after(cc_best_kernel, grid, 256, 0, s, a);
+        launch_after(cc_flag_kernel, grid, 256, 0, s, a);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = scan_exclusive(flag, n_pairs, off, sc, s);
     if (e == cudaSuccess && capacity > 0) {
-        cc_write_kernel<<<grid, 256, 0, s>>>(a, off, capacity, out, out_d);
+        launch_after(cc_write_kernel, grid, 256, 0, s, a, off, capacity, out, out_d);
         e = cudaGetLastError();
     }
     int64_t total = 0;

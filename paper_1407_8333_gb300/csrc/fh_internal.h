@@ -56,7 +56,9 @@ __device__ __forceinline__ int64_t floor_times_2p32(double x)
 // (and so, as every kernel of a chain waits, all before it).  A kernel that calls
 // let_next_start() allows its successor in once all its own blocks have started.
 // Without a kernel before it, or in a plain launch, both do nothing.  Worth 1 - 2 us
-// per launch of a chain: a step of four kernels on 200 FFTs 45.2 -> 42.6 us.
+// per launch of a chain: a step of four kernels on 200 FFTs 45.2 -> 42.6 us, the
+// selection and vetoes of 150 days (13 launches) 262 -> 250, clustering and coincidences
+// of 10^5 candidates (30 launches) 560 -> 513.
 __device__ __forceinline__ void wait_for_previous()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

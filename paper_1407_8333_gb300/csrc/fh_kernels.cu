@@ -319,6 +319,7 @@ __device__ __forceinline__ void flush_prep(const PrepArgs &a, int32_t e, unsigne
 // (b - 1) * 1024 ... b * 1024 - 1.
 __global__ void __launch_bounds__(1024, 1) prep_kernel(const PrepArgs a)
 {
+    let_next_start();
     int32_t e = 0;
     unsigned long long amax = 0;
     if (blockIdx.x == 0) {
@@ -382,6 +383,8 @@ __global__ void validate_device_inputs_kernel(const double *__restrict__ t,
                                               const double *__restrict__ sky, int32_t n_fft,
                                               int32_t n_dir, int32_t *err)
 {
+    let_next_start();
+    wait_for_previous();
     const int lane = threadIdx.x & 31;
     const int gw = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     int32_t e = 0;
@@ -2088,8 +2091,8 @@ cudaError_t launch_validate_device_inputs(const double *t, const double *freq,
     const int64_t threads = (int64_t)(n_fft > 0 ? n_fft : 0) * 32 > n_dir
                                 ? (int64_t)n_fft * 32 : (int64_t)n_dir;
     if (threads <= 0) return cudaSuccess;
-    validate_device_inputs_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(
-        t, freq, offsets, v, sky, n_fft, n_dir, err);
+    launch_after(validate_device_inputs_kernel, (unsigned)((threads + 255) / 256), 256, 0, s, t,
+                 freq, offsets, v, sky, n_fft, n_dir, err);
     return cudaGetLastError();
 }
 

@@ -120,6 +120,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 // ratios are formed in place; flags and counts as in select_mask_kernel.
 __global__ void __launch_bounds__(kSegThreads) select_mask_bulk_kernel(const SelArgs a)
 {
+    let_next_start();
     __shared__ __align__(128) float p_s[kSegBins + 8];  // p_s[4 + k]: S_P, then R, of bin j0 + k
     __shared__ __align__(128) float q_s[kSegBins];
     __shared__ __align__(8) unsigned long long bar;
@@ -196,6 +197,7 @@ __global__ void __launch_bounds__(kSegThreads) select_mask_bulk_kernel(const Sel
 template <bool VEC>
 __global__ void __launch_bounds__(kSegThreads) select_mask_kernel(const SelArgs a)
 {
+    let_next_start();
     __shared__ float r_s[kSegBins + 2];  // r_s[1 + k] = R(j0 + k); halos at 0 and kSegBins + 1
     __shared__ int32_t warp_cnt[kSegThreads / 32];
     const int row = blockIdx.y, seg = blockIdx.x;
@@ -276,6 +278,8 @@ struct ExpandArgs {
 // bin order and written as contiguous runs.
 __global__ void __launch_bounds__(kSegWords) select_expand_kernel(const ExpandArgs a)
 {
+    let_next_start();
+    wait_for_previous();
     __shared__ int32_t wsum[kSegWords / 32];
     __shared__ int32_t peaks_s[kSegBins / 2];  // strict maxima: at most every other bin
     const int row = blockIdx.y, seg = blockIdx.x;
@@ -329,6 +333,8 @@ constexpr int kScanTile = kScanThreads * kScanPer;
 __global__ void __launch_bounds__(kScanThreads)
 tile_sums_kernel(const int32_t *cnt, int64_t n, int64_t *sums)
 {
+    let_next_start();
+    wait_for_previous();
     __shared__ int64_t part[kScanThreads / 32];
     const int64_t base = (int64_t)blockIdx.x * kScanTile;
     int64_t s = 0;
@@ -367,6 +373,8 @@ __global__ void __launch_bounds__(kScanThreads)
 scan_counts_kernel(const int32_t *cnt, int64_t n, T *pref, int32_t stride, int64_t *strided,
                    const int64_t *sums, int64_t *total)
 {
+    let_next_start();
+    wait_for_previous();
     __shared__ int64_t part[kScanThreads / 32];
     __shared__ int64_t carry;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -521,6 +529,7 @@ __global__ void __launch_bounds__(256)
 gross_setup_kernel(const int64_t *o, int32_t n_fft, int64_t n_peaks, GrossGrid g, int64_t *edge,
                    int32_t *hist, int64_t cells, int32_t *err)
 {
+    let_next_start();
     const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
     check_csr(o, n_fft, n_peaks, first, step, err);
@@ -556,6 +565,8 @@ __global__ void __launch_bounds__(kFftThreads)
 gross_hist_kernel(const int64_t *o, const int32_t *bins, int64_t n_peaks, GrossGrid g,
                   const int64_t *__restrict__ edge, int32_t *cell, int32_t *hist)
 {
+    let_next_start();
+    wait_for_previous();
     __shared__ int64_t it_s;
     const int i = blockIdx.x, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) it_s = g.it_of(i);
@@ -605,6 +616,7 @@ __global__ void __launch_bounds__(256)
 bin_hist_kernel(const int64_t *o, const int32_t *bins, int32_t n_fft, int64_t n_peaks,
                 int32_t n_bins, int32_t *hist, int32_t *err)
 {
+    let_next_start();
     const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
     check_csr(o, n_fft, n_peaks, first, step, err);
@@ -634,6 +646,8 @@ __device__ __forceinline__ void count_values(const int32_t *hist, int32_t n_bins
 __global__ void count_hist_kernel(const int32_t *hist, int32_t n_bins, int32_t vmax, int32_t *hc,
                                   int32_t *err)
 {
+    let_next_start();
+    wait_for_previous();
     count_values(hist, n_bins, vmax, blockIdx.x * blockDim.x + threadIdx.x,
                  gridDim.x * blockDim.x, hc, err);
 }
@@ -683,6 +697,8 @@ __global__ void __launch_bounds__(kScanThreads)
 robust_stats_kernel(const int32_t *counts, int32_t *hc, int32_t vmax, int32_t n_bins, int32_t *hd,
                     double k_sigma, Result *res_out)
 {
+    let_next_start();
+    wait_for_previous();
     extern __shared__ int32_t small_s[];
     __shared__ int64_t part[kScanThreads / 32];
     __shared__ int64_t res[2];
@@ -751,6 +767,8 @@ __global__ void __launch_bounds__(kFftThreads)
 filter_count_kernel(const int64_t *o, const int32_t *bins, int64_t n_peaks, Keep keep,
                     int32_t *cnt)
 {
+    let_next_start();
+    wait_for_previous();
     __shared__ int sum;
     const int i = blockIdx.x;
     if (threadIdx.x == 0) sum = 0;
@@ -772,6 +790,8 @@ filter_write_kernel(const int64_t *o, const int32_t *bins, int64_t n_peaks, Keep
                     const int64_t *o_out, int64_t capacity, FreqOf fq, int32_t *bins_out,
                     double *freq_out)
 {
+    let_next_start();
+    wait_for_previous();
     constexpr int kWarps = kFftThreads / 32;
     __shared__ int kept[2][kWarps];
     const int i = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -810,11 +830,10 @@ cudaError_t scan_exclusive(const int32_t *cnt, int64_t n, T *pref, Scratch &sc, 
     if (tiles > 2) {  // one or two tiles: one block, one launch
         const cudaError_t e = sc.get(&sums, (size_t)tiles);
         if (e != cudaSuccess) return e;
-        tile_sums_kernel<<<(unsigned)tiles, kScanThreads, 0, s>>>(cnt, n, sums);
+        launch_after(tile_sums_kernel, (unsigned)tiles, kScanThreads, 0, s, cnt, n, sums);
     }
-    scan_counts_kernel<T><<<sums ? (unsigned)tiles : 1u, kScanThreads, 0, s>>>(cnt, n, pref, 1,
-                                                                              nullptr, sums,
-                                                                              nullptr);
+    launch_after(scan_counts_kernel<T>, sums ? (unsigned)tiles : 1u, kScanThreads, 0, s, cnt, n,
+                 pref, 1, nullptr, sums, nullptr);
     return cudaGetLastError();
 }
 template cudaError_t scan_exclusive<int32_t>(const int32_t *, int64_t, int32_t *, Scratch &,
@@ -834,18 +853,18 @@ int run_filter(const int64_t *o, const int32_t *bins, int32_t n_fft, int64_t n_p
     int32_t *cnt = nullptr;
     cudaError_t e = sc.get(&cnt, (size_t)n_fft);
     if (e == cudaSuccess && n_fft > 0) {
-        filter_count_kernel<<<n_fft, kFftThreads, 0, s>>>(o, bins, n_peaks, keep, cnt);
+        launch_after(filter_count_kernel<Keep>, n_fft, kFftThreads, 0, s, o, bins, n_peaks, keep,
+                     cnt);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-        scan_counts_kernel<int64_t><<<1, kScanThreads, 0, s>>>(cnt, n_fft, o_out, 1, nullptr,
-                                                               nullptr, &res->total);
+        launch_after(scan_counts_kernel<int64_t>, 1, kScanThreads, 0, s, cnt, n_fft, o_out, 1,
+                     nullptr, nullptr, &res->total);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && n_fft > 0) {
-        filter_write_kernel<<<n_fft, kFftThreads, 0, s>>>(o, bins, n_peaks, keep, o_out, capacity,
-                                                          make_freq_of(k0, t_fft), bins_out,
-                                                          freq_out);
+        launch_after(filter_write_kernel<Keep>, n_fft, kFftThreads, 0, s, o, bins, n_peaks, keep,
+                     o_out, capacity, make_freq_of(k0, t_fft), bins_out, freq_out);
         e = cudaGetLastError();
     }
     Result h{};
@@ -955,14 +974,14 @@ int fh_peakmap_select(const float *s_p, const float *s_ar, int32_t n_fft, int32_
         select_mask_kernel<false><<<dim3(n_seg, n_fft), kSegThreads, 0, s>>>(a);
     e = cudaGetLastError();
     if (e == cudaSuccess) {
-        scan_counts_kernel<int64_t><<<1, kScanThreads, 0, s>>>(
-            seg_count, (int64_t)n_fft * n_seg, seg_base, n_seg, offsets, nullptr, &res->total);
+        launch_after(scan_counts_kernel<int64_t>, 1, kScanThreads, 0, s, seg_count,
+                     (int64_t)n_fft * n_seg, seg_base, n_seg, offsets, nullptr, &res->total);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
         ExpandArgs x{mask, seg_base, n_seg, n_words, capacity, make_freq_of(k0, t_fft), bins,
                      freq};
-        select_expand_kernel<<<dim3(n_seg, n_fft), kSegWords, 0, s>>>(x);
+        launch_after(select_expand_kernel, dim3(n_seg, n_fft), kSegWords, 0, s, x);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return cuda_error(e, "peak selection");
@@ -1013,8 +1032,8 @@ int fh_peakmap_gross_veto(const double *t, const int64_t *offsets, const int32_t
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && n_fft > 0) {
-        gross_hist_kernel<<<n_fft, kFftThreads, 0, s>>>(offsets, bins, n_peaks, g, edge, cell,
-                                                        hist);
+        launch_after(gross_hist_kernel, n_fft, kFftThreads, 0, s, offsets, bins, n_peaks, g, edge,
+                     cell, hist);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return cuda_error(e, "gross histogram");
@@ -1057,12 +1076,13 @@ int fh_peakmap_persistency_veto(const int64_t *offsets, const int32_t *bins, int
     }
     if (e == cudaSuccess && !small) {
         const int grid = (int)std::min<int64_t>(((int64_t)n_bins + 255) / 256, 4096);
-        count_hist_kernel<<<grid, 256, 0, s>>>(hist, n_bins, vmax, hc, &res->err);
+        launch_after(count_hist_kernel, grid, 256, 0, s, hist, n_bins, vmax, hc, &res->err);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-        robust_stats_kernel<<<1, kScanThreads, small ? sizeof(int32_t) * (nv + nd) : 0, s>>>(
-            small ? hist : nullptr, hc, vmax, n_bins, hc ? hc + nv : nullptr, k_sigma, res);
+        launch_after(robust_stats_kernel, 1, kScanThreads, small ? sizeof(int32_t) * (nv + nd) : 0,
+                     s, small ? hist : nullptr, hc, vmax, n_bins, hc ? hc + nv : nullptr, k_sigma,
+                     res);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return cuda_error(e, "persistency histogram");

@@ -77,6 +77,8 @@ constexpr int kRefList = 64;  // (FFT, peak) entries a warp collects before it p
 // places list x directions, a lane each.
 __global__ void __launch_bounds__(kRefThreads) refine_kernel(const RefineArgs a)
 {
+    let_next_start();
+    wait_for_previous();
     extern __shared__ int32_t hist[];  // [direction][row][3 K], then the sky
     __shared__ int32_t list_fft[kRefThreads / 32][kRefList];
     __shared__ int64_t list_peak[kRefThreads / 32][kRefList];
@@ -237,6 +239,8 @@ struct PickArgs {
 constexpr int kPickThreads = 256;
 __global__ void __launch_bounds__(kPickThreads) refine_pick_kernel(const PickArgs a)
 {
+    let_next_start();
+    wait_for_previous();
     __shared__ int32_t best_s[kPickThreads / 32][3];  // count, (direction, row), cell
     const int c = a.cand0 + blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -491,9 +495,9 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
                 const unsigned groups =
                     (unsigned)((ra.n_dir + ra.dirs_per - 1) / ra.dirs_per * row_groups);
                 dim3 grid(nc, (n + ra.ffts_per - 1) / ra.ffts_per, groups);
-                refine_kernel<<<grid, kRefThreads, smem, s>>>(ra);
+                launch_after(refine_kernel, grid, kRefThreads, smem, s, ra);
             }
-            refine_pick_kernel<<<nc, kPickThreads, 0, s>>>(pk);
+            launch_after(refine_pick_kernel, nc, kPickThreads, 0, s, pk);
             e = cudaGetLastError();
             if (e != cudaSuccess) return cuda_error(e, "refinement");
         }
