@@ -34,6 +34,7 @@
 // longitudes, divided by (w1 + w2) * 0.5; ((k_l^2 + k_b^2) + k_f^2) + k_fd^2 and
 // its square root), so every link and every coincidence is decided exactly as
 // the definition decides it.
+#include <climits>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -396,18 +397,18 @@ __device__ __forceinline__ void uf_union(int32_t *parent, int32_t a, int32_t b, 
 // through its ranges of sorted positions (neighbouring lanes read neighbouring
 // records); pairs that the rejects leave go to the warp's list, and 32 of them at a
 // time are decided, a lane each.  (Decided where they are found, one lane in four was
-// busy and the scan of 10^5 candidates took 144 us, link, and 98 us, coincidences;
-// a thread per candidate also left three quarters of the warps empty.)
+// busy and the scan of 10^5 candidates took 144 us, link, and 98 us, coincidences,
+// now 56 and 25; a thread per candidate also left three quarters of the warps empty.)
 //   range(t, k, lo, hi): the k-th of `ranges` ranges of position t
 //   decide(t, u): what to do with the pair of positions t and u
 constexpr int kScanLanes = 4;
 constexpr int kPairThreads = 256;
 constexpr int kPairCands = kPairThreads / kScanLanes;  // candidates of a block
 template <typename R, typename D>
-__device__ __forceinline__ void scan_pairs(const Sorted &o, unsigned n, int ranges, const float4 &hi_lim,
-                                           const float4 &tol, R &&range, D &&decide)
+__device__ __forceinline__ void scan_pairs(const Sorted &o, unsigned n, int ranges,
+                                           const float4 &hi_lim, const float4 &tol, R &&range, D &&decide)
 {
-    __shared__ uint2 list_s[kPairThreads / 32][64];
+    __shared__ uint2 list_s[kPairThreads / 32][96];
     uint2 *list = list_s[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31, sub = lane % kScanLanes;
     const unsigned lt = (1u << lane) - 1u;
@@ -418,15 +419,28 @@ __device__ __forceinline__ void scan_pairs(const Sorted &o, unsigned n, int rang
     for (int k = 0; k < ranges; ++k) {
         unsigned lo = 0, hi = 0;
         if (t < n) range(t, k, lo, hi);
-        for (unsigned u = lo + sub; __any_sync(kFull, u < hi); u += kScanLanes) {
-            bool near = false;
-            if (u < hi)
-                near = !far_apart(apart(xa, o.x(u)), wid(ha, o.h(u)), hi_lim, tol);
-            const unsigned m = __ballot_sync(kFull, near);
-            if (m == 0) continue;
-            if (near) list[listed + __popc(m & lt)] = make_uint2(t, u);
-            listed += __popc(m);
-            if (listed >= 32) {
+        // every lane takes the warp's longest share, two records at a time
+        const unsigned longest =
+            __reduce_max_sync(kFull, hi > lo ? (hi - lo + kScanLanes - 1) / kScanLanes : 0u);
+        unsigned u = lo + sub;
+        for (unsigned step = 0; step < longest; step += 2, u += 2 * kScanLanes) {
+            float4 xu[2], hu[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const unsigned v = u + r * kScanLanes < hi ? u + r * kScanLanes : 0u;
+                xu[r] = o.x(v);
+                hu[r] = o.h(v);
+            }
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const unsigned v = u + r * kScanLanes;
+                const bool near =
+                    v < hi && !far_apart(apart(xa, xu[r]), wid(ha, hu[r]), hi_lim, tol);
+                const unsigned m = __ballot_sync(kFull, near);
+                if (near) list[listed + __popc(m & lt)] = make_uint2(t, v);
+                listed += __popc(m);
+            }
+            while (listed >= 32) {
                 __syncwarp();
                 listed -= 32;
                 const uint2 q = list[listed + lane];
@@ -448,9 +462,9 @@ __device__ __forceinline__ void scan_pairs(const Sorted &o, unsigned n, int rang
 // whose distance lies within the bound of d_max take the binary64 divisions and
 // square root (GB300's binary64 rate is a small fraction of its binary32 one).
 // 10^5 candidates of one 1 Hz band: 4.0 ms with buckets of frequency alone and the
-// binary64 records gathered per pair (117 million pairs looked at, now 7), 59 us
-// now; 10^6 over 10 Hz: 25.4 -> 0.41 ms.
-__global__ void __launch_bounds__(kPairThreads)
+// binary64 records gathered per pair, 56 us now; 10^6 over 10 Hz: 25.4 -> 0.37 ms (0.41
+// with the 64 registers that leave four blocks on an SM).
+__global__ void __launch_bounds__(kPairThreads, 5)
 link_kernel(const fh_cand_params *c, int32_t max_cells, double d_max, Limits lim, const Head *hp,
             const int32_t *start, Sorted o, int32_t *parent, int32_t *err)
 {
@@ -517,34 +531,53 @@ struct CoinArgs {
     const int32_t *start; // set 1's cells, then set 2's (max_cells each)
     int32_t max_cells;
     Sorted o;             // set 1's candidates, then set 2's
-    int32_t *keep;        // [set-1 sorted position][kKeep]
+    int32_t *keep;        // [set-1 sorted position][kKeep], 16-byte aligned
 };
 
-// all four windows hold in binary64 (frequencies at the common time)
-__device__ bool coincide(const CoinArgs &a, int32_t i, int32_t j)
+// bins_apart(...) <= window, mostly without its division.  With a the distance, b the
+// mean width and t = RN(a - window b), which has the sign of the exact difference:
+// t <= 0 means a / b <= window, and so its rounding; t above 2^-50 a means a quotient
+// more than two units above the window; the division decides in between, and for
+// widths and windows next to the ends of binary64's range.
+__device__ __forceinline__ bool within(double x1, double x2, double w1, double w2, bool wrap,
+                                       double window)
 {
-    const fh_cand_params x = a.s1.c[i], y = a.s2.c[j];
-    return bins_apart(a.s1.freq(x), a.s2.freq(y), x.df, y.df, false) <= a.w[2] &&
-           bins_apart(x.fdot, y.fdot, x.dfdot, y.dfdot, false) <= a.w[3] &&
-           bins_apart(x.beta, y.beta, x.dbeta, y.dbeta, false) <= a.w[1] &&
-           bins_apart(x.lam, y.lam, x.dlam, y.dlam, true) <= a.w[0];
+    double a = fabs(__dsub_rn(x2, x1));
+    if (wrap && a > kPi) a = __dsub_rn(kTwoPi, a);
+    const double b = __dmul_rn(__dadd_rn(w1, w2), 0.5);
+    const double t = __fma_rn(-window, b, a);
+    const int ea = __double2hiint(a) >> 20, eb = __double2hiint(b) >> 20,
+              ew = __double2hiint(window) >> 20, et = __double2hiint(t) >> 20;
+    // (signs would make these negative or 2048 and more)
+    if (ea < 2047 && eb > 60 && eb < 2000 && ew > 60 && ew < 2000) {
+        if (__double_as_longlong(t) <= 0) return true;
+        if (et >= ea - 49) return false;
+    }
+    return __ddiv_rn(a, b) <= window;
 }
 
 // whether the records at sorted positions t (set 1) and u coincide, after the rejects:
-// clearly inside every window in binary32, else the exact test
+// each parameter clearly inside its window in binary32, else the exact test of that
+// one (values on the grid of a search are often whole windows apart)
 __device__ __forceinline__ bool inside(const CoinArgs &a, unsigned t, unsigned u, const float4 &tol)
 {
     const float4 d = apart(a.o.x(t), a.o.x(u)), w = wid(a.o.h(t), a.o.h(u));
-    const bool in = !a.lim.exact && ordinary(d, w) && d.x + tol.x < a.lim.lo.x * w.x &&
-                    d.y + tol.y < a.lim.lo.y * w.y && d.z + tol.z < a.lim.lo.z * w.z &&
-                    d.w + tol.w < a.lim.lo.w * w.w;
-    return in || coincide(a, a.o.index(t), a.o.index(u));
+    const bool ok = !a.lim.exact && ordinary(d, w);
+    const bool il = ok && d.x + tol.x < a.lim.lo.x * w.x, ib = ok && d.y + tol.y < a.lim.lo.y * w.y,
+               jf = ok && d.z + tol.z < a.lim.lo.z * w.z, id = ok && d.w + tol.w < a.lim.lo.w * w.w;
+    if (il && ib && jf && id) return true;
+    const fh_cand_params &x = a.s1.c[a.o.index(t)], &y = a.s2.c[a.o.index(u)];
+    return (jf || within(a.s1.freq(x), a.s2.freq(y), x.df, y.df, false, a.w[2])) &&
+           (id || within(x.fdot, y.fdot, x.dfdot, y.dfdot, false, a.w[3])) &&
+           (ib || within(x.beta, y.beta, x.dbeta, y.dbeta, false, a.w[1])) &&
+           (il || within(x.lam, y.lam, x.dlam, y.dlam, true, a.w[0]));
 }
 
 // Partners of every set-1 candidate, counted, the first kKeep found kept (in any
-// order; the write sorts them).  10^5 x 10^5 candidates of one 1 Hz band: 1.20 ms -> 55 us
-// for the count and 1.45 ms -> 36 us for the write; 10^6 x 10^6 over 10 Hz: 9.7 -> 0.35 ms
-// and 11.4 ms -> 61 us.  cnt1 starts at zero.
+// order; the write sorts them).  10^5 x 10^5 candidates of one 1 Hz band: 1.20 ms -> 25 us
+// for the count and 1.45 ms -> 30 us for the write; 10^6 x 10^6 over 10 Hz: 9.7 -> 0.18 ms
+// and 11.4 ms -> 44 us.  (With the four divisions of every pair that binary32 left open,
+// binary64 operations set the count's time, 55 us and 0.37 ms.)  cnt1 starts at zero.
 __global__ void __launch_bounds__(kPairThreads) coin_count_kernel(const CoinArgs a, int32_t *cnt1,
                                                                   int32_t *cnt2)
 {
@@ -607,10 +640,31 @@ coin_write_kernel(const CoinArgs a, const int32_t *cnt1, const int64_t *off, int
             }
             ++o;
         };
-        if (c <= kKeep)
-            for (int k = 0; k < c; ++k) put(a.keep[(int64_t)t * kKeep + k]);
-        else
+        if (c > kKeep) {
             for_partners(a, t, put);
+            continue;
+        }
+        // the kept ones, sorted in registers (insertion in memory waits for each store)
+        const int4 *kept = reinterpret_cast<const int4 *>(a.keep + (int64_t)t * kKeep);
+        const int4 p0 = kept[0], p1 = kept[1];
+        int32_t v[kKeep] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k)
+            if (k >= c) v[k] = INT_MAX;
+#pragma unroll
+        for (int r = 0; r < kKeep; ++r)
+#pragma unroll
+            for (int k = r & 1; k + 1 < kKeep; k += 2) {
+                const int32_t lo = min(v[k], v[k + 1]);
+                v[k + 1] = max(v[k], v[k + 1]);
+                v[k] = lo;
+            }
+#pragma unroll
+        for (int k = 0; k < kKeep; ++k)
+            if (k < c && o0 + k < capacity) {
+                pairs[2 * (o0 + k)] = i;
+                pairs[2 * (o0 + k) + 1] = v[k];
+            }
     }
 }
 
@@ -663,6 +717,12 @@ __global__ void cc_insert_kernel(const CCArgs a)
             a.slot[p] = -1;
             continue;
         }
+        // (the distance before the probes: the lanes part there, and binary64
+        // operations of half-empty warps had doubled the time)
+        const fh_cand_params x = a.c1[i], y = a.c2[j];
+        const double fx = __dadd_rn(x.f, __dmul_rn(x.fdot, a.dt1));
+        const double fy = __dadd_rn(y.f, __dmul_rn(y.fdot, a.dt2));
+        const double d = norm_distance(x, y, fx, fy);
         const unsigned long long key = ((unsigned long long)(uint32_t)la << 32) | (uint32_t)lb;
         int64_t h = (int64_t)(mix64(key) & (unsigned long long)a.tmask);
         int32_t at = -1;
@@ -679,10 +739,6 @@ __global__ void cc_insert_kernel(const CCArgs a)
             a.slot[p] = -1;
             continue;
         }
-        const fh_cand_params x = a.c1[i], y = a.c2[j];
-        const double fx = __dadd_rn(x.f, __dmul_rn(x.fdot, a.dt1));
-        const double fy = __dadd_rn(y.f, __dmul_rn(y.fdot, a.dt2));
-        const double d = norm_distance(x, y, fx, fy);
         a.dist[p] = d;
         a.slot[p] = at;
         atomicMin(a.dmin + at, (unsigned long long)__double_as_longlong(d));
