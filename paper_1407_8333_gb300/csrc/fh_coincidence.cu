@@ -531,7 +531,8 @@ struct CoinArgs {
     const int32_t *start; // set 1's cells, then set 2's (max_cells each)
     int32_t max_cells;
     Sorted o;             // set 1's candidates, then set 2's
-    int32_t *keep;        // [set-1 sorted position][kKeep], 16-byte aligned
+    int32_t *keep;        // [set-1 sorted position][kKeep], 16-byte aligned; null: the
+                          // write looks for every candidate's partners again
 };
 
 // bins_apart(...) <= window, mostly without its division.  With a the distance, b the
@@ -594,7 +595,7 @@ __global__ void __launch_bounds__(kPairThreads) coin_count_kernel(const CoinArgs
             if (!inside(a, t, u, tol)) return;
             const int32_t j = a.o.index(u);
             const int c = atomicAdd(cnt1 + a.o.index(t), 1);
-            if (c < kKeep) a.keep[(int64_t)t * kKeep + c] = j;
+            if (a.keep && c < kKeep) a.keep[(int64_t)t * kKeep + c] = j;
             if (cnt2) atomicAdd(cnt2 + j, 1);
         });
 }
@@ -640,7 +641,7 @@ coin_write_kernel(const CoinArgs a, const int32_t *cnt1, const int64_t *off, int
             }
             ++o;
         };
-        if (c > kKeep) {
+        if (!a.keep || c > kKeep) {
             for_partners(a, t, put);
             continue;
         }
@@ -940,7 +941,11 @@ int fh_coincidences(const fh_cand_params *c1, int32_t n1, double t_ref1,
     e = build_cells(a.s1, a.s2, win[2], win[3], nullptr, g, sc, s);
     if (e == cudaSuccess && !cnt1) e = sc.get(&cnt1, (size_t)n1);
     if (e == cudaSuccess) e = sc.get(&off, (size_t)n1 + 1);
-    if (e == cudaSuccess) e = sc.get(&a.keep, (size_t)n1 * kKeep);
+    // (sets so large that these 32 bytes per candidate do not fit do without)
+    if (e == cudaSuccess && sc.get(&a.keep, (size_t)n1 * kKeep) != cudaSuccess) {
+        cudaGetLastError();
+        a.keep = nullptr;
+    }
     // (candidates of set 1 outside the grid have no partner and no sorted position)
     if (e == cudaSuccess) e = cudaMemsetAsync(cnt1, 0, 4 * (size_t)n1, s);
     if (e != cudaSuccess) return cuda_error(e, "coincidences set-up");
