@@ -126,6 +126,9 @@ struct TransformJob {
     int32_t tile_cells;      // W
     int32_t n_slabs, n_tiles;
     int32_t dir_begin, n_dir;
+    // runs of FFTs of the transform's warps (launch_transform): warp w's first run is
+    // [w run0, (w + 1) run0), run r >= warps the run1 FFTs from run_base + r run1
+    int32_t run0, run1, run_base;
 };
 
 struct JobTable {

@@ -1101,8 +1101,6 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                            J->unit_delta[d_abs] <= J->delta_alloc);
         const int64_t base_shift = (int64_t)(b0 - K + 1) * 4294967296LL;
         const int64_t e_fixed = (int64_t)E * 4294967296LL;
-        const int nchunks = (n_fft + 31) >> 5;
-
         // One pass over the tile: zero the counters, accumulate rows j0 .. j0 +
         // R - 1 of direction d_a + dsel (QUAD: of both directions of the pair, d_a
         // in the low halves, d_b in the high halves), emit.  The windows of a pair
@@ -1146,10 +1144,9 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
             // comes out of a shuffle so that the compiler knows it to be the same in all
             // lanes (else it guards every round's shuffles against divergence: 33
             // million more branch instructions per launch and 2 % of the time).
-            const int run0 = (3 * nchunks) / (4 * nwarps), run1 = max(1, run0 >> 4);
             int run = warp;  // runs below nwarps are first runs
-            int i0 = run0 > 0 ? run0 * warp * 32 : warp * 32;
-            int i_end = run0 > 0 ? run0 * (warp + 1) * 32 : i0 + 32;
+            int i0 = J->run0 * warp;
+            int i_end = i0 + J->run0;
             int skip = 0;
             while (i0 < n_fft) {
                 int64_t cb, dv, q0;
@@ -1418,9 +1415,8 @@ transform_kernel(const __grid_constant__ JobTable tbl, int64_t total_items, int3
                     if (i0 >= i_end) {
                         if (lane == 0) run = atomicAdd(next_chunk, 1);
                         run = __shfl_sync(kFull, run, 0);
-                        const int r = run - nwarps;
-                        i0 = (run0 > 0 ? run0 * nwarps + r * run1 : run) * 32;
-                        i_end = i0 + run1 * 32;
+                        i0 = J->run_base + run * J->run1;
+                        i_end = i0 + J->run1;
                     }
                 }
             }
@@ -2204,8 +2200,21 @@ cudaError_t launch_transform(int32_t mode, const JobTable &tbl, int64_t total_it
     }
     const int pack = dirs ? 1 : rows ? 2 : 0;
     if (weighted && pack) return cudaErrorInvalidValue;  // packed counters hold plain counts only
+    // Runs of FFTs (see the walk): three quarters of a warp's share first, then short ones.
+    // Where the share is below 32 FFTs each warp takes its share at once: 200 FFTs dealt
+    // 32 to a warp kept 7 warps of 20 busy, for 4 rounds each (256 directions of them:
+    // step 140 -> 132 us).
+    JobTable t = tbl;
+    for (int j = 0; j < t.n_jobs; ++j) {
+        TransformJob &x = t.job[j];
+        const int32_t share = 3 * ((x.n_fft + 31) / 32) / (4 * nwarps);  // of 32 FFTs
+        x.run1 = share > 0 ? 32 * std::max(1, share / 16)
+                           : std::min(32, (x.n_fft + nwarps - 1) / nwarps);
+        x.run0 = share > 0 ? 32 * share : x.run1;
+        x.run_base = nwarps * (x.run0 - x.run1);
+    }
     return with_transform_kernel(mode, nwarps, weighted, pack, maps, [&](auto k) {
-        return launch_after(k, grid, nwarps * 32, smem, s, tbl, total_items, hist_words, guard,
+        return launch_after(k, grid, nwarps * 32, smem, s, t, total_items, hist_words, guard,
                             kRows * 4u, sched);
     });
 }

@@ -59,6 +59,16 @@ def test_runs_of_ffts(fh, n_fft, n_dir, n_fdot):
         check(fh, inp, pp, block_warps=4, tile_cells=128)
 
 
+# below 43 chunks for 32 warps a warp's run is its share of the FFTs, at most 32 (a warp
+# without one, the last one short, 31 and 32 to a warp, and more FFTs than 32 to each)
+@pytest.mark.parametrize("n_fft", [1, 31, 33, 65, 200, 992, 993, 1023, 1025, 1300])
+@pytest.mark.parametrize("n_dir, n_fdot, warps", [(1, 5, 32), (1, 40, 24), (2, 34, 32), (2, 4, 20)])
+def test_few_ffts_per_warp(fh, n_fft, n_dir, n_fdot, warps):
+    inp, pp = synth.random_case(1300 + n_fft + n_fdot, n_fft=n_fft, n_bins=24, n_fdot=n_fdot,
+                                n_dir=n_dir, p=0.2, vmax=2e-6)
+    check(fh, inp, pp, block_warps=warps, tile_cells=96)
+
+
 @pytest.mark.parametrize("n_fft", [193, 351])
 def test_runs_of_ffts_weighted(fh, n_fft):
     inp, pp = synth.random_case(77 + n_fft, n_fft=n_fft, n_bins=30, n_fdot=20, n_dir=2, p=0.2)
