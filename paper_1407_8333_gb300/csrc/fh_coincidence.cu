@@ -271,7 +271,8 @@ cell_count_kernel(CandSet a, CandSet b, const Head *hp, int32_t max_cells, int32
     for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const bool in_b = k >= (unsigned)a.n;
         const fh_cand_params *p = in_b ? b.c + (k - a.n) : a.c + k;
-        const double2 q = *reinterpret_cast<const double2 *>(&p->f);  // f, fdot
+        // (8 bytes at a time: a caller's records start on any multiple of 8)
+        const double2 q = make_double2(p->f, p->fdot);
         const CandSet &s = in_b ? b : a;
         const double f = s.shift ? __dadd_rn(q.x, __dmul_rn(q.y, s.dt)) : q.x;
         const int32_t c = cell_of(h, f, q.y);

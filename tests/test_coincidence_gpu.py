@@ -251,6 +251,29 @@ def test_counts_of_any_alignment(fh, co, n, skip):
     assert np.array_equal(pairs.cpu().numpy()[:len(want)], want.reshape(-1, 2))
 
 
+@pytest.mark.parametrize("skip", [1, 2, 5])
+def test_candidates_on_any_multiple_of_8_bytes(fh, co, skip):
+    """Candidate records that do not start on 16 bytes."""
+    import torch
+
+    def shifted(c):
+        buf = torch.zeros(c.size + 8, dtype=torch.float64, device="cuda")
+        view = buf[skip:skip + c.size].view(c.shape)
+        view.copy_(torch.from_numpy(c))
+        assert view.data_ptr() % 16 == 8 * (skip % 2)
+        return view
+
+    a = synth.candidate_set(56, 1, 500, clusters=10, cluster_size=4)
+    b = synth.candidate_set(56, 2, 300, clusters=10, cluster_size=4)
+    want, wn = co.cluster(a, 2.0)
+    lab, n = fh.fh_cluster(shifted(a), 2.0)
+    assert n == wn and np.array_equal(lab.cpu().numpy(), want)
+    p, m1, m2 = fh.fh_coincidences(shifted(a), shifted(b), 0.0, 0.0, 0.0, (2, 2, 2, 2))
+    wp, w1, w2 = co.coincidences(a, b, 0.0, 0.0, 0.0, (2, 2, 2, 2))
+    assert np.array_equal(p.cpu().numpy(), wp.reshape(-1, 2))
+    assert np.array_equal(m1.cpu().numpy(), w1) and np.array_equal(m2.cpu().numpy(), w2)
+
+
 def test_scratch_shared_by_threads_and_streams(fh):
     """Calls of several threads, each on its own stream, share the library's
     scratch pool: every result is that of a call alone; the last plan's
