@@ -41,9 +41,11 @@
  * its work on one stream at a time (its buffers, the transform's item counter
  * among them, are shared by every call on the plan); a server is thread-safe.
  * Calls without a plan's buffers (clustering, coincidences, peakmap steps,
- * refinement) take their scratch stream-ordered from a pool of the library that
- * keeps up to 256 MiB per device between calls and returns it when the process
- * destroys its last plan.
+ * refinement) take their scratch, and plans their table of peak windows (grown by
+ * fh_transform where a call needs more of it), stream-ordered from a pool of the
+ * library.  The pool keeps up to 256 MiB per device between calls and returns it
+ * when the process destroys its last plan (a process that never makes a plan keeps
+ * it until it ends).
  */
 #ifndef FH_H
 #define FH_H

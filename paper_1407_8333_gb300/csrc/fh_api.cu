@@ -81,8 +81,9 @@ int max_optin_smem(int device)
 }
 
 // One pool per device for the scratch of calls that hold no plan (clustering,
-// vetoes, refinement): memory freed by one call serves the next one, on any
-// thread or stream (the driver orders the reuse).  It keeps at most kScratchKeep
+// vetoes, refinement) and the plans' window tables: memory freed by one call serves
+// the next one, on any thread or stream (the driver orders the reuse; so what is
+// taken from it goes back by cudaFreeAsync, or after a wait for its last use).  It keeps at most kScratchKeep
 // bytes across synchronisations, and nothing once the last plan of the process
 // is destroyed.  The default pool keeps nothing, so that every call mapped its
 // memory anew: about 100 us of each clustering, veto or refinement call.
@@ -302,6 +303,8 @@ struct fh_plan_s {
                                          // zero between launches)
     uint32_t *win = nullptr;             // peak windows of the directions being transformed
     size_t win_bytes = 0;
+    bool win_pooled = false;             // the table is the scratch pool's (window_table)
+    std::vector<uint32_t *> old_win;     // tables replaced under capture
     int32_t guard = 0;                   // guard cells for the transform's fast path (32 rows)
     unsigned long long drift = 0;        // bound of max |D_i| the guards are sized for
     int32_t pair_pref = 0;               // 0: pairs (of directions, or of one direction's row
@@ -333,6 +336,8 @@ struct fh_plan_s {
                         A,    profile, cand, err, win,  wq,  ws, sched};  // dmax, unit_delta: in err's block
         for (void *b : bufs)
             if (b) cudaFree(b);
+        for (uint32_t *b : old_win) cudaFree(b);
+        old_win.clear();
         if (h_err) cudaFreeHost(h_err);
         t = freq = v = sky = nullptr;
         offsets = S0 = D = A = offsets_raw = nullptr;
@@ -912,6 +917,41 @@ static int32_t filling_tile(int32_t widest, int32_t n_f0, int64_t stacks, int32_
     return std::min<int32_t>(widest, (int32_t)std::max<int64_t>(128, (w + 15) / 16 * 16));
 }
 
+// The plan's window table with room for `need` bytes, for work on stream s.  It comes
+// from the scratch pool, which has kept memory at hand (a mapping of its own costs
+// the first transform of a plan about 100 us), except under capture, where the graph
+// would own it.  The table that it replaces may still be read by the plan's earlier
+// transforms: pool memory goes back in stream order (cudaFree does not wait for work on
+// such memory, and the pool serves other streams at once); under capture, where neither
+// form of release is part of the step, it stays until the plan is destroyed.
+static int window_table(fh_plan p, size_t need, cudaStream_t s)
+{
+    if (need <= p->win_bytes) return FH_OK;
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(s, &capturing);
+    const bool captured = capturing != cudaStreamCaptureStatusNone;
+    if (p->win && captured) {
+        p->old_win.push_back(p->win);
+    } else if (p->win) {
+        const cudaError_t e = p->win_pooled ? cudaFreeAsync(p->win, s) : cudaFree(p->win);
+        if (e != cudaSuccess) return cuda_error(e, "release of the peak windows");
+    }
+    p->win = nullptr;
+    p->win_bytes = 0;
+    cudaMemPool_t pool = captured ? nullptr : scratch_pool();
+    p->win_pooled = pool != nullptr;
+    const cudaError_t e =
+        pool ? cudaMallocFromPoolAsync(reinterpret_cast<void **>(&p->win), need, pool, s)
+             : cudaMalloc(&p->win, need);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        p->win = nullptr;
+        return set_error(FH_ERR_NOMEM, "cudaMalloc of %zu bytes (peak windows) failed", need);
+    }
+    p->win_bytes = need;
+    return FH_OK;
+}
+
 static int run_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *out_maps,
                          int32_t tile, int32_t nwarps, int32_t schedule, cudaStream_t s,
                          int32_t pair_pref, int32_t item_counter, bool tile_auto = false)
@@ -982,25 +1022,8 @@ static int run_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *o
                               per_unit * (win_cap / per_dir_win)));
     if (pairs && group < n_dir) group = std::max(2, group & ~1);
     const size_t need = per_dir_win * (size_t)((group + per_unit - 1) / per_unit);
-    if (need > p->win_bytes) {
-        if (p->win) cudaFree(p->win);
-        p->win = nullptr;
-        p->win_bytes = 0;
-        // from the scratch pool, which has kept memory at hand (a mapping of its own
-        // costs the first transform of a plan about 100 us), except under capture,
-        // where the graph would own it
-        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-        cudaStreamIsCapturing(s, &capturing);
-        cudaMemPool_t pool =
-            capturing == cudaStreamCaptureStatusNone ? scratch_pool() : nullptr;
-        e = pool ? cudaMallocFromPoolAsync(reinterpret_cast<void **>(&p->win), need, pool, s)
-                 : cudaMalloc(&p->win, need);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return set_error(FH_ERR_NOMEM, "cudaMalloc of %zu bytes (peak windows) failed", need);
-        }
-        p->win_bytes = need;
-    }
+    const int rc = window_table(p, need, s);
+    if (rc) return rc;
     JobTable tbl{};
     tbl.n_jobs = 1;
     for (int32_t g0 = 0; g0 < n_dir; g0 += group) {

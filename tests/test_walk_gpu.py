@@ -185,3 +185,60 @@ def test_correction_and_window_blocks(fh, n_fft, n_dir):
     inp, pp = synth.random_case(500 + n_fft, n_fft=n_fft, n_bins=110, n_fdot=4, n_dir=n_dir, p=0.05,
                                 vmax=2e-6)
     check(fh, inp, pp, tile_cells=32)
+
+
+@pytest.mark.parametrize("n_dir, n_fdot", [(24, 40), (9, 70)])
+def test_window_table_grows_between_transforms_in_flight(fh, n_dir, n_fdot):
+    """One direction, then more and more of them, queued without a wait: each call
+    replaces the window table that the one before may still read, while clustering
+    calls on other threads' streams take and return memory of the same pool.  Every
+    map equals the oracle's."""
+    import threading
+
+    import oracle
+    import torch
+    n_fft = 400
+    inp, pp = synth.random_case(1500 + n_dir, n_fft=n_fft, n_bins=200, n_fdot=n_fdot, n_dir=n_dir,
+                                p=0.2, vmax=2e-6)
+    want = oracle.search(inp, pp, want_maps=True)["maps"]
+    dev = [torch.from_numpy(np.ascontiguousarray(x)).cuda()
+           for x in (inp.t, inp.offsets, inp.freq, inp.v, inp.sky)]
+    cand = torch.from_numpy(synth.candidate_set(71, 0, 20000, clusters=40)).cuda()
+    labels = fh.fh_cluster(cand, 3.0)[0].clone()
+    torch.cuda.synchronize()
+    stop, bad = threading.Event(), []
+
+    def cluster():
+        try:
+            st = torch.cuda.Stream()
+            while not stop.is_set():
+                lab, _ = fh.fh_cluster(cand, 3.0, stream=st)
+                st.synchronize()
+                if not torch.equal(lab, labels):
+                    bad.append("labels")
+        except Exception as e:  # noqa: BLE001
+            bad.append(repr(e))
+
+    threads = [threading.Thread(target=cluster) for _ in range(2)]
+    for t in threads:
+        t.start()
+    try:
+        st = torch.cuda.Stream()
+        for _ in range(10):
+            counts = [1, 2, 5, n_dir]
+            maps = [torch.empty((k, n_fdot, pp["n_f0"]), dtype=torch.int32, device="cuda")
+                    for k in counts]
+            plan = fh.fh_create_plan(fh.make_desc(pp, n_fft, n_dir, inp.n_peaks))
+            torch.cuda.synchronize()
+            fh.fh_correct_doppler(plan, *dev, stream=st)
+            for k, m in zip(counts, maps):
+                fh.fh_transform(plan, 0, k, m, stream=st)
+            st.synchronize()
+            fh.fh_destroy_plan(plan)
+            for k, m in zip(counts, maps):
+                assert np.array_equal(m.cpu().numpy(), want[:k])
+    finally:
+        stop.set()
+        for t in threads:
+            t.join()
+    assert not bad
