@@ -51,14 +51,20 @@ __device__ __forceinline__ int64_t floor_times_2p32(double x)
 }
 
 // Programmatic dependent launch: a kernel launched by launch_after may be set up, and
-// its blocks become resident, while the kernel before it on the stream drains; its
-// first statement, wait_for_previous(), holds it until that one has completed
-// (and so, as every kernel of a chain waits, all before it).  A kernel that calls
-// let_next_start() allows its successor in once all its own blocks have started.
-// Without a kernel before it, or in a plain launch, both do nothing.  Worth 1 - 2 us
-// per launch of a chain: a step of four kernels on 200 FFTs 45.2 -> 42.6 us, the
-// selection and vetoes of 150 days (13 launches) 262 -> 250, clustering and coincidences
-// of 10^5 candidates (30 launches) 560 -> 513.
+// its blocks become resident, while the kernel before it on the stream drains;
+// wait_for_previous(), before its first access to memory, holds it until that one has
+// completed (and so, as every kernel of a chain waits, all before it).  The first
+// kernel of a chain is launched plainly and has no wait.  A kernel that calls
+// let_next_start() allows its successor in once all its own blocks have got there.
+// Without a kernel before it, or in a plain launch, both do nothing.
+// The read-only path (__ldg, const __restrict__ parameters) is for data that no kernel
+// writes while the reader is resident: the caller's inputs, and for the transform the
+// correction's output too, because the window pre-pass lets it in only after its own
+// wait (without a pre-pass it is launched plainly).  What the kernel just before, or
+// one that it overlaps, writes is read by ordinary loads.
+// Worth 1 - 2 us per launch of a chain: a step of four kernels on 200 FFTs
+// 45.2 -> 42.6 us, the selection and vetoes of 150 days (13 launches) 262 -> 250,
+// clustering and coincidences of 10^5 candidates (30 launches) 560 -> 513.
 __device__ __forceinline__ void wait_for_previous()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

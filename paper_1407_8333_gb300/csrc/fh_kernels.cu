@@ -376,9 +376,10 @@ correct_kernel(const PrepArgs a, const double *__restrict__ freq, double f0_min,
 // device-side checks): one warp per FFT (its peaks are read coalesced and
 // compared with their left neighbour, through an already sanitised CSR) and
 // one thread per sky direction.
+// (offsets: written by the kernel before, which this one overlaps)
 __global__ void validate_device_inputs_kernel(const double *__restrict__ t,
                                               const double *__restrict__ freq,
-                                              const int64_t *__restrict__ offsets,
+                                              const int64_t *offsets,
                                               const double *__restrict__ v,
                                               const double *__restrict__ sky, int32_t n_fft,
                                               int32_t n_dir, int32_t *err)
@@ -551,8 +552,8 @@ windows_kernel(const TransformJob J, uint32_t *__restrict__ windows)
     constexpr int kPeaks = PAIR ? 736 : 1024;
     // rows padded by one word: lanes on different FFTs fall on different banks
     __shared__ int32_t cell_s[NR][8][kPeaks + 1];
-    let_next_start();
     wait_for_previous();
+    let_next_start();  // (after the wait: the transform reads the correction's output by __ldg)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int unit = blockIdx.y;
     const int nd = PAIR ? min(2, J.n_dir - 2 * unit) : 1;  // directions of the unit
@@ -2191,8 +2192,9 @@ cudaError_t launch_transform(int32_t mode, const JobTable &tbl, int64_t total_it
     }
     // the launch's packing: every job with direction pairs (1), or with row pairs (2)
     bool weighted = false, dirs = mode == FH_MODE_START && tbl.n_jobs > 0, rows = dirs;
-    bool maps = false;
+    bool maps = false, windows = true;
     for (int j = 0; j < tbl.n_jobs; ++j) {
+        windows = windows && tbl.job[j].windows != nullptr;
         maps = maps || tbl.job[j].maps != nullptr;
         weighted = weighted || tbl.job[j].weights != nullptr;
         dirs = dirs && tbl.job[j].dir_pairs != 0;
@@ -2214,6 +2216,12 @@ cudaError_t launch_transform(int32_t mode, const JobTable &tbl, int64_t total_it
         x.run_base = nwarps * (x.run0 - x.run1);
     }
     return with_transform_kernel(mode, nwarps, weighted, pack, maps, [&](auto k) {
+        if (!windows) {
+            // straight behind the correction, whose output it reads by __ldg
+            k<<<grid, nwarps * 32, smem, s>>>(t, total_items, hist_words, guard, kRows * 4u,
+                                              sched);
+            return cudaGetLastError();
+        }
         return launch_after(k, grid, nwarps * 32, smem, s, t, total_items, hist_words, guard,
                             kRows * 4u, sched);
     });

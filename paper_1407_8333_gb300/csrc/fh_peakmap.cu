@@ -563,7 +563,7 @@ constexpr int kFftThreads = 128;
 // column from binary64 and warp-wide matches.
 __global__ void __launch_bounds__(kFftThreads)
 gross_hist_kernel(const int64_t *o, const int32_t *bins, int64_t n_peaks, GrossGrid g,
-                  const int64_t *__restrict__ edge, int32_t *cell, int32_t *hist)
+                  const int64_t *edge, int32_t *cell, int32_t *hist)
 {
     let_next_start();
     wait_for_previous();
