@@ -107,6 +107,10 @@ cudaMemPool_t scratch_pool()
         props.location.id = dev;
         cudaMemPool_t pool = nullptr;
         uint64_t keep = kScratchKeep;
+        // (making a pool is no part of anybody's capture, this thread's or another's, and
+        // would end it in the default mode)
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
         if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
             if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) ==
                 cudaSuccess)
@@ -114,6 +118,7 @@ cudaMemPool_t scratch_pool()
             else
                 cudaMemPoolDestroy(pool);
         }
+        cudaThreadExchangeStreamCaptureMode(&mode);
         cudaGetLastError();
     }
     return g_pool[dev];

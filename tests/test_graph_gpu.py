@@ -108,3 +108,47 @@ def test_step_replays_from_a_cuda_graph(fh, oracle_mod, schedule):
     finally:
         torch.cuda.synchronize()
         fh.fh_destroy_plan(plan)
+
+
+FIRST_CALL = r'''
+import sys
+sys.path.insert(0, %(root)r)
+import numpy as np, torch
+import oracle
+from paper_1407_8333_gb300 import build, fh, synth
+build.build(); fh.load()
+s = synth.spectra_case(7, 6, 600, wander_amp=30.0, wander_f=(50.01, 50.05), wander_width=5)
+sp, sa = torch.from_numpy(s.s_p).cuda(), torch.from_numpy(s.s_ar).cuda()
+ws = torch.empty(fh.fh_peakmap_select_workspace(6, 600), dtype=torch.uint8, device="cuda")
+out = (torch.zeros(7, dtype=torch.int64, device="cuda"),
+       torch.zeros(1800, dtype=torch.int32, device="cuda"),
+       torch.zeros(1800, dtype=torch.float64, device="cuda"))
+st = torch.cuda.Stream()
+torch.cuda.synchronize()
+g = torch.cuda.CUDAGraph()
+with torch.cuda.graph(g, stream=st):
+    fh.fh_peakmap_select(sp, sa, 2.5, s.k0, s.t_fft, out=out, workspace=%(ws)s, stream=st)
+for k in range(2):
+    for x in out:
+        x.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    o, b = oracle.peakmap.select_peaks(s.s_p, s.s_ar, 2.5)
+    assert np.array_equal(out[0].cpu().numpy(), o)
+    assert np.array_equal(out[1].cpu().numpy()[:len(b)], b)
+print("ok")
+'''
+
+
+@pytest.mark.parametrize("ws", ["ws", "None"])
+def test_first_call_of_a_process_is_captured(ws):
+    """The selection captured as a process's first call of the library, with a
+    caller's workspace and with scratch of its own: making the scratch pool ends no
+    capture."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FIRST_CALL % dict(root=root, ws=ws)],
+                       capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stderr[-2000:]
