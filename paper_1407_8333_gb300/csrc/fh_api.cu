@@ -911,7 +911,9 @@ static int32_t plan_guard(fh_plan p, int32_t kind)
 // The library's default tile for a call of `stacks` (unit, slab) stacks of tiles:
 // the widest, unless its items fill less than half of the SMs; then as narrow
 // as gives half of them an item (not below 128 cells: every tile repeats the
-// guard cells' work and its windows).  One direction of 21 rows x 10240 cells
+// guard cells' work and its windows), which makes fewer items than SMs: a width of
+// at least n_f0 stacks / half leaves each stack at most half / stacks + 1 tiles, and
+// stacks < half.  One direction of 21 rows x 10240 cells
 // (8 items at the widest tile): transform 16.6 us, 10.7 us at 128 cells, with the
 // window pre-pass 24.2 and 20.7 us (256 cells: 20.0, 96 cells: 23.5).
 static int32_t filling_tile(int32_t widest, int32_t n_f0, int64_t stacks, int32_t n_sm)
@@ -1027,7 +1029,14 @@ static int run_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *o
                               per_unit * (win_cap / per_dir_win)));
     if (pairs && group < n_dir) group = std::max(2, group & ~1);
     const size_t need = per_dir_win * (size_t)((group + per_unit - 1) / per_unit);
-    const int rc = window_table(p, need, s);
+    // (the library's own tile: a call of fewer directions, whose tiles filling_tile
+    // narrows, takes fewer than n_sm items; it finds room for them, as a capture after
+    // this call must)
+    const size_t narrowed =
+        tile_auto ? std::min(win_cap, sizeof(uint32_t) * (size_t)p->n_sm *
+                                          (size_t)std::max(1, p->n_fft))
+                  : 0;
+    const int rc = window_table(p, std::max(need, narrowed), s);
     if (rc) return rc;
     JobTable tbl{};
     tbl.n_jobs = 1;

@@ -152,3 +152,33 @@ def test_first_call_of_a_process_is_captured(ws):
     r = subprocess.run([sys.executable, "-c", FIRST_CALL % dict(root=root, ws=ws)],
                        capture_output=True, text=True, timeout=600)
     assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("eager, captured", [(8, 6), (2, 1), (3, 1)])
+def test_fewer_directions_are_captured_after_more(fh, oracle_mod, eager, captured):
+    """An eager call sizes the window table for every smaller one: fewer directions
+    make narrower and so more tiles (8 directions of 600 rows x 640 cells in 76 items,
+    6 in 114), and a capture cannot allocate."""
+    import torch
+    inp, pp = synth.random_case(92, n_fft=30, n_bins=64, n_fdot=600, n_dir=eager, p=0.3)
+    want = oracle_mod.search(inp, pp, want_maps=True)["maps"][:captured]
+    plan = fh.fh_create_plan(fh.make_desc(pp, 30, eager, inp.n_peaks))
+    try:
+        dev = [torch.from_numpy(x).cuda() for x in (inp.t, inp.offsets, inp.freq, inp.v, inp.sky)]
+        maps = torch.empty((captured, pp["n_fdot"], pp["n_f0"]), dtype=torch.int32, device="cuda")
+        s = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        fh.fh_correct_doppler(plan, *dev, stream=s)
+        fh.fh_transform(plan, 0, eager, stream=s)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            fh.fh_transform(plan, 0, captured, maps, stream=s)
+        for _ in range(2):
+            maps.fill_(-1)
+            g.replay()
+            torch.cuda.synchronize()
+            assert np.array_equal(maps.cpu().numpy(), want)
+    finally:
+        torch.cuda.synchronize()
+        fh.fh_destroy_plan(plan)
