@@ -1307,7 +1307,8 @@ int fh_autotune(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *tile_cells
                         widths.push_back((int32_t)(((d.n_f0 + tiles - 1) / tiles + 15) / 16 * 16));
                 }
             for (int32_t w : widths) {
-                if (w < 64 || w > wmax || w > d.n_f0) continue;
+                // (of the added widths none below 64 cells; the widest may be)
+                if ((w < 64 && w != wmax) || w > wmax || w > d.n_f0) continue;
                 if (transform_smem_bytes(w, d.k_over, p->mode, nw, guard) > (size_t)lim) continue;
                 bool dup = false;
                 for (const auto &c : cands) dup = dup || (c.tile == w && c.warps == nw && c.pairs == pr);

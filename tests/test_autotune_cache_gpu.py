@@ -84,3 +84,32 @@ def test_a_written_entry_is_taken_as_given(tmp_path, n_dir):
         got = _child(cache, n_dir)
         assert (got["tile"], got["warps"]) == (512, 20)
         assert got["oracle_equal"]
+
+
+NARROW = r'''
+import json, sys
+sys.path.insert(0, %(root)r)
+import numpy as np, torch
+from paper_1407_8333_gb300 import build, fh, synth
+build.build(); fh.load()
+inp, pp = synth.random_case(9, n_fft=3000, n_bins=6, k_over=10, n_fdot=320, n_dir=64, p=0.3,
+                            vmax=2e-6)
+dev = [torch.from_numpy(np.ascontiguousarray(x)).cuda()
+       for x in (inp.t, inp.offsets, inp.freq, inp.v, inp.sky)]
+plan = fh.fh_create_plan(fh.make_desc(pp, 3000, 64, inp.n_peaks))
+fh.fh_correct_doppler(plan, *dev)
+tile, warps = fh.fh_autotune(plan, 0, 64)
+fh.fh_destroy_plan(plan)
+print(tile, warps, pp["n_f0"])
+'''
+
+
+def test_narrow_plans_are_tuned(tmp_path):
+    """A band below 64 cells (64 directions x 3000 FFTs, so that pairs halve the time):
+    its one width is timed in every form."""
+    cache = str(tmp_path / "t.json")
+    r = subprocess.run([sys.executable, "-c", NARROW % {"root": ROOT}], capture_output=True,
+                       text=True, timeout=600, env=dict(os.environ, FH_AUTOTUNE_CACHE=cache))
+    assert r.returncode == 0, r.stderr[-2000:]
+    e = json.load(open(cache))["entries"][0]
+    assert e["dir_pairs"] == 1 and e["tile_cells"] == 60
