@@ -540,7 +540,9 @@ struct CoinArgs {
 // mean width and t = RN(a - window b), which has the sign of the exact difference:
 // t <= 0 means a / b <= window, and so its rounding; t above 2^-50 a means a quotient
 // more than two units above the window; the division decides in between, and for
-// widths and windows next to the ends of binary64's range.
+// widths and windows next to the ends of binary64's range.  (b and the window are at
+// least 2^-500 each, so their product lies far above the subnormals and a t that
+// rounds to zero means a quotient that rounds to the window.)
 __device__ __forceinline__ bool within(double x1, double x2, double w1, double w2, bool wrap,
                                        double window)
 {
@@ -551,7 +553,7 @@ __device__ __forceinline__ bool within(double x1, double x2, double w1, double w
     const int ea = __double2hiint(a) >> 20, eb = __double2hiint(b) >> 20,
               ew = __double2hiint(window) >> 20, et = __double2hiint(t) >> 20;
     // (signs would make these negative or 2048 and more)
-    if (ea < 2047 && eb > 60 && eb < 2000 && ew > 60 && ew < 2000) {
+    if (ea < 2047 && eb > 523 && eb < 2000 && ew > 523 && ew < 2000) {
         if (__double_as_longlong(t) <= 0) return true;
         if (et >= ea - 49) return false;
     }

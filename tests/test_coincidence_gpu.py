@@ -307,3 +307,15 @@ def test_scratch_shared_by_threads_and_streams(fh):
     for t in threads:
         t.join()
     assert not bad
+
+
+def test_windows_next_to_the_ends_of_binary64(fh, co):
+    """A smallest subnormal apart, with windows whose product with the width lies
+    within half of it: the quotient decides."""
+    a = synth.candidate_set(3, 1, 40, clusters=2, cluster_size=3)
+    a[:, 0] = 0.0
+    a[:, 4] = 2.0 ** -474
+    b = a.copy()
+    b[:, 0] = 2.0 ** -1074
+    for w in (0.5, 0.75, 1.0, 1.25):
+        check_coinc(fh, co, a, b, 0.0, 0.0, 0.0, (w * 2.0 ** -600, 1.0, 1.0, 1.0))
