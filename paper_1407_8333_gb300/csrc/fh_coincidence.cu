@@ -313,9 +313,11 @@ cell_scatter_kernel(CandSet a, CandSet b, const Head *hp, int32_t max_cells, con
             make_float4(to_float(x.lam), to_float(x.beta),
                         to_float(__dsub_rn((in_b ? b : a).freq(x), f0)),
                         to_float(__dsub_rn(x.fdot, d0)));
+        // (never below 1e-37: the rejects take a product with the widths, and `ordinary`
+        // leaves such narrow ones to binary64)
+        auto half = [](double width) { return fmaxf(0.5f * to_float(width), 1e-37f); };
         o.rec[2 * (size_t)t + 1] =
-            make_float4(0.5f * to_float(x.dlam), 0.5f * to_float(x.dbeta), 0.5f * to_float(x.df),
-                        0.5f * to_float(x.dfdot));
+            make_float4(half(x.dlam), half(x.dbeta), half(x.df), half(x.dfdot));
     }
 }
 
@@ -796,16 +798,19 @@ int grid_for(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n 
 
 unsigned pair_grid(int64_t n) { return (unsigned)((n + kPairCands - 1) / kPairCands); }
 
-// reach per parameter -> binary32 bounds (see Limits)
+// reach per parameter -> binary32 bounds (see Limits); a positive reach below 1e-30 is
+// rejected as if it were that, so that the bound is no subnormal
 Limits make_limits(const double *reach, double d_max)
 {
     Limits l{};
     l.exact = false;
     const double up = 1.0 + 2e-5, dn = 1.0 - 2e-5;
-    for (int q = 0; q < 4; ++q)
+    float hi[4];
+    for (int q = 0; q < 4; ++q) {
         if (!(reach[q] > 1e-6 && reach[q] < 1e9)) l.exact = true;
-    l.hi = make_float4((float)(reach[0] * up), (float)(reach[1] * up), (float)(reach[2] * up),
-                       (float)(reach[3] * up));
+        hi[q] = reach[q] > 0.0 ? (float)(std::max(reach[q], 1e-30) * up) : 0.0f;
+    }
+    l.hi = make_float4(hi[0], hi[1], hi[2], hi[3]);
     l.lo = make_float4((float)(reach[0] * dn), (float)(reach[1] * dn), (float)(reach[2] * dn),
                        (float)(reach[3] * dn));
     l.d2_hi = (float)(d_max * d_max * (1.0 + 4e-5));

@@ -319,3 +319,19 @@ def test_windows_next_to_the_ends_of_binary64(fh, co):
     b[:, 0] = 2.0 ** -1074
     for w in (0.5, 0.75, 1.0, 1.25):
         check_coinc(fh, co, a, b, 0.0, 0.0, 0.0, (w * 2.0 ** -600, 1.0, 1.0, 1.0))
+
+
+# a reach below binary32's range on a very wide width, and a very wide reach on a width
+# below it: a tenth of what is allowed apart, and ten times that
+@pytest.mark.parametrize("width, reach", [(1e30, 1e-50), (1e-50, 1e20)])
+def test_reaches_beyond_binary32(fh, co, width, reach):
+    a = synth.candidate_set(4, 1, 60, clusters=2, cluster_size=3)
+    a[:, 1] = 0.0
+    a[:, 5] = width
+    b = a.copy()
+    b[:30, 1] = 0.1 * width * reach
+    b[30:, 1] = 10.0 * width * reach
+    check_coinc(fh, co, a, b, 0.0, 0.0, 0.0, (1.0, reach, 1.0, 1.0))
+    c = np.concatenate([a, b])
+    c[:, [0, 2, 3]] = c[0, [0, 2, 3]]
+    check_cluster(fh, co, c, reach)
