@@ -144,9 +144,10 @@ __global__ void __launch_bounds__(kRefThreads) refine_kernel(const RefineArgs a)
             const int64_t s0r = a.S0[i] + j_off * a.D[i] + lo_cell * 4294967296LL;
             const int64_t last = (int64_t)(a.n_rows - 1) * dr;
             // the band's two ends in half cells from f0_min: the cells below and above
-            // the extreme shifts, (1 - K) - 1 and (2 K + 1) + 1, less 0.5 - 0.5 K
-            const int32_t x_lo = (int32_t)((s0r + (last < 0 ? last : 0)) >> 32);
-            const int32_t x_hi = (int32_t)((s0r + (last > 0 ? last : 0)) >> 32) + 1;
+            // the extreme shifts, (1 - K) - 1 and (2 K + 1) + 1, less 0.5 - 0.5 K (in 64
+            // bits: a row far outside the plan's shifts by up to 2^31 cells)
+            const int64_t x_lo = (s0r + (last < 0 ? last : 0)) >> 32;
+            const int64_t x_hi = ((s0r + (last > 0 ? last : 0)) >> 32) + 1;
             const double u_lo = __fma_rn((double)(2 * x_lo - K - 1), a.half_inv_kt, a.f0_min);
             const double u_hi = __fma_rn((double)(2 * x_hi + 5 * K + 3), a.half_inv_kt, a.f0_min);
             const float vx = (float)a.v[3 * (int64_t)i], vy = (float)a.v[3 * (int64_t)i + 1],

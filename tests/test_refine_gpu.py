@@ -172,3 +172,36 @@ def test_groups_and_shares(fh, oracle_mod, k_over, k_fdot, n_fft, n_cand, n_ref)
     g = gpu_refine(fh, inp, pp, cells, rows, sky, k_fdot)
     o = oracle_mod.refine(inp, pp, cells, rows, sky, k_fdot)
     check(g, o, n_cand)
+
+
+def _far_case(f_cells):
+    n_fft, kt, f0 = 40, 16.0, 100.0
+    f = f0 + (2.0 ** 30 + f_cells) / kt
+    t = np.arange(n_fft) * 1.0 + 1e5
+    inp = synth.Inputs(w=None, t=t, offsets=np.arange(n_fft + 1, dtype=np.int64) * len(f),
+                       freq=np.tile(f, n_fft), v=np.zeros((n_fft, 3)), sky=np.array([[0., 0., 1.]]))
+    pp = dict(t_fft=1.0, k_over=16, f0_min=f0, n_f0=2000, fdot_min=0.0, fdot_step=5e-6, n_fdot=9,
+              t_ref=0.0, subband_cells=100, top_k=1, excl_cells=0, sep_cells=0, n_thr=0, p0=0.1)
+    return inp, pp
+
+
+def test_rows_far_outside_the_plan(fh):
+    """A candidate row whose shift (8 cells a row) lies 2^30 cells from the plan's band:
+    peaks there are beyond the fixed-point range and reported, by the device checks
+    (1) as by the host's, which look at every peak."""
+    sky = np.array([[[0.0, 0.0, 1.0]]])
+    for cells, refused in ((np.arange(-4000.0, 40000.0), True), (np.arange(1e6, 1e6 + 50), False)):
+        inp, pp = _far_case(cells)
+        plan = fh.fh_create_plan(fh.make_desc(pp, inp.t.shape[0], 1, inp.n_peaks))
+        try:
+            for checks in (0, 1):
+                fh.fh_plan_set_input_checks(plan, checks)
+                args = (plan, inp.t, inp.offsets, inp.freq, inp.v, [1000], [2 ** 27 - 2], sky, 1)
+                if refused or checks == 0:
+                    with pytest.raises(fh.FHError) as ei:
+                        fh.fh_refine(*args)
+                    assert ei.value.code == fh.FH_ERR_RANGE
+                else:
+                    assert fh.fh_refine(*args)["count"][0] == 0
+        finally:
+            fh.fh_destroy_plan(plan)
