@@ -521,8 +521,8 @@ struct GrossGrid {
     }
 };
 
-// Set-up of the gross veto: the CSR check, the cleared histogram and the column
-// edges: edge[y], y = 0 .. n_fh, the first bin whose frequency cell is y or more
+// Set-up of the gross veto: the CSR check, the cleared histogram and (edge not null)
+// the column edges: edge[y], y = 0 .. n_fh, the first bin whose frequency cell is y or more
 // (2^31 where no bin's is).  The bin that the grid names first, two to each side,
 // brackets nearly every edge; else the whole range of bins is searched.
 __global__ void __launch_bounds__(256)
@@ -534,7 +534,7 @@ gross_setup_kernel(const int64_t *o, int32_t n_fft, int64_t n_peaks, GrossGrid g
     const int64_t step = (int64_t)gridDim.x * blockDim.x;
     check_csr(o, n_fft, n_peaks, first, step, err);
     for (int64_t k = first; k < cells; k += step) hist[k] = 0;
-    for (int64_t y = first; y <= g.n_fh; y += step) {
+    for (int64_t y = first; edge && y <= g.n_fh; y += step) {
         const int64_t kmin = INT_MIN, kmax = (int64_t)INT_MAX + 1;
         int64_t lo = kmin, hi = kmax;  // column(lo - 1) < y <= column(hi)
         const double guess = (g.f0_h + (double)y * g.df_h) * g.fq.t_fft - (double)g.fq.k0;
@@ -553,6 +553,13 @@ gross_setup_kernel(const int64_t *o, int32_t n_fft, int64_t n_peaks, GrossGrid g
     }
 }
 
+// Column edges from this many peaks per column on: an edge costs a few columns in
+// binary64 and 8 bytes, and saves each peak its own.  The veto call on 1.96 million
+// peaks: 10^4 columns 126 us with edges, 141 without; 5 x 10^4 143 and 142; 10^5 158 and
+// 148; 10^6 212 and 153 (20 peaks, 10^6 columns: 162 and 61).  On 2 x 10^5 peaks no
+// difference up to 10^4 columns.
+constexpr int kPeaksPerEdge = 64;
+
 // a block per FFT: 620 peaks in 5 steps of 128 (a warp per FFT left two thirds of
 // the SMs' warps empty and every FFT a chain of 20 steps)
 constexpr int kFftThreads = 128;
@@ -560,7 +567,9 @@ constexpr int kFftThreads = 128;
 // The gross cell of every peak (kept for the veto pass) and the histogram: one
 // atomic per run of peaks in one cell of a warp (an FFT's peaks come in bin
 // order).  1.96 million peaks: 75 -> 17 us against a warp per FFT with each
-// column from binary64 and warp-wide matches.
+// column from binary64 and warp-wide matches.  EDGES: columns by the edges of
+// gross_setup_kernel, else each peak's own in binary64 (kPeaksPerEdge).
+template <bool EDGES>
 __global__ void __launch_bounds__(kFftThreads)
 gross_hist_kernel(const int64_t *o, const int32_t *bins, int64_t n_peaks, GrossGrid g,
                   const int64_t *edge, int32_t *cell, int32_t *hist)
@@ -574,14 +583,17 @@ gross_hist_kernel(const int64_t *o, const int32_t *bins, int64_t n_peaks, GrossG
     const int64_t it = it_s;
     int64_t lo, hi;
     peak_range(o, i, n_peaks, lo, hi);
-    const int64_t e0 = edge[0], e1 = edge[g.n_fh];
-    const float per_bin = (float)g.n_fh / fmaxf(1.0f, (float)(e1 - e0));
+    const int64_t e0 = EDGES ? edge[0] : 0, e1 = EDGES ? edge[g.n_fh] : 0;
+    const float per_bin = EDGES ? (float)g.n_fh / fmaxf(1.0f, (float)(e1 - e0)) : 0.0f;
     for (int64_t q0 = lo + (threadIdx.x & ~31); q0 < hi; q0 += kFftThreads) {
         const int64_t q = q0 + lane;
         int32_t c = -1;
         if (q < hi && it >= 0) {
             const int32_t b = __ldg(bins + q);
-            if (b >= e0 && b < e1) {
+            if constexpr (!EDGES) {
+                const double y = g.column(b);
+                if (y >= 0.0 && y < (double)g.n_fh) c = (int32_t)(it * g.n_fh + (int64_t)y);
+            } else if (b >= e0 && b < e1) {
                 int32_t y = min((int32_t)((float)(b - e0) * per_bin), g.n_fh - 1);
                 // the edges are evenly spaced to a bin, so the estimate is off by one at
                 // most; a grid that is not takes the search
@@ -1018,22 +1030,23 @@ int fh_peakmap_gross_veto(const double *t, const int64_t *offsets, const int32_t
     Result *res = nullptr;
     int32_t *cell = nullptr;
     int64_t *edge = nullptr;
+    const bool edges = n_fh < n_peaks / kPeaksPerEdge;
     cudaError_t e = sc.get(&res, 1);
     if (e == cudaSuccess) e = sc.get(&cell, (size_t)n_peaks);
-    if (e == cudaSuccess) e = sc.get(&edge, (size_t)n_fh + 1);
+    if (e == cudaSuccess && edges) e = sc.get(&edge, (size_t)n_fh + 1);
     if (e == cudaSuccess) e = cudaMemsetAsync(res, 0, sizeof(Result), s);
     const GrossGrid g{t, make_freq_of(k0, t_fft), t0_h, dt_h, f0_h, df_h, 1.0 / df_h, n_th, n_fh};
     const int64_t cells = (int64_t)n_th * n_fh;
     if (e == cudaSuccess) {
-        const int64_t work = std::max({cells, (int64_t)n_fh + 1, (int64_t)n_fft + 1});
+        const int64_t work = std::max(cells, (int64_t)n_fft + 1);  // (cells: n_fh or more)
         const int grid = (int)std::min<int64_t>((work + 255) / 256, 4096);
         gross_setup_kernel<<<grid, 256, 0, s>>>(offsets, n_fft, n_peaks, g, edge, hist, cells,
                                                 &res->err);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && n_fft > 0) {
-        launch_after(gross_hist_kernel, n_fft, kFftThreads, 0, s, offsets, bins, n_peaks, g, edge,
-                     cell, hist);
+        launch_after(edges ? gross_hist_kernel<true> : gross_hist_kernel<false>, n_fft,
+                     kFftThreads, 0, s, offsets, bins, n_peaks, g, edge, cell, hist);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return cuda_error(e, "gross histogram");

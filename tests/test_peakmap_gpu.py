@@ -315,3 +315,40 @@ def test_persistency_in_and_out_of_shared_memory(fh, pm, n_fft, n_bins):
         go, gb, _, gh, st = fh.fh_peakmap_persistency_veto(dev(o), dev(b), n_bins, k, 0, 8192.0)
         assert np.array_equal(host(gh), wh) and st == (m1, m2, thr)
         assert np.array_equal(host(go), wo) and np.array_equal(host(gb), wb)
+
+
+# with and without column edges (64 peaks per column): both sides of the line, columns
+# off both ends of the peaks' range, and far more columns than peaks
+@pytest.mark.parametrize("f0_h, df_h, n_fh", [
+    (50.0, 0.01, 46), (50.0, 0.01, 47), (50.0, 0.01, 48), (50.1, 0.002, 60), (49.0, 1e-4, 20000),
+    (50.0, 1.0 / 8192, 2048), (50.0, 1e-7, 1 << 20)])
+def test_gross_columns_with_and_without_edges(fh, pm, f0_h, df_h, n_fh):
+    o, b = _csr([1000, 2000, 2, 6], 2048, 8)   # 3008 peaks: edges up to 46 columns
+    t = np.arange(len(o) - 1) * 4096.0
+    for thr in (0, 3):
+        args = (409600, 8192.0, 0.0, 9000.0, 2, f0_h, df_h, n_fh, thr)
+        wo, wb, wh = pm.gross_veto(t, o, b, *args)
+        go, gb, gf, gh = fh.fh_peakmap_gross_veto(dev(t), dev(o), dev(b), *args)
+        assert np.array_equal(host(gh), wh)
+        assert np.array_equal(host(go), wo) and np.array_equal(host(gb), wb)
+        assert np.array_equal(host(gf).view(np.uint64),
+                              pm.peak_frequencies(wb, 409600, 8192.0).view(np.uint64))
+
+
+def test_a_fine_grid_takes_no_scratch_of_its_size(fh, pm):
+    """2^27 columns for six peaks: the call keeps no gigabyte of column edges (what it
+    took and freed is still the pool's when it returns)."""
+    import torch
+    t, n_fh = np.arange(4) * 512.0, 1 << 27
+    o = np.array([0, 2, 2, 3, 6], dtype=np.int64)
+    b = np.array([3, 900, 17, 3, 4, 70000], dtype=np.int32)
+    d = dev(t), dev(o), dev(b)
+    fh.fh_peakmap_gross_veto(*d, 0, 1024.0, 0.0, 1e6, 1, 0.0, 1.0, 4, 0)
+    torch.empty(n_fh, dtype=torch.int32, device="cuda")   # (in torch's cache for the histogram)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    go, gb, _, gh = fh.fh_peakmap_gross_veto(*d, 0, 1024.0, 0.0, 1e6, 1, 0.0, 3e-7, n_fh, 1)
+    assert before - torch.cuda.mem_get_info()[0] < 300 << 20
+    wo, wb, wh = pm.gross_veto(t, o, b, 0, 1024.0, 0.0, 1e6, 1, 0.0, 3e-7, n_fh, 1)
+    assert np.array_equal(host(go), wo) and np.array_equal(host(gb), wb)
+    assert np.array_equal(host(gh), wh)
