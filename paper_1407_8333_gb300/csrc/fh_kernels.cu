@@ -2061,15 +2061,17 @@ cudaError_t launch_correct(const PrepArgs &a, const double *freq, double f0_min,
     const double cshift = 0.5 - 0.5 * (double)k_over;
     const PosGrid G = make_pos_grid(f0_min, a.kt, k_over);
     // Four directions per block while that leaves every SM blocks; 8 FFTs, or 2 where
-    // even that leaves few, so that a block's chain of loads is short (one direction
-    // of 3164 FFTs: 19.5 -> 15.3 us, of 200: 8.9 -> 6.2; but 3 x 5003 FFTs of 83 peaks,
-    // 1881 blocks of 8: 14.5 us, 21.5 with 2).
+    // blocks of 8 are few or their FFTs long (a block takes 256 peaks at a time, one after
+    // another): a line through the measured crossings, 200 blocks of 8 for FFTs of up to
+    // 32 peaks, 300 - 400 for 64 - 150, above 3000 for 600.  One direction, us with 2 | 8
+    // FFTs: 200 FFTs x 64 peaks 6.2 | 8.0, 3200 x 8 12.4 | 8.5, 3200 x 150 12.4 | 10.6,
+    // 3200 x 600 20.6 | 23.8; two directions: 1600 x 32 9.8 | 7.9, 1600 x 600 18.5 | 20.7.
     const int32_t n_dir = std::max(1, a.n_dir), n = std::max(0, a.n_fft);
-    const int64_t g8 = (n + 7) / 8;
+    const int64_t g8 = (n + 7) / 8, per_fft = a.n_peaks / std::max(1, n);
     if (n_dir >= 4 && g8 * ((n_dir + 3) / 4) >= 1024) {
         dim3 grid(1 + g8, (n_dir + 3) / 4);
         correct_kernel<4, 8><<<grid, kPosThreads, 0, s>>>(a, freq, f0_min, cshift, G, A, out_r);
-    } else if (g8 * n_dir >= 600) {
+    } else if (g8 * n_dir >= 100 + 2 * per_fft) {
         dim3 grid(1 + g8, n_dir);
         correct_kernel<1, 8><<<grid, kPosThreads, 0, s>>>(a, freq, f0_min, cshift, G, A, out_r);
     } else {
