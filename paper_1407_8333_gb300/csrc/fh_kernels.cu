@@ -1932,29 +1932,31 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const SelectArgs a)
 // A_q - A_p < K 2^32), so c_i <= the most positions of FFT i inside a
 // half-open window of K cells: for every peak p the positions from it up to the
 // first one K cells or more away (ascending positions: two neighbours looked at,
-// then a binary search).  One warp per (direction, FFT), lanes on consecutive
-// peaks, so the loads are coalesced; one thread per FFT walking two pointers
-// took 218 us on the 50 Hz workload (3164 FFTs of 370 peaks), this 11 us.
+// then a binary search).  L lanes per (direction, FFT), on consecutive peaks, so that
+// the loads are coalesced: a warp from 32 peaks per FFT on, else 8 lanes.  (One thread
+// per FFT walking two pointers took 218 us on the 50 Hz workload, 3164 FFTs of 370
+// peaks; a warp takes 11 us.  17000 FFTs of 4 peaks in 16 directions, the whole call: 366
+// us with a thread per FFT, 385 with a warp, 351 with 8 lanes.)
 // bound[d] receives sum_i W_{d,i} c_{d,i} (each product capped at 2^40, which
 // already exceeds any admissible bound).  Every index stays inside the FFT's CSR
 // range (a valid CSR) and the search ends for any values; unsorted positions give
 // some bound, and such inputs are reported by the device checks.
 constexpr int kBoundThreads = 256;
+template <int L>
 __global__ void __launch_bounds__(kBoundThreads)
 weight_bound_kernel(const int64_t *__restrict__ A, const int64_t *__restrict__ offsets,
                     const int32_t *__restrict__ W, int32_t n_fft, int64_t n_peaks,
                     int32_t k_over, unsigned long long *__restrict__ bound)
 {
-    const int d = blockIdx.y, lane = threadIdx.x & 31;
-    const int i = blockIdx.x * (kBoundThreads / 32) + (threadIdx.x >> 5);
+    const int d = blockIdx.y, lane = threadIdx.x & 31, sub = threadIdx.x % L;
+    const int i = blockIdx.x * (kBoundThreads / L) + (int)threadIdx.x / L;
     __shared__ unsigned long long sum[kBoundThreads / 32];
-    unsigned long long v = 0;
+    int64_t c = 0;
     if (i < n_fft) {
         const int64_t *Ad = A + (int64_t)d * n_peaks;
         const int64_t o0 = offsets[i], o1 = offsets[i + 1];
         const unsigned long long width = (unsigned long long)k_over << 32;
-        int64_t c = 0;
-        for (int64_t p = o0 + lane; p < o1; p += 32) {
+        for (int64_t p = o0 + sub; p < o1; p += L) {
             // (unsigned difference: a wrap from unsorted input ends the window)
             const int64_t ap = Ad[p];
             auto in = [&](int64_t q) { return (unsigned long long)(Ad[q] - ap) < width; };
@@ -1972,15 +1974,19 @@ weight_bound_kernel(const int64_t *__restrict__ A, const int64_t *__restrict__ o
             }
             c = q - p > c ? q - p : c;
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            const int64_t y = __shfl_xor_sync(kFull, c, o);
-            c = y > c ? y : c;
-        }
+    }
+    for (int o = L / 2; o > 0; o >>= 1) {
+        const int64_t y = __shfl_xor_sync(kFull, c, o);
+        c = y > c ? y : c;
+    }
+    unsigned long long v = 0;
+    if (i < n_fft && sub == 0) {
         const unsigned long long w = (unsigned long long)(uint32_t)W[(int64_t)d * n_fft + i];
         const unsigned long long cap = 1ull << 40;
         v = (c >= (int64_t)(cap >> 1) || w * (unsigned long long)c > cap) ? cap
                                                                           : w * (unsigned long long)c;
     }
+    for (int o = 16; o >= L; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
     if (lane == 0) sum[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -2267,10 +2273,16 @@ cudaError_t launch_weight_bound(const int64_t *A, const int64_t *offsets, const 
                                 unsigned long long *bound, cudaStream_t s)
 {
     if (n_fft <= 0 || n_dir <= 0) return cudaSuccess;
-    constexpr int per = kBoundThreads / 32;
-    dim3 grid((n_fft + per - 1) / per, n_dir);
-    weight_bound_kernel<<<grid, kBoundThreads, 0, s>>>(A, offsets, W, n_fft, n_peaks, k_over,
-                                                       bound);
+    auto go = [&](auto lanes) {
+        constexpr int L = decltype(lanes)::value, per = kBoundThreads / L;
+        dim3 grid((n_fft + per - 1) / per, n_dir);
+        weight_bound_kernel<L><<<grid, kBoundThreads, 0, s>>>(A, offsets, W, n_fft, n_peaks,
+                                                              k_over, bound);
+    };
+    if (n_peaks < 32 * (int64_t)n_fft)
+        go(std::integral_constant<int, 8>{});
+    else
+        go(std::integral_constant<int, 32>{});
     return cudaGetLastError();
 }
 

@@ -210,3 +210,48 @@ def test_dense_off_grid_peaks_large_weights_refused_on_both_sides(fh, oracle_mod
         assert np.array_equal(m.cpu().numpy(), o["maps"])
     finally:
         fh.fh_destroy_plan(plan)
+
+
+# 8 lanes per FFT below 32 peaks per FFT on average, a warp from there on; FFT counts at
+# the edges of a block (32 and 8 FFTs), FFTs of none, one and more peaks than the lanes
+@pytest.mark.parametrize("n_fft", [1, 8, 9, 32, 33, 65])
+@pytest.mark.parametrize("per", [3, 31, 32, 70])
+def test_count_bound_lanes(fh, oracle_mod, n_fft, per):
+    """The count bound is exact: of a direction in which one FFT alone has a weight
+    (or all have the same one), the largest weight whose bound stays below 2^31 is
+    taken and the next one refused."""
+    import torch
+    rng = np.random.RandomState(97 * n_fft + per)
+    counts = rng.randint(0, 2, n_fft) * per
+    counts[-1] = per * n_fft - counts[:-1].sum()     # (the mean is per)
+    # 0.5, 2.5 or 7 cells between neighbours, K = 10
+    freq = np.concatenate([50.0 + (100.0 + (0.5, 2.5, 7.0)[i % 3] * np.arange(c)) / 10240.0
+                           for i, c in enumerate(counts)])
+    offsets = np.zeros(n_fft + 1, dtype=np.int64)
+    np.cumsum(counts, out=offsets[1:])
+    v, sky = np.zeros((n_fft, 3)), np.array([[0.0, 0.0, 1.0], [1.0, 0.0, 0.0]])
+    pp = dict(t_fft=1024.0, k_over=10, f0_min=50.0, n_f0=400, fdot_min=0.0, fdot_step=1e-13,
+              n_fdot=3, t_ref=0.0, subband_cells=100, top_k=1, excl_cells=0, sep_cells=0, n_thr=0,
+              p0=0.1)
+    r = oracle_mod.doppler_factor(v, sky)
+    A = oracle_mod.positions(offsets, freq, r, pp["f0_min"], 10240.0, 10)
+    c = oracle_mod.stripe_overlap(offsets, A[0], 10)
+    plan = fh.fh_create_plan(fh.make_desc(pp, n_fft, 2, len(freq)))
+    try:
+        fh.fh_correct_doppler(plan, *[torch.from_numpy(x).cuda() for x in
+                                      (np.arange(n_fft) * 512.0, offsets, freq, v, sky)])
+        for on in [np.arange(n_fft) == i for i in np.nonzero(c >= 3)[0][[0, -1]]] + [c > 0]:
+            total = int(c[on].sum())
+            most = (2 ** 31 - 1) // total
+            if total <= 2 * on.sum():                # (the sum of weights refuses first)
+                continue
+            for d in (0, 1):
+                w = np.zeros((2, n_fft))
+                w[d, on] = most
+                fh.fh_set_weights(plan, w, 0)
+                w[d, on] = most + 1
+                with pytest.raises(fh.FHError) as ei:
+                    fh.fh_set_weights(plan, w, 0)
+                assert ei.value.code == fh.FH_ERR_RANGE and "2^31" in str(ei.value)
+    finally:
+        fh.fh_destroy_plan(plan)
