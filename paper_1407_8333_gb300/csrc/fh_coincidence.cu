@@ -19,7 +19,7 @@
 // sorted order carries a 32-byte binary32 record per candidate (four parameters,
 // four half widths): what the pair loop reads, coalesced or broadcast, with the
 // binary64 records read only by the few pairs that the binary32 arithmetic
-// cannot decide.
+// cannot decide (sets whose records do not fit in memory form them at each use).
 //
 // Clustering links each candidate to those behind it in the sorted order through
 // a lock-free union-find: a root is only ever hung below a smaller root (one
@@ -282,8 +282,23 @@ cell_count_kernel(CandSet a, CandSet b, const Head *hp, int32_t max_cells, int32
     }
 }
 
-// sorted candidates: [position] -> index and cell, and the binary32 record, a sector
-// of 32 bytes: (lam, beta, f, fdot) and their half widths
+// a candidate's binary32 record: (lam, beta, f, fdot), f and fdot from the grid's
+// origin, and the half widths (never below 1e-37: the rejects take a product with the
+// widths, and `ordinary` leaves such narrow ones to binary64)
+__device__ __forceinline__ float4 record_x(const CandSet &s, const fh_cand_params &x, double f0,
+                                           double d0)
+{
+    return make_float4(to_float(x.lam), to_float(x.beta), to_float(__dsub_rn(s.freq(x), f0)),
+                       to_float(__dsub_rn(x.fdot, d0)));
+}
+__device__ __forceinline__ float4 record_h(const fh_cand_params &x)
+{
+    auto half = [](double width) { return fmaxf(0.5f * to_float(width), 1e-37f); };
+    return make_float4(half(x.dlam), half(x.dbeta), half(x.df), half(x.dfdot));
+}
+
+// sorted candidates (set a's, then set b's): [position] -> index and cell, and the
+// record, a sector of 32 bytes
 struct Sorted {
     int2 *who;
     float4 *rec;
@@ -291,6 +306,29 @@ struct Sorted {
     __device__ __forceinline__ int32_t cell(unsigned t) const { return who[t].y; }
     __device__ __forceinline__ float4 x(unsigned t) const { return rec[2 * (size_t)t]; }
     __device__ __forceinline__ float4 h(unsigned t) const { return rec[2 * (size_t)t + 1]; }
+};
+// the same without the records, formed anew at each use: for sets whose 32 bytes per
+// candidate do not fit in memory
+struct SortedLean {
+    int2 *who;
+    CandSet a, b;
+    const int32_t *n_a;  // candidates of set a among the sorted ones
+    const Head *head;
+    __device__ __forceinline__ int32_t index(unsigned t) const { return who[t].x; }
+    __device__ __forceinline__ int32_t cell(unsigned t) const { return who[t].y; }
+    __device__ __forceinline__ const CandSet &set(unsigned t) const
+    {
+        return t < (unsigned)*n_a ? a : b;
+    }
+    __device__ __forceinline__ float4 x(unsigned t) const
+    {
+        const CandSet &s = set(t);
+        return record_x(s, s.c[who[t].x], head->f0, head->d0);
+    }
+    __device__ __forceinline__ float4 h(unsigned t) const
+    {
+        return record_h(set(t).c[who[t].x]);
+    }
 };
 
 __global__ void __launch_bounds__(256)
@@ -309,15 +347,9 @@ cell_scatter_kernel(CandSet a, CandSet b, const Head *hp, int32_t max_cells, con
         const fh_cand_params x = in_b ? b.c[i] : a.c[i];
         const unsigned t = (unsigned)start[(in_b ? max_cells : 0) + w.x] + (unsigned)w.y;
         o.who[t] = make_int2(i, w.x);
-        o.rec[2 * (size_t)t] =
-            make_float4(to_float(x.lam), to_float(x.beta),
-                        to_float(__dsub_rn((in_b ? b : a).freq(x), f0)),
-                        to_float(__dsub_rn(x.fdot, d0)));
-        // (never below 1e-37: the rejects take a product with the widths, and `ordinary`
-        // leaves such narrow ones to binary64)
-        auto half = [](double width) { return fmaxf(0.5f * to_float(width), 1e-37f); };
-        o.rec[2 * (size_t)t + 1] =
-            make_float4(half(x.dlam), half(x.dbeta), half(x.df), half(x.dfdot));
+        if (!o.rec) continue;
+        o.rec[2 * (size_t)t] = record_x(in_b ? b : a, x, f0, d0);
+        o.rec[2 * (size_t)t + 1] = record_h(x);
     }
 }
 
@@ -407,8 +439,8 @@ __device__ __forceinline__ void uf_union(int32_t *parent, int32_t a, int32_t b, 
 constexpr int kScanLanes = 4;
 constexpr int kPairThreads = 256;
 constexpr int kPairCands = kPairThreads / kScanLanes;  // candidates of a block
-template <typename R, typename D>
-__device__ __forceinline__ void scan_pairs(const Sorted &o, unsigned n, int ranges,
+template <typename S, typename R, typename D>
+__device__ __forceinline__ void scan_pairs(const S &o, unsigned n, int ranges,
                                            const float4 &hi_lim, const float4 &tol, R &&range, D &&decide)
 {
     __shared__ uint2 list_s[kPairThreads / 32][96];
@@ -467,9 +499,10 @@ __device__ __forceinline__ void scan_pairs(const Sorted &o, unsigned n, int rang
 // 10^5 candidates of one 1 Hz band: 4.0 ms with buckets of frequency alone and the
 // binary64 records gathered per pair, 56 us now; 10^6 over 10 Hz: 25.4 -> 0.37 ms (0.41
 // with the 64 registers that leave four blocks on an SM).
+template <typename S>
 __global__ void __launch_bounds__(kPairThreads, 5)
 link_kernel(const fh_cand_params *c, int32_t max_cells, double d_max, Limits lim, const Head *hp,
-            const int32_t *start, Sorted o, int32_t *parent, int32_t *err)
+            const int32_t *start, S o, int32_t *parent, int32_t *err)
 {
     let_next_start();
     wait_for_previous();
@@ -526,6 +559,7 @@ __global__ void __launch_bounds__(256) finish_labels_kernel(int32_t *label, int3
 
 // ---------------------------------------------------------------- coincidences
 constexpr int kKeep = 8;  // partners of a candidate kept from the count for the write
+template <typename S>
 struct CoinArgs {
     CandSet s1, s2;
     double w[4];          // windows: lam, beta, f, fdot
@@ -533,7 +567,7 @@ struct CoinArgs {
     const Head *h;
     const int32_t *start; // set 1's cells, then set 2's (max_cells each)
     int32_t max_cells;
-    Sorted o;             // set 1's candidates, then set 2's
+    S o;                  // set 1's candidates, then set 2's
     int32_t *keep;        // [set-1 sorted position][kKeep], 16-byte aligned; null: the
                           // write looks for every candidate's partners again
 };
@@ -565,7 +599,9 @@ __device__ __forceinline__ bool within(double x1, double x2, double w1, double w
 // whether the records at sorted positions t (set 1) and u coincide, after the rejects:
 // each parameter clearly inside its window in binary32, else the exact test of that
 // one (values on the grid of a search are often whole windows apart)
-__device__ __forceinline__ bool inside(const CoinArgs &a, unsigned t, unsigned u, const float4 &tol)
+template <typename S>
+__device__ __forceinline__ bool inside(const CoinArgs<S> &a, unsigned t, unsigned u,
+                                       const float4 &tol)
 {
     const float4 d = apart(a.o.x(t), a.o.x(u)), w = wid(a.o.h(t), a.o.h(u));
     const bool ok = !a.lim.exact && ordinary(d, w);
@@ -584,8 +620,9 @@ __device__ __forceinline__ bool inside(const CoinArgs &a, unsigned t, unsigned u
 // for the count and 1.45 ms -> 30 us for the write; 10^6 x 10^6 over 10 Hz: 9.7 -> 0.18 ms
 // and 11.4 ms -> 44 us.  (With the four divisions of every pair that binary32 left open,
 // binary64 operations set the count's time, 55 us and 0.37 ms.)  cnt1 starts at zero.
-__global__ void __launch_bounds__(kPairThreads) coin_count_kernel(const CoinArgs a, int32_t *cnt1,
-                                                                  int32_t *cnt2)
+template <typename S>
+__global__ void __launch_bounds__(kPairThreads) coin_count_kernel(const CoinArgs<S> a,
+                                                                  int32_t *cnt1, int32_t *cnt2)
 {
     let_next_start();
     wait_for_previous();
@@ -606,8 +643,8 @@ __global__ void __launch_bounds__(kPairThreads) coin_count_kernel(const CoinArgs
 }
 
 // the partners of set 1's candidate at sorted position t, one thread: f(index in set 2)
-template <typename F>
-__device__ __forceinline__ void for_partners(const CoinArgs &a, unsigned t, F &&f)
+template <typename S, typename F>
+__device__ __forceinline__ void for_partners(const CoinArgs<S> &a, unsigned t, F &&f)
 {
     const float4 tol = a.h->tol;
     for (int k = -1; k <= 1; ++k) {
@@ -620,8 +657,9 @@ __device__ __forceinline__ void for_partners(const CoinArgs &a, unsigned t, F &&
     }
 }
 
+template <typename S>
 __global__ void __launch_bounds__(256)
-coin_write_kernel(const CoinArgs a, const int32_t *cnt1, const int64_t *off, int64_t capacity,
+coin_write_kernel(const CoinArgs<S> a, const int32_t *cnt1, const int64_t *off, int64_t capacity,
                   int32_t *pairs)
 {
     let_next_start();
@@ -819,11 +857,16 @@ Limits make_limits(const double *reach, double d_max)
 }
 
 // the candidates of a and b in cells: head, start (2 max_cells + 1) and the
-// sorted arrays (set a's candidates first), on scratch memory
+// sorted arrays (set a's candidates first), on scratch memory.  52 bytes per candidate;
+// where the records' 32 do not fit, without them (o.rec null: lean()).
 struct Cells {
     Head *head = nullptr;
     int32_t *start = nullptr, max_cells = 0;
     Sorted o{};
+    SortedLean lean(const CandSet &a, const CandSet &b) const
+    {
+        return SortedLean{o.who, a, b, start + max_cells, head};
+    }
 };
 cudaError_t build_cells(const CandSet &a, const CandSet &b, double reach_f, double reach_d,
                         int32_t *label, Cells &g, Scratch &sc, cudaStream_t s)
@@ -844,13 +887,18 @@ cudaError_t build_cells(const CandSet &a, const CandSet &b, double reach_f, doub
     const size_t o_start = take(4 * (cells + 1)), o_at = take(8 * n), o_who = take(8 * n),
                  o_rec = take(32 * n);
     cudaError_t e = sc.get(&base, at);
+    const bool lean = e == cudaErrorMemoryAllocation;
+    if (lean) {
+        cudaGetLastError();
+        e = sc.get(&base, o_rec);
+    }
     if (e != cudaSuccess) return e;
     g.head = reinterpret_cast<Head *>(base + o_head);
     int32_t *cnt = reinterpret_cast<int32_t *>(base + o_cnt);
     g.start = reinterpret_cast<int32_t *>(base + o_start);
     int2 *where = reinterpret_cast<int2 *>(base + o_at);
     g.o.who = reinterpret_cast<int2 *>(base + o_who);
-    g.o.rec = reinterpret_cast<float4 *>(base + o_rec);
+    g.o.rec = lean ? nullptr : reinterpret_cast<float4 *>(base + o_rec);
     e = cudaMemsetAsync(base, 0, zeroed, s);
     if (e != cudaSuccess) return e;
     const int grid = grid_for((int64_t)n);
@@ -898,9 +946,15 @@ int fh_cluster(const fh_cand_params *cands, int32_t n, double d_max, int32_t *la
     cudaError_t e = build_cells(none, set, d_max, d_max, label, g, sc, s);
     if (e == cudaSuccess) {
         // (with no set a the starts of the second half are the set's own)
-        launch_after(link_kernel, pair_grid(n), kPairThreads, 0, s, cands, g.max_cells, d_max,
-                     make_limits(reach, d_max), g.head, g.start + g.max_cells, g.o, label,
-                     &g.head->err);
+        auto link = [&](auto o) {
+            launch_after(link_kernel<decltype(o)>, pair_grid(n), kPairThreads, 0, s, cands,
+                         g.max_cells, d_max, make_limits(reach, d_max), g.head,
+                         g.start + g.max_cells, o, label, &g.head->err);
+        };
+        if (g.o.rec)
+            link(g.o);
+        else
+            link(g.lean(none, set));
         launch_after(finish_labels_kernel, grid_for(n), 256, 0, s, label, n, g.head);
         e = cudaGetLastError();
     }
@@ -938,36 +992,46 @@ int fh_coincidences(const fh_cand_params *c1, int32_t n1, double t_ref1,
     }
     Scratch sc(s);
     // frequencies at the common time: f + fdot (t_c - t_ref)
-    CoinArgs a{};
-    a.s1 = CandSet{c1, t_c - t_ref1, n1, 1};
-    a.s2 = CandSet{c2, t_c - t_ref2, n2, 1};
-    for (int q = 0; q < 4; ++q) a.w[q] = win[q];
-    a.lim = make_limits(win, 0.0);
+    const CandSet s1{c1, t_c - t_ref1, n1, 1}, s2{c2, t_c - t_ref2, n2, 1};
     Cells g;
     int64_t *off = nullptr;
-    int32_t *cnt1 = n_match1;
-    e = build_cells(a.s1, a.s2, win[2], win[3], nullptr, g, sc, s);
-    if (e == cudaSuccess && !cnt1) e = sc.get(&cnt1, (size_t)n1);
+    int32_t *cnt1 = n_match1, *keep = nullptr;
+    if (!cnt1) e = sc.get(&cnt1, (size_t)n1);
     if (e == cudaSuccess) e = sc.get(&off, (size_t)n1 + 1);
+    if (e == cudaSuccess) e = build_cells(s1, s2, win[2], win[3], nullptr, g, sc, s);
     // (sets so large that these 32 bytes per candidate do not fit do without)
-    if (e == cudaSuccess && sc.get(&a.keep, (size_t)n1 * kKeep) != cudaSuccess) {
+    if (e == cudaSuccess && sc.get(&keep, (size_t)n1 * kKeep) != cudaSuccess) {
         cudaGetLastError();
-        a.keep = nullptr;
+        keep = nullptr;
     }
     // (candidates of set 1 outside the grid have no partner and no sorted position)
     if (e == cudaSuccess) e = cudaMemsetAsync(cnt1, 0, 4 * (size_t)n1, s);
     if (e != cudaSuccess) return cuda_error(e, "coincidences set-up");
-    a.h = g.head;
-    a.start = g.start;
-    a.max_cells = g.max_cells;
-    a.o = g.o;
-    launch_after(coin_count_kernel, pair_grid(n1), kPairThreads, 0, s, a, cnt1, n_match2);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = scan_exclusive(cnt1, n1, off, sc, s);
-    if (e == cudaSuccess && capacity > 0) {
-        launch_after(coin_write_kernel, grid_for(n1), 256, 0, s, a, cnt1, off, capacity, pairs);
+    auto run = [&](auto o) {
+        CoinArgs<decltype(o)> a{};
+        a.s1 = s1;
+        a.s2 = s2;
+        for (int q = 0; q < 4; ++q) a.w[q] = win[q];
+        a.lim = make_limits(win, 0.0);
+        a.keep = keep;
+        a.h = g.head;
+        a.start = g.start;
+        a.max_cells = g.max_cells;
+        a.o = o;
+        launch_after(coin_count_kernel<decltype(o)>, pair_grid(n1), kPairThreads, 0, s, a, cnt1,
+                     n_match2);
         e = cudaGetLastError();
-    }
+        if (e == cudaSuccess) e = scan_exclusive(cnt1, n1, off, sc, s);
+        if (e == cudaSuccess && capacity > 0) {
+            launch_after(coin_write_kernel<decltype(o)>, grid_for(n1), 256, 0, s, a, cnt1, off,
+                         capacity, pairs);
+            e = cudaGetLastError();
+        }
+    };
+    if (g.o.rec)
+        run(g.o);
+    else
+        run(g.lean(s1, s2));
     int64_t total = 0;
     int32_t h_err = 0;
     if (e == cudaSuccess)

@@ -335,3 +335,47 @@ def test_reaches_beyond_binary32(fh, co, width, reach):
     c = np.concatenate([a, b])
     c[:, [0, 2, 3]] = c[0, [0, 2, 3]]
     check_cluster(fh, co, c, reach)
+
+
+def test_sets_whose_records_do_not_fit_in_memory(fh):
+    """With the device's memory taken up to what the sets' cells need, clustering and
+    coincidences do without the 32-byte records (and the kept partners): labels and
+    pairs are those of the calls with room."""
+    import torch
+    n = 16_000_000                        # records 512 MB per set, all else below 400 MB
+    g = torch.Generator(device="cuda")
+    g.manual_seed(11)
+
+    def rand():
+        return torch.rand(n, dtype=torch.float64, device="cuda", generator=g)
+
+    a = torch.empty((n, 8), dtype=torch.float64, device="cuda")
+    a[:, 0] = 6.28 * rand()
+    a[:, 1] = 3.0 * rand() - 1.5
+    a[:, 2] = 50.0 + 200.0 * rand()
+    a[:, 3] = -1e-9 * rand()
+    a[:, 4:] = torch.tensor([2e-2, 2e-2, 2e-4, 2e-11], dtype=torch.float64, device="cuda")
+    b = a[torch.randperm(n, device="cuda", generator=g)].contiguous()
+    b[:, 0] += 0.5 * 2e-2
+    m = 4_000_000                         # set 1 of the coincidences
+    win = (2.0, 2.0, 2.0, 2.0)
+    lab, k = fh.fh_cluster(a, 3.0)
+    p, m1, m2 = fh.fh_coincidences(a[:m], b, 0.0, 0.0, 0.0, win, capacity=2 * m)
+    assert 0 < k < n and len(p) >= m // 4
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    outputs = torch.empty(1 << 29, dtype=torch.uint8, device="cuda")
+    fill, left = [], 500 << 20
+    while torch.cuda.mem_get_info()[0] > left + (2 << 20):
+        step = min(4 << 30, torch.cuda.mem_get_info()[0] - left)
+        fill.append(torch.empty(step, dtype=torch.uint8, device="cuda"))
+    assert torch.cuda.mem_get_info()[0] < 2 * left
+    del outputs                           # (into torch's cache, for the calls' outputs)
+    try:
+        lab2, k2 = fh.fh_cluster(a, 3.0)
+        p2, n1, n2 = fh.fh_coincidences(a[:m], b, 0.0, 0.0, 0.0, win, capacity=2 * m)
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    assert k2 == k and torch.equal(lab2, lab)
+    assert torch.equal(p2, p) and torch.equal(n1, m1) and torch.equal(n2, m2)
