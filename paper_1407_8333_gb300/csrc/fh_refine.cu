@@ -345,10 +345,17 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
     // caller's page-locked arrays are copied from until the call's synchronisation.
     {
         double m = 0.0;
-        for (int32_t i = 0; i < n; ++i) {
-            const double x = std::fabs(step_ref * ((pm->t_fft[i] - d.t_ref) * kt));
-            if (x > m && x < 1e9) m = x;  // non-finite times are left to the checks
-        }
+        auto drift = [&](int32_t i) {
+            return std::fabs(step_ref * ((pm->t_fft[i] - d.t_ref) * kt));
+        };
+        // (checked times ascend: the largest drift is at an end)
+        if (host_checks && n > 0 && drift(0) < 1e9 && drift(n - 1) < 1e9)
+            m = std::max(drift(0), drift(n - 1));
+        else
+            for (int32_t i = 0; i < n; ++i) {
+                const double x = drift(i);
+                if (x > m && x < 1e9) m = x;  // non-finite times are left to the checks
+            }
         const int32_t guard = guard_for((unsigned long long)(m * 4294967296.0) + 4);
         int dev = 0;
         cudaGetDevice(&dev);
