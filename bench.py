@@ -384,7 +384,7 @@ def measure_step(fh, torch, w, inp, pp, dev, steps, warmup, flush, world=1, cloc
                                     "binary64 adds and multiplies: %.0f Gop/s"
                                     % (fp64_ops, fp64_peak / 1e9),
                  "duration_ms": corr_ms,
-                 "duration_note": "CUDA events around fh_correct_doppler (one 32-byte memset "
+                 "duration_note": "CUDA events around fh_correct_doppler (one memset "
                                   "and the correction kernel)"}
     res = {"updates_per_step": upd_step, "ms_per_step": total_ms / steps,
            "value": upd_step * steps * world / (total_ms * 1e-3),

@@ -272,7 +272,10 @@ int fh_sync(fh_plan plan, void *stream);
  * shape (GPU model, counting mode, weighting, n_f0, n_fdot, K, T_FFT, N_t,
  * n_dir); when the environment variable FH_AUTOTUNE_CACHE names a file, they
  * are also read from and written to it (JSON, one entry per line), so later
- * processes reuse them without timing. */
+ * processes reuse them without timing.  An entry is taken as it is, whatever
+ * version of the library wrote it: remove the file to time the present kernels.
+ * Timed without a map; calls that write one run kernels of their own in the
+ * same shape. */
 int fh_autotune(fh_plan plan, int32_t dir_begin, int32_t n_dir, int32_t *tile_cells,
                 int32_t *block_warps, void *stream);
 

@@ -2242,7 +2242,11 @@ cudaError_t launch_windows(const TransformJob &job, uint32_t *windows, cudaStrea
     // tiles per lane and pass: enough for all tiles in one pass, at most kWinMaxM; where
     // there are too few blocks to fill the SMs, one tile per lane and the passes side by
     // side, each staging the peaks again (200 FFTs x 72 tiles: 7.1 -> 5.0 us; 3164 FFTs x
-    // 82 tiles x 19 slabs: 30.3 -> 28.4 us)
+    // 82 tiles x 19 slabs: 30.3 -> 28.4 us).  Between 200 and 1000 blocks the two forms lie
+    // within 10 % of a transform call of each other, either way with the shape (400
+    // FFTs x 10,000 cells, 50 blocks: 10.6 us side by side, 12.0 not; 1600 FFTs, 200 blocks:
+    // 14.3 and 14.9; 3200 FFTs x 20,000 cells, 400 blocks: 26.9 and 25.6; 8000 FFTs, 1000
+    // blocks: 32.9 and 29.0).
     const int passes = std::max(1, (job.n_tiles + 31) / 32);
     const bool few = (int64_t)grid.x * grid.y < 600;
     const int m = few ? 1 : std::min(kWinMaxM, passes);
