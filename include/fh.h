@@ -160,7 +160,8 @@ int fh_create_plan(const fh_plan_desc *desc, fh_plan *out);
 /* Synchronise the device and free the plan.  NULL is accepted. */
 int fh_destroy_plan(fh_plan plan);
 
-/* Bytes of device memory a plan with this desc allocates (0 if invalid). */
+/* Bytes of device memory fh_create_plan allocates for this desc (0 if invalid); the
+ * table of peak windows that fh_transform takes comes on top. */
 int64_t fh_plan_device_bytes(const fh_plan_desc *desc);
 
 /* Steps a1-a3 (Sec. VI, Eq. fdopp): Doppler factor of every (direction,

@@ -254,10 +254,10 @@ int validate_desc(const fh_plan_desc &d)
 namespace {
 
 struct Sizes {
-    int64_t t, offsets, tables, freq, v, sky, A, profile, cand;
+    int64_t t, offsets, tables, freq, v, sky, A, profile, cand, err;
     int64_t total() const
     {
-        return t + 2 * offsets + 2 * tables + freq + v + sky + A + profile + cand + 256;
+        return t + 2 * offsets + 2 * tables + freq + v + sky + A + profile + cand + err + 256;
     }
 };
 
@@ -274,6 +274,7 @@ Sizes plan_sizes(const fh_plan_desc &d)
     s.A = 8 * (int64_t)d.max_dir * d.max_peaks;
     s.profile = 8 * (int64_t)d.max_dir * d.n_f0;
     s.cand = (int64_t)sizeof(fh_candidate) * d.max_dir * n_sb * d.top_k;
+    s.err = err_block_bytes(d.max_dir);
     return s;
 }
 
@@ -536,7 +537,7 @@ int fh_create_plan(const fh_plan_desc *desc, fh_plan *out)
                   {(void **)&p->freq, s.freq},     {(void **)&p->v, s.v},
                   {(void **)&p->sky, s.sky},       {(void **)&p->A, s.A},
                   {(void **)&p->profile, s.profile}, {(void **)&p->cand, s.cand},
-                  {(void **)&p->err, err_block_bytes(desc->max_dir)},
+                  {(void **)&p->err, s.err},
                   {(void **)&p->sched, 16}};
     for (auto &a : allocs) {
         e = cudaMalloc(a.ptr, (size_t)std::max<int64_t>(a.bytes, 16));

@@ -86,6 +86,16 @@ def test_invalid_plan_is_rejected_without_gpu(lib):
         fh.fh_create_plan(fh.make_desc(pp, 10, 1, 100))
 
 
+def test_plan_bytes_count_every_buffer(lib):
+    """Per direction: its sky vector, positions, profile, candidates and pair distance."""
+    from paper_1407_8333_gb300 import fh, synth
+    _, pp = synth.random_case(1)
+    n_sb = -(-pp["n_f0"] // pp["subband_cells"])
+    per_dir = 24 + 8 * 100 + 8 * pp["n_f0"] + 48 * n_sb * pp["top_k"] + 4
+    size = [fh.fh_plan_device_bytes(fh.make_desc(pp, 10, n, 100)) for n in (1, 60001)]
+    assert size[1] - size[0] == 60000 * per_dir
+
+
 def test_selection_workspace_size(lib):
     """fh_peakmap_select_workspace covers a bit per bin and a count per
     4096-bin segment of every FFT, grows with both sizes, and refuses
