@@ -383,25 +383,33 @@ int refine_impl(const fh_plan_desc &d, int n_sm, const fh_peakmap *pm,
     // A block's histogram of starts in shared memory: all directions and rows where
     // they fit in 40 KB, else groups of directions, else of rows.  In memory, the
     // starts of as many candidates and directions at a time as 1 GiB holds (and as
-    // give a grid at most 65535 groups).
+    // give a grid at most 65535 groups), or as half of that, and so on, where memory is
+    // short.
     const int32_t E = 3 * K;
-    const int64_t per_dir = (int64_t)n_rows * E, most = (int64_t)1 << 28, room = 40 * 1024 / 4;
+    const int64_t per_dir = (int64_t)n_rows * E, room = 40 * 1024 / 4;
     RefineArgs ra{};
     ra.rows_per = (int32_t)std::max<int64_t>(1, std::min<int64_t>(n_rows, room / E));
     const int64_t row_groups = (n_rows + ra.rows_per - 1) / ra.rows_per;
-    const int32_t dir_batch = (int32_t)std::max<int64_t>(
-        1, std::min<int64_t>({n_ref, most / per_dir, 65535 / row_groups}));
-    ra.dirs_per = (int32_t)std::max<int64_t>(
-        1, std::min<int64_t>(dir_batch, room / ((int64_t)ra.rows_per * E + 3)));  // + its sky
-    const int32_t cand_batch = (int32_t)std::max<int64_t>(
-        1, std::min<int64_t>(n_cand, most / (per_dir * dir_batch)));
-    const size_t n_starts = (size_t)cand_batch * dir_batch * per_dir;
     // what is read back (the candidates, then the error word) and what starts at zero
     // beside it (largest |D|, stripe starts), in one block
     const size_t out_bytes = sizeof(fh_candidate) * (size_t)n_cand;
+    int32_t dir_batch = 1, cand_batch = 1;
+    size_t n_starts = 0;
     char *zero = nullptr;
     int32_t *best = nullptr;
-    if (e == cudaSuccess) e = sc.get(&zero, out_bytes + 64 + 4 * n_starts);
+    for (int64_t most = (int64_t)1 << 28; e == cudaSuccess; most /= 2) {
+        dir_batch = (int32_t)std::max<int64_t>(
+            1, std::min<int64_t>({n_ref, most / per_dir, 65535 / row_groups}));
+        cand_batch = (int32_t)std::max<int64_t>(
+            1, std::min<int64_t>(n_cand, most / (per_dir * dir_batch)));
+        n_starts = (size_t)cand_batch * dir_batch * per_dir;
+        e = sc.get(&zero, out_bytes + 64 + 4 * n_starts);
+        if (e != cudaErrorMemoryAllocation || (dir_batch == 1 && cand_batch == 1)) break;
+        cudaGetLastError();
+        e = cudaSuccess;
+    }
+    ra.dirs_per = (int32_t)std::max<int64_t>(
+        1, std::min<int64_t>(dir_batch, room / ((int64_t)ra.rows_per * E + 3)));  // + its sky
     if (e == cudaSuccess && dir_batch < n_ref) e = sc.get(&best, 3 * (size_t)n_cand);
     if (e != cudaSuccess) return cuda_error(e, "cudaMallocAsync (refinement)");
     fh_candidate *d_out = reinterpret_cast<fh_candidate *>(zero);

@@ -234,3 +234,29 @@ def test_a_refused_refinement_queues_nothing(fh):
     finally:
         torch.cuda.synchronize()
         fh.fh_destroy_plan(plan)
+
+
+def test_starts_that_do_not_fit_in_memory(fh):
+    """600 MB of stripe starts (108 candidates x 60 directions x 256 rows x 90 starts)
+    with less than 450 MB to be had: taken in turns, the result is that of one turn."""
+    import torch
+    inp, pp = synth.random_case(77, n_fft=40, n_bins=60, k_over=30, n_fdot=9, n_dir=1, p=0.3)
+    rng = np.random.RandomState(5)
+    cells, rows = rng.randint(0, pp["n_f0"], 108), rng.randint(0, 9, 108)
+    sky = random_sky_ref(6, 108, 60)
+    plan = fh.fh_create_plan(fh.make_desc(pp, 40, 1, inp.n_peaks))
+    args = (plan, inp.t, inp.offsets, inp.freq, inp.v, cells, rows, sky, 64)
+    fill, left = [], 150 << 20
+    try:
+        want = fh.fh_refine(*args)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        while torch.cuda.mem_get_info()[0] > left + (2 << 20):
+            fill.append(torch.empty(min(4 << 30, torch.cuda.mem_get_info()[0] - left),
+                                    dtype=torch.uint8, device="cuda"))
+        got = fh.fh_refine(*args)
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+        fh.fh_destroy_plan(plan)
+    assert want["count"].max() > 5 and np.array_equal(got, want)
