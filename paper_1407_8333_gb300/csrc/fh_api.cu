@@ -971,6 +971,7 @@ static int run_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *o
     const int32_t guard = plan_guard(p, kind);
     const int32_t wmax = default_tile(d, p->device, p->mode, nwarps, guard);
     if (tile > wmax) tile = wmax;
+    const int32_t widest = tile;
     if (tile_auto) {
         const int32_t rows = kind == kPairRows ? 2 * kRows : kRows;
         tile = filling_tile(tile, d.n_f0,
@@ -1038,6 +1039,9 @@ static int run_transform(fh_plan p, int32_t dir_begin, int32_t n_dir, int32_t *o
                                           (size_t)std::max(1, p->n_fft))
                   : 0;
     const int rc = window_table(p, std::max(need, narrowed), s);
+    if (rc == FH_ERR_NOMEM && tile_auto)  // the widest tile has the smallest table
+        return run_transform(p, dir_begin, n_dir, out_maps, widest, nwarps, schedule, s,
+                             pair_pref, item_counter);
     if (rc) return rc;
     JobTable tbl{};
     tbl.n_jobs = 1;

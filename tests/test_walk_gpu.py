@@ -242,3 +242,37 @@ def test_window_table_grows_between_transforms_in_flight(fh, n_dir, n_fdot):
         for t in threads:
             t.join()
     assert not bad
+
+
+def test_window_table_that_does_not_fit_in_memory(fh):
+    """A million FFTs of one peak: the narrowed tiles of one direction want a table of
+    300 MB and room for 600; with less to be had the widest tile serves."""
+    import torch
+    n_fft = 1_000_000
+    rng = np.random.RandomState(3)
+    t = np.arange(n_fft) * 512.0
+    freq = 50.0 + rng.uniform(0.1, 1.9, n_fft)
+    offsets = np.arange(n_fft + 1, dtype=np.int64)
+    pp = dict(t_fft=1024.0, k_over=10, f0_min=50.0, n_f0=20480, fdot_min=0.0,
+              fdot_step=1.0 / (1024.0 * t[-1]), n_fdot=8, t_ref=0.0, subband_cells=1024, top_k=2,
+              excl_cells=20, sep_cells=40, n_thr=0, p0=0.1)
+    dev = [torch.from_numpy(x).cuda() for x in
+           (t, offsets, freq, np.zeros((n_fft, 3)), np.array([[0.0, 0.0, 1.0]]))]
+
+    got = []
+    for left in (0, 200 << 20):               # 0: with all the room there is
+        fill = []
+        plan = fh.fh_create_plan(fh.make_desc(pp, n_fft, 1, n_fft))
+        try:
+            fh.fh_correct_doppler(plan, *dev)
+            torch.cuda.synchronize()
+            while left and torch.cuda.mem_get_info()[0] > left + (2 << 20):
+                fill.append(torch.empty(min(4 << 30, torch.cuda.mem_get_info()[0] - left),
+                                        dtype=torch.uint8, device="cuda"))
+            fh.fh_transform(plan, 0, 1)
+            got.append(fh.fh_select_candidates(plan, 0, 1))
+        finally:
+            del fill
+            torch.cuda.empty_cache()
+            fh.fh_destroy_plan(plan)
+    assert got[0]["count"].max() > 0 and np.array_equal(got[0], got[1])
