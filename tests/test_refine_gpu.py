@@ -207,30 +207,37 @@ def test_rows_far_outside_the_plan(fh):
             fh.fh_destroy_plan(plan)
 
 
-def test_a_refused_refinement_queues_nothing(fh):
-    """A refined drift too wide for shared memory is refused before any copy from the
-    caller's page-locked arrays is queued or any scratch for them is taken (256 MB),
-    behind work that keeps the stream busy."""
+def test_a_refused_refinement_leaves_nothing_queued(fh):
+    """A refined drift too wide for shared memory is refused with nothing left on the
+    stream that reads the caller's page-locked arrays (256 MB), behind work that keeps
+    the stream busy."""
     import torch
     n_fft, per = 64, 500_000
-    t, v = np.arange(n_fft) * 512.0, np.zeros((n_fft, 3))
-    offsets = np.arange(n_fft + 1, dtype=np.int64) * per
-    freq = torch.from_numpy(np.tile(50.0 + np.arange(per) * 1e-6, n_fft)).pin_memory().numpy()
+
+    def pinned(x):
+        return torch.from_numpy(np.ascontiguousarray(x)).pin_memory().numpy()
+
+    t, v = pinned(np.arange(n_fft) * 512.0), pinned(np.zeros((n_fft, 3)))
+    offsets = pinned(np.arange(n_fft + 1, dtype=np.int64) * per)
+    freq = pinned(np.tile(50.0 + np.arange(per) * 1e-6, n_fft))
+    cells, rows = pinned(np.array([1000], np.int32)), pinned(np.array([3], np.int32))
+    sky = pinned(np.array([[[0.0, 0.0, 1.0]]]))
     _, pp = synth.random_case(5)
+    plan = fh.fh_create_plan(fh.make_desc(pp, n_fft, 1, 1000))   # (kernels loaded)
+    fh.fh_refine(plan, t, offsets, freq, v, cells, rows, sky, 1)
+    fh.fh_destroy_plan(plan)
     pp["fdot_step"] = 100.0 / (pp["k_over"] * pp["t_fft"] * t[-1])   # 100 cells a row
     pp["t_ref"] = 0.0
     plan = fh.fh_create_plan(fh.make_desc(pp, n_fft, 1, 1000))
     try:
         st = torch.cuda.Stream()
         torch.cuda.synchronize()
-        before = torch.cuda.mem_get_info()[0]
         with torch.cuda.stream(st):
             torch.cuda._sleep(1_000_000_000)
         with pytest.raises(fh.FHError) as ei:
-            fh.fh_refine(plan, t, offsets, freq, v, [1000], [3], np.array([[[0.0, 0.0, 1.0]]]), 1,
-                         stream=st)
+            fh.fh_refine(plan, t, offsets, freq, v, cells, rows, sky, 1, stream=st)
         assert ei.value.code == fh.FH_ERR_CUDA
-        assert before - torch.cuda.mem_get_info()[0] < 64 << 20
+        assert st.query()
     finally:
         torch.cuda.synchronize()
         fh.fh_destroy_plan(plan)
